@@ -372,13 +372,13 @@ dab_contraction dab_get_contraction(void);
  *                      shared by the up to kh*kw patches that contain it.  Patches it cannot settle (a hull of more
  *                      than 1024 values, a constant row without zeros, magnitudes outside 2^-40..2^40, a NaN or an
  *                      infinity in the tile) are sorted in full by a second kernel;
- *   DAB_PATCHES_HIST   rows and patches of 257..8192 values, one warp each: a histogram of the row's own values
- *                      quantised to 24 bits of its range, the same bound per bucket with a margin for the
- *                      quantisation, exact search of what survives; rows it cannot settle fall to the sorting kernel;
+ *   DAB_PATCHES_HIST   patches of 257..8192 values, one warp each: a histogram of the patch's own values
+ *                      quantised to 24 bits of the tile's range, the same bound per bucket with a margin for the
+ *                      quantisation, exact search of what survives; what it cannot settle falls to the sorting kernel.
+ *                      Rows of a matrix of more than 256 values: a CTA per row, exact counts and sums per bucket;
  *   DAB_PATCHES_AUTO   (default) patches: DAB_PATCHES_PIXEL wherever a patch spans several pixels and the layer has
  *                      at least 1024 patches; otherwise per tile of the input the sorting kernels for tiles with few non-zero values
- *                      and DAB_PATCHES_HIST for the others.  Rows of a matrix: DAB_PATCHES_HIST from 2048 rows on,
- *                      DAB_PATCHES_SORT below.
+ *                      and DAB_PATCHES_HIST for the others.  Rows of a matrix: DAB_PATCHES_HIST.
  * Process-wide, read once at the start of each call.
  */
 typedef enum { DAB_PATCHES_AUTO = 0, DAB_PATCHES_SORT = 1, DAB_PATCHES_HIST = 2, DAB_PATCHES_PIXEL = 3 } dab_patch_coder;
