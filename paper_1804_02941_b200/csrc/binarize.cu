@@ -114,22 +114,12 @@ static cudaError_t launch_rows_group(const float* values, int64_t rows, int32_t 
 // ---------------------------------------------------------------------------------------------------------
 // Rows of a matrix through the bucket-pruned search of rowbucket.cuh, a CTA per row.
 // ---------------------------------------------------------------------------------------------------------
-struct MatrixRow {
-  const float* v;
-  int n;
-  bool aligned;  // 16-byte loads reach every value
-  __device__ __forceinline__ float operator()(int i) const { return __ldg(v + DAB_IDX(i, n)); }
-  __device__ __forceinline__ bool quads() const { return aligned; }
-  __device__ __forceinline__ float4 quad(int q) const { return __ldg(reinterpret_cast<const float4*>(v + DAB_IDX(4 * q, n - 3))); }
-};
-
 template <int T>
 __global__ void __launch_bounds__(T, 1024 / T) binarize_rows_bucket_kernel(const float* __restrict__ values, int32_t n, int64_t ld_values,
                                                                  const RowOut out) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   for (int64_t row = blockIdx.x; row < out.rows; row += gridDim.x) {
-    const float* v = values + row * ld_values;
-    block_code_row<T>(MatrixRow{v, n, (n & 3) == 0 && (reinterpret_cast<uintptr_t>(v) & 15) == 0}, n, smem_raw, out, row);
+    block_code_row<T>(MatrixRow(values + row * ld_values, n), n, smem_raw, out, row);
     __syncthreads();
   }
 }

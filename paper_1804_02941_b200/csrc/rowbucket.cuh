@@ -163,11 +163,44 @@ struct RowOut {
   int64_t rows;
 };
 
-// Codes row `row`.  value(i): element i of the row; value.quads(): whether value.quad(q) gives elements 4q .. 4q+3 (for the
-// whole row; the same for all threads).  smem: block_row_bytes<T>(n) bytes.  All threads of the CTA call it;
-// the shared memory is free again when it returns in all threads (a barrier is the caller's).
-template <int T, typename Value>
-__device__ __forceinline__ void block_code_row(Value value, int n, unsigned char* smem, const RowOut& out, int64_t row) {
+// A row of values in global memory, as block_code_row takes it.  stage<T>: the CTA copies the row to `vals`, padded with
+// zeros (which no pass counts) to `quads` quadruples, and each thread returns the largest magnitude bits it saw; restage<T>:
+// the same values once more; finish: called by every thread when the row's code is known, with the row still staged.
+struct MatrixRow {
+  const float* v;
+  int n;
+  bool aligned;  // 16-byte loads reach every value
+  __device__ __forceinline__ MatrixRow(const float* row, int n_) : v(row), n(n_), aligned((n_ & 3) == 0 && (reinterpret_cast<uintptr_t>(row) & 15) == 0) {}
+  template <int T>
+  __device__ __forceinline__ uint32_t stage(float* vals, int quads, BlockShared<T>*) const {
+    uint32_t top = 0u;
+    if (aligned) {
+#pragma unroll 4
+      for (int q = threadIdx.x; q < quads; q += T) {
+        const float4 x = 4 * q < n ? __ldg(reinterpret_cast<const float4*>(v + DAB_IDX(4 * q, n - 3))) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        *reinterpret_cast<float4*>(vals + 4 * q) = x;
+        top = max(max(top, max(magnitude_bits(x.x), magnitude_bits(x.y))), max(magnitude_bits(x.z), magnitude_bits(x.w)));
+      }
+    } else {
+#pragma unroll 8
+      for (int i = threadIdx.x; i < 4 * quads; i += T) {
+        const float x = i < n ? __ldg(v + DAB_IDX(i, n)) : 0.0f;
+        vals[i] = x;
+        top = max(top, magnitude_bits(x));
+      }
+    }
+    return top;
+  }
+  template <int T>
+  __device__ __forceinline__ void restage(float* vals, int quads) const { stage<T>(vals, quads, nullptr); }
+  template <int T>
+  __device__ __forceinline__ void finish(const float*, const RowResult&) const {}
+};
+
+// Codes row `row`.  smem: block_row_bytes<T>(n) bytes.  All threads of the CTA call it; the shared memory is free again
+// when it has returned in all threads (a barrier is the caller's).
+template <int T, typename Source>
+__device__ __forceinline__ void block_code_row(const Source& source, int n, unsigned char* smem, const RowOut& out, int64_t row) {
   constexpr int W = T / 32, PB = BucketShape<T>::PB, NB = PB * T / 2, SHIFT = 23 - BucketShape<T>::LOG2M;
   BlockShared<T>* const bs = reinterpret_cast<BlockShared<T>*>(smem);
   uint32_t* const hist = reinterpret_cast<uint32_t*>(bs + 1);  // [2 NB] counts, then [2 NB] low sums
@@ -178,26 +211,8 @@ __device__ __forceinline__ void block_code_row(Value value, int n, unsigned char
 #pragma unroll
   for (int j = 0; j < 2 * PB; ++j) hist[j * T + tid] = 0u;
   if (tid == 0) bs->fill = bs->overflow = 0;
-  uint32_t top = 0u;
-  const int words = (n + 31) >> 5, quads = 8 * words;  // the staged row is padded with zeros, which no pass counts
-  auto stage = [&]() {
-    if (value.quads()) {
-#pragma unroll 4
-      for (int q = tid; q < quads; q += T) {
-        const float4 v = 4 * q < n ? value.quad(q) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        *reinterpret_cast<float4*>(vals + 4 * q) = v;
-        top = max(max(top, max(magnitude_bits(v.x), magnitude_bits(v.y))), max(magnitude_bits(v.z), magnitude_bits(v.w)));
-      }
-    } else {
-#pragma unroll 8
-      for (int i = tid; i < 32 * words; i += T) {
-        const float v = i < n ? value(i) : 0.0f;
-        vals[i] = v;
-        top = max(top, magnitude_bits(v));
-      }
-    }
-  };
-  stage();
+  const int words = (n + 31) >> 5, quads = 8 * words;
+  uint32_t top = source.template stage<T>(vals, quads, bs);
   top = __reduce_max_sync(0xFFFFFFFFu, top);
   if (lane == 0) bs->wmax[warp] = top;
   __syncthreads();
@@ -428,7 +443,7 @@ __device__ __forceinline__ void block_code_row(Value value, int n, unsigned char
     if (retry) {
       __syncthreads();
       block_sort_code<T>(reinterpret_cast<uint32_t*>(vals), n, bs);
-      stage();  // for the mask
+      source.template restage<T>(vals, quads);  // for the mask
       __syncthreads();
     }
     res = bs->result;
@@ -460,6 +475,7 @@ __device__ __forceinline__ void block_code_row(Value value, int n, unsigned char
   }
   for (int w = words + tid; w < out.ld; w += T)
     if (DAB_IN_BOUNDS(row * out.ld + w, out.rows * out.ld)) mrow[w] = 0u;
+  source.template finish<T>(vals, res);
 }
 
 }  // namespace dab
