@@ -16,9 +16,10 @@
 //              them as its base.  The mask is a threshold compare over the patch.
 // The bounds are evaluated in fp32 from fp64 inputs with a relative margin of 2e-5 (see prune_margin); a patch the
 // search does not settle (a hull above the cap, a degenerate row, an extreme dynamic range, a NaN or infinity in
-// the tile) is marked K = kRowMark and coded by the full-sort kernel that follows on the stream.
+// the tile) is marked K = kRowMark and coded by the CTA-per-patch kernel of patchrows.cu that follows on the stream.
 #include <cmath>
 
+#include "bucket_bound.cuh"
 #include "histcode.cuh"
 #include "rowcode.cuh"
 
@@ -32,8 +33,6 @@ namespace {
 
 constexpr int kPixUnroll = DAB_PIX_UNROLL;
 
-constexpr int kFixWarps = 8;      // warps of the kernel that sorts the marked patches
-constexpr int kFixThreads = kFixWarps * 32;
 constexpr int kHullCap = 256;        // values the exact search takes at most from the per-warp scratch array (8 per lane)
 constexpr int kHullCapRegs = 1024;   // the same when the hull goes straight into registers (3 x 3 windows; 32 per lane)
 
@@ -73,7 +72,7 @@ struct PixQuant {
   int shift;  // per-octave grid: 23 - m; 0: equal widths
   int p;      // per-octave grid: the base of the shifted bit pattern; equal widths: the bits of 2^k as a float
   int B0;     // first bucket of the positive values (0: none negative, B: none positive, B/2: both signs)
-  bool ok;    // false: magnitudes outside [2^-40, 2^40]; the tile goes to the sorting kernel
+  bool ok;    // false: magnitudes outside [2^-40, 2^40]; the tile goes to the CTA-per-patch kernel
 };
 
 #ifndef DAB_PIX_COST_PATCH
@@ -153,20 +152,6 @@ __device__ __forceinline__ void pix_bucket_range(const PixQuant& q, int b, int B
   vhi = vlo + width;
   inv_width = (double)__int_as_float(q.p);
 }
-
-// Objective in fp32 from fp64 coordinates: every input is rounded once (relative 2^-24), both terms are
-// non-negative, the two quotients are good to 2 ulp: the result is within 1e-6 relative of the exact value for
-// results inside the normal fp32 range.  s = 0 and s = n stand for the limits (P = 0 resp. P = T there).
-__device__ __forceinline__ float objective_bound(double s, double P, double T, double nd) {
-  const float Pf = (float)P, Qf = (float)(T - P), sf = (float)s, rf = (float)(nd - s);
-  const float a = sf > 0.0f ? __fdividef(Pf * Pf, sf) : 0.0f;
-  const float b = rf > 0.0f ? __fdividef(Qf * Qf, rf) : 0.0f;
-  return a + b;
-}
-
-// A candidate is kept if its fp32 value reaches best * prune_margin: with both sides within 1e-6 of their exact
-// values, anything whose exact bound reaches the exact best edge value is kept.
-constexpr float prune_margin = 0.99998f;
 
 template <int E, bool kTable>
 __device__ __noinline__ RowResult pix_sort_select(const uint32_t* scratch, int m, int z, int n, int lane,
@@ -323,7 +308,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) binarize_patches_pixhist_ker
     const bool any_nonzero = tkmin <= tkmax;
     PixQuant qz = make_pix_quant<kOctaves>(any_nonzero ? tkmin : kZeroKey + 1u, any_nonzero ? tkmax : kZeroKey + 1u, LOG2B);
     if (any_nonzero && (key_range_nonfinite(tkmin, tkmax) || !qz.ok)) {
-      // every patch of the tile is left to the sorting kernel
+      // every patch of the tile is left to the CTA-per-patch kernel
       for (int p = threadIdx.x; p < npatch; p += THREADS) {
         const int64_t pi = tile_base + (int64_t)(p / tw) * a.Wo + p % tw;
         if (DAB_IN_BOUNDS(pi, patch_count(a))) a.pK[pi] = kRowMark;
@@ -646,61 +631,6 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) binarize_patches_pixhist_ker
   }
 }
 
-// ---------------------------------------------------------------------------------------------------------
-// The kernel that follows on the stream: patches marked K = kRowMark are coded by the full sort of rowcode.cuh,
-// one CTA (a group of 8 warps) per marked patch, values read straight from global memory.  Every CTA looks at a
-// run of `run` (32 to 256) patch slots at a time and queues the marked ones; short runs spread the marked patches
-// of a small layer over all SMs.
-// ---------------------------------------------------------------------------------------------------------
-template <int R>
-__global__ void __launch_bounds__(kFixThreads) binarize_patches_fixup_kernel(const PixArgs a, int scratch_words, int run) {
-  constexpr int W = kFixWarps;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  GroupShared* gs = reinterpret_cast<GroupShared*>(smem_raw);
-  uint32_t* scratch = reinterpret_cast<uint32_t*>(gs + 1);
-  int* queue = reinterpret_cast<int*>(scratch + scratch_words);
-  __shared__ int qn;
-  const int tig = threadIdx.x;
-  const int64_t total = (int64_t)a.d.N * a.Ho * a.Wo;
-  const int khw = a.d.kh * a.d.kw;
-  for (int64_t chunk = (int64_t)blockIdx.x * run; chunk < total; chunk += (int64_t)gridDim.x * run) {
-    __syncthreads();
-    if (tig == 0) qn = 0;
-    __syncthreads();
-    if (tig < run && chunk + tig < total && a.pK[DAB_IDX(chunk + tig, total)] == kRowMark) queue[atomicAdd(&qn, 1)] = tig;
-    __syncthreads();
-    const int count = qn;
-    for (int qi = 0; qi < count; ++qi) {
-      const int64_t pi = chunk + queue[qi];
-      const int wo = (int)(pi % a.Wo);
-      const int ho = (int)((pi / a.Wo) % a.Ho);
-      const int img = (int)(pi / ((int64_t)a.Wo * a.Ho));
-      const float* ximg = a.x + (int64_t)img * a.d.C * a.d.H * a.d.W;
-      const int hb = ho * a.d.stride_h - a.d.pad_h, wb = wo * a.d.stride_w - a.d.pad_w;
-      auto keyof = [&](int i) {
-        const int c = i / khw, rs = i - c * khw;
-        const int r = rs / a.d.kw, s = rs - r * a.d.kw;
-        const int h = hb + r, w = wb + s;
-        float v = 0.0f;
-        if ((unsigned)h < (unsigned)a.d.H && (unsigned)w < (unsigned)a.d.W)
-          v = __ldg(ximg + DAB_IDX(((int64_t)c * a.d.H + h) * a.d.W + w, (int64_t)a.d.C * a.d.H * a.d.W));
-        return order_key(v);
-      };
-      uint32_t kreg[R];
-      group_code_row<W, R, false, false>(keyof, a.n, tig, scratch, gs, 1, nullptr, kreg);
-      const RowResult res = gs->result;
-      if (tig == 0 && DAB_IN_BOUNDS(pi, total)) {
-        a.pK[pi] = res.K;
-        a.pgamma[pi] = res.alpha;
-        a.pdelta[pi] = res.beta;
-        if (a.pflags) a.pflags[pi] = res.flags;
-      }
-      group_store_mask<W, R, false>(kreg, a.n, a.ldp, tig, res, a.pmask, pi, total);
-      group_barrier(1, 32 * W);  // gs->result is overwritten by the next patch
-    }
-  }
-}
-
 void set_pix_tile(const dab_conv_desc& d, int Ho, int Wo, int th, int tw, PixArgs* a) {
   const int TH = th < Ho ? th : Ho, TW = tw < Wo ? tw : Wo;
   a->TH = TH; a->TW = TW;
@@ -824,25 +754,9 @@ cudaError_t launch_pix_for(PixArgs& a, cudaStream_t stream, bool* applicable) {
   return launch_pix<BPL, 0, uint16_t, kTable>(a, stream, applicable);
 }
 
-template <int R>
-cudaError_t launch_fixup(const PixArgs& a, cudaStream_t stream) {
-  const int sw = scratch_words_for(a.n, kFixWarps);
-  const size_t smem = sizeof(GroupShared) + sizeof(uint32_t) * (size_t)sw + sizeof(int) * kFixThreads;
-  auto kern = binarize_patches_fixup_kernel<R>;
-  cudaError_t e = ensure_dynamic_smem(kern, smem);
-  if (e != cudaSuccess) return e;
-  const int64_t total = (int64_t)a.d.N * a.Ho * a.Wo;
-  int run = kFixThreads;  // patch slots a CTA scans at a time: fewer for small layers, so that every SM gets some
-  while (run > 32 && (total + run - 1) / run < 4 * (int64_t)sm_count()) run >>= 1;
-  int64_t blocks = (total + run - 1) / run;
-  if (blocks > sm_count() * 4) blocks = sm_count() * 4;
-  kern<<<(unsigned)blocks, kFixThreads, smem, stream>>>(a, sw, run);
-  return cudaGetLastError();
-}
-
 }  // namespace
 
-// Patches of 257..8192 values through the pixel-histogram coder and the kernel that sorts what it marked.
+// Patches of 257..8192 values through the pixel-histogram coder and the kernel that codes what it marked.
 // *applicable = false (nothing launched) when the geometry has no tile that fits shared memory.
 cudaError_t launch_binarize_patches_pixhist(const dab_conv_desc& d, int32_t Ho, int32_t Wo, const float* x,
                                             int32_t* pK, float* pgamma, float* pdelta, uint32_t* pmask, int32_t ldp,
@@ -861,9 +775,7 @@ cudaError_t launch_binarize_patches_pixhist(const dab_conv_desc& d, int32_t Ho, 
   else if (a.n < DAB_PIX_N4) e = launch_pix_for<2>(a, stream, applicable);
   else e = launch_pix_for<4>(a, stream, applicable);
   if (e != cudaSuccess || !*applicable) return e;
-  if (a.n <= 2048) return launch_fixup<8>(a, stream);
-  if (a.n <= 4096) return launch_fixup<16>(a, stream);
-  return launch_fixup<32>(a, stream);
+  return launch_binarize_patches_bucket(d, Ho, Wo, x, pK, pgamma, pdelta, pmask, ldp, pflags, /*marked_only=*/true, stream);
 }
 
 }  // namespace dab
