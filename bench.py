@@ -27,7 +27,7 @@ WORDS_PER_POPC = 1.5              # the contraction compresses 3 AND-ed words in
 
 
 # Sources of the patch coder: a measured DRAM-traffic record is only quoted while these files are unchanged.
-PATCH_CODER_SOURCES = ("pixhist.cu", "patches.cu", "rowcode.cuh", "histcode.cuh", "common.cuh")
+PATCH_CODER_SOURCES = ("pixtile.cu", "patchrows.cu", "patches.cu", "rowbucket.cuh", "rowcode.cuh", "common.cuh")
 TRAFFIC_RECORD = os.path.join(ROOT, "profiles", "patch_coder_dram_traffic.json")
 
 
@@ -235,7 +235,9 @@ def patch_launches(L, coder):
         return 1
     pixel = n <= 8192 and L.kh * L.kw >= 4 and L.patches >= 1024
     if coder == "pixel" or (coder == "auto" and pixel):
-        return 2                      # pixel-histogram coder, then the kernel that sorts the patches it marked
+        return 2                      # tile coder, then the kernel that codes the patches it marked
+    if coder == "auto" and (L.kh * L.kw >= 4 or L.patches < 1024 or n > 8192):
+        return 1                      # a CTA per patch
     if coder == "auto":
         return 3                      # sort-based coder, histogram coder on the dense tiles, group kernel on the rest
     if coder == "hist":
@@ -396,7 +398,7 @@ def run_dab(args):
     patch_bytes = sum(4 * L.N * L.C * L.H * L.W + L.patches * (4 * dab.dab_words_per_row(L.n) + 12) for L in layers)
     binarize_gbs = patch_bytes * args.steps / (k_ms["binarize_patches"] * 1e-3) / 1e9
     traffic = measured_patch_coder_traffic([L.name for L in layers], args.batch, args.dense) if args.patch_coder == "auto" else None
-    roofline = {"kernel": "binarize_patches_pixhist_kernel (+ binarize_patches_fixup_kernel, which finds nothing marked on "
+    roofline = {"kernel": "binarize_patches_tile_kernel (+ binarize_patches_marked_kernel, which finds nothing marked on "
                           "this workload)", "bound": "hbm", "achieved": binarize_gbs,
                 "peak": hbm_peak, "unit": "GB/s", "frac": binarize_gbs / hbm_peak, "traffic": traffic,
                 "traffic_note": "dram__bytes_read.sum + dram__bytes_write.sum per layer launch, average over the layers, from "

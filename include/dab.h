@@ -364,21 +364,23 @@ dab_contraction dab_get_contraction(void);
  * in dab_binarize (Section 4.1 / Algorithm 1 per row; every choice gives the same codes bit for bit):
  *   DAB_PATCHES_SORT   every row is sorted in full (its exact zeros are only counted) and every split evaluated;
  *   DAB_PATCHES_PIXEL  patches of 257..8192 values: the values of every input pixel (its C channels) are counted once
- *                      per tile into buckets of power-of-two width, with exact fp64 sums; a patch adds the tables of
+ *                      per tile into buckets (ranges of bit patterns), with exact fp64 sums; a patch adds the tables of
  *                      its kh*kw pixels, which gives the split size and prefix sum at every bucket edge exactly.  The
  *                      objective is convex in (split size, prefix sum), so inside a bucket it is bounded by its values
  *                      at the corners of the region the bucket's count, sum and value bounds allow; only the few
  *                      buckets whose bound reaches the best edge value are searched exactly.  Work per pixel is
  *                      shared by the up to kh*kw patches that contain it.  Patches it cannot settle (a hull of more
  *                      than 1024 values, a constant row without zeros, magnitudes outside 2^-40..2^40, a NaN or an
- *                      infinity in the tile) are sorted in full by a second kernel;
+ *                      infinity in the tile) are coded by a second kernel, a CTA per patch.  At most 512 channels and 32
+ *                      pixels per window;
  *   DAB_PATCHES_HIST   patches of 257..8192 values, one warp each: a histogram of the patch's own values
  *                      quantised to 24 bits of the tile's range, the same bound per bucket with a margin for the
  *                      quantisation, exact search of what survives; what it cannot settle falls to the sorting kernel.
  *                      Rows of a matrix of more than 256 values: a CTA per row, exact counts and sums per bucket;
- *   DAB_PATCHES_AUTO   (default) patches: DAB_PATCHES_PIXEL wherever a patch spans several pixels and the layer has
- *                      at least 1024 patches; otherwise per tile of the input the sorting kernels for tiles with few non-zero values
- *                      and DAB_PATCHES_HIST for the others.  Rows of a matrix: DAB_PATCHES_HIST.
+ *   DAB_PATCHES_AUTO   (default) patches: DAB_PATCHES_PIXEL for windows of at least four pixels; layers of few patches and
+ *                      patches of more than 8192 values a CTA per patch, which prunes by buckets of its own; windows of one to
+ *                      three pixels in larger layers per tile of the input the sorting kernels for tiles with few
+ *                      non-zero values and DAB_PATCHES_HIST for the others.  Rows of a matrix: DAB_PATCHES_HIST.
  * Process-wide, read once at the start of each call.
  */
 typedef enum { DAB_PATCHES_AUTO = 0, DAB_PATCHES_SORT = 1, DAB_PATCHES_HIST = 2, DAB_PATCHES_PIXEL = 3 } dab_patch_coder;

@@ -164,15 +164,16 @@ cudaError_t read_mma_wait_timeouts(unsigned int* count);
 cudaError_t launch_binarize_patches(const dab_conv_desc& d, int32_t Ho, int32_t Wo, const float* x, int32_t* pK,
                                     float* pgamma, float* pdelta, uint32_t* pmask, int32_t ldp, uint32_t* pflags,
                                     cudaStream_t stream);
-// Pixel-histogram patch coder (pixhist.cu): per-pixel bucket tables shared by the overlapping patches of a tile,
-// then the full-sort kernel on the patches it marked.  *applicable = false: nothing was launched (no tile fits).
-cudaError_t launch_binarize_patches_pixhist(const dab_conv_desc& d, int32_t Ho, int32_t Wo, const float* x,
-                                            int32_t* pK, float* pgamma, float* pdelta, uint32_t* pmask, int32_t ldp,
-                                            uint32_t* pflags, cudaStream_t stream, bool* applicable);
 // A CTA per patch (patchrows.cu): every patch, or those whose K holds kRowMark.
 cudaError_t launch_binarize_patches_bucket(const dab_conv_desc& d, int32_t Ho, int32_t Wo, const float* x, int32_t* pK,
                                            float* pgamma, float* pdelta, uint32_t* pmask, int32_t ldp, uint32_t* pflags,
                                            bool marked_only, cudaStream_t stream);
+// Patch coder on per-pixel bucket tables shared by the overlapping patches of a tile (pixtile.cu), then the CTA-per-patch
+// kernel on the patches it marked.  *applicable = false: nothing was launched (no tile fits or, unless `always`, a CTA per
+// patch is expected to be faster).
+cudaError_t launch_binarize_patches_tile(const dab_conv_desc& d, int32_t Ho, int32_t Wo, const float* x, int32_t* pK,
+                                         float* pgamma, float* pdelta, uint32_t* pmask, int32_t ldp, uint32_t* pflags,
+                                         bool always, cudaStream_t stream, bool* applicable);
 // Patch coder selection: 0 default, 1 sort-based only, 2 histogram-pruned per patch wherever it applies,
 // 3 pixel-histogram coder wherever it applies.
 int patch_coder_mode();

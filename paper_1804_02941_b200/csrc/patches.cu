@@ -518,19 +518,15 @@ cudaError_t launch_binarize_patches(const dab_conv_desc& d, int32_t Ho, int32_t 
   if (a.n <= 256) return launch_patches_warp<8, false>(a, stream);
   const int mode = patch_coder_mode();
   cudaError_t e;
-  // The pixel-histogram coder shares work between overlapping patches: it is the default wherever a patch spans
-  // several pixels and the layer has enough patches to fill the device with its tiles (measured: from about a
-  // thousand patches).
-  const bool pixel_default = d.kh * d.kw >= 4 && (int64_t)d.N * Ho * Wo >= 1024;
-  if (mode == 3 || (mode == 0 && pixel_default)) {
+  // The tile coder shares work between overlapping patches; a CTA per patch takes what it cannot (long rows) and layers of
+  // few patches.  What is left of the default are windows of one to three pixels in larger layers, which share little:
+  // the chain of kernels below.
+  if (mode == 3 || (mode == 0 && d.kh * d.kw >= 4)) {
     bool applicable = false;
-    e = launch_binarize_patches_pixhist(d, Ho, Wo, x, pK, pgamma, pdelta, pmask, ldp, pflags, stream, &applicable);
+    e = launch_binarize_patches_tile(d, Ho, Wo, x, pK, pgamma, pdelta, pmask, ldp, pflags, /*always=*/mode == 3, stream, &applicable);
     if (e != cudaSuccess || applicable) return e;
   }
-  // What is left of the default are layers of few patches, which a CTA per patch finishes soonest (35 us of mostly idle
-  // kernels before, 8 us now for 225 patches of 2304 values), patches of more than 8192 values, and patches of one to
-  // three pixels in larger layers, which share little: the chain of kernels below.
-  if (mode == 0 && ((int64_t)d.N * Ho * Wo < 1024 || a.n > 8192)) {
+  if (mode == 0 && (d.kh * d.kw >= 4 || (int64_t)d.N * Ho * Wo < 1024 || a.n > 8192)) {
     if (Ho == 1 && Wo == 1 && d.kh == d.H && d.kw == d.W && d.pad_h == 0 && d.pad_w == 0)  // fully connected: rows of a matrix
       return launch_binarize(x, d.N, a.n, a.n, pK, pgamma, pdelta, pmask, ldp, pflags, stream);
     return launch_binarize_patches_bucket(d, Ho, Wo, x, pK, pgamma, pdelta, pmask, ldp, pflags, /*marked_only=*/false, stream);

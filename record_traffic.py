@@ -4,7 +4,7 @@
 Capture (one B200, one pass per launch, after the same bench command has run without ncu):
 
     python bench.py --steps 1 --warmup 3 --no-e2e --no-wbin --no-cpu-baseline
-    ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none -k regex:"pixhist|patches" \\
+    ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none -k regex:binarize_patches \\
         -s <launches of the warm-up steps> -c <launches of one step> --csv --log-file traffic.csv \\
         python bench.py --steps 1 --warmup 3 --no-e2e --no-wbin --no-cpu-baseline
     python record_traffic.py traffic.csv
@@ -41,7 +41,7 @@ def main():
     if i != len(launches):
         raise SystemExit("captured %d launches, one step has %d" % (len(launches), i))
     rec = {"source_sha256": bench.patch_coder_source_hash(), "batch": 256, "dense": False,
-           "command": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none -k regex:pixhist|patches "
+           "command": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none -k regex:binarize_patches "
                       "python bench.py --steps 1 --warmup 3 --no-e2e --no-wbin --no-cpu-baseline (the timed step's launches)",
            "dram_bytes_per_launch": out}
     with open(bench.TRAFFIC_RECORD, "w") as f:
