@@ -112,29 +112,6 @@ __device__ __forceinline__ void tmem_load_8(uint32_t taddr, uint32_t (&v)[8]) {
 
 __device__ __forceinline__ void tmem_load_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// Four mask bits -> four bytes of 0/1 (bit i to byte i): the products i + 7j land on distinct bit positions.
-__device__ __forceinline__ uint32_t spread4(uint32_t nibble) { return (nibble * 0x00204081u) & 0x01010101u; }
-
-// One 16-byte piece (four mask words) of one row -> eight 16-byte K chunks in the stage.
-// dst points at the row's slot in the K chunk of the first word; consecutive K chunks are 128 bytes apart.
-__device__ __forceinline__ void expand_words(uint4 q, unsigned char* dst) {
-  const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    uint4 lo, hi;
-    lo.x = spread4(w[m] & 15u);
-    lo.y = spread4((w[m] >> 4) & 15u);
-    lo.z = spread4((w[m] >> 8) & 15u);
-    lo.w = spread4((w[m] >> 12) & 15u);
-    hi.x = spread4((w[m] >> 16) & 15u);
-    hi.y = spread4((w[m] >> 20) & 15u);
-    hi.z = spread4((w[m] >> 24) & 15u);
-    hi.w = spread4(w[m] >> 28);
-    *reinterpret_cast<uint4*>(dst + (2 * m) * 128) = lo;
-    *reinterpret_cast<uint4*>(dst + (2 * m + 1) * 128) = hi;
-  }
-}
-
 // Four mask bits -> four bytes of 0 / -1 with one byte permutation: the selector's nibbles are bits s, s+4, s+8
 // and s+12 of the word shifted right by s (their lowest bit picks byte 0x00 or 0xFF of the source; the other
 // selector bits pick among copies of the same two bytes, and sign replication of 0x00 / 0xFF changes nothing).
@@ -144,26 +121,30 @@ __device__ __forceinline__ uint32_t select4(uint32_t selector) {
   return d;
 }
 
-// One 16-byte piece (four mask words) of one row -> eight 16-byte K chunks of 0 / -1 bytes (signed 8-bit
+// One mask word of one row -> two 16-byte K chunks of 0 / -1 bytes (signed 8-bit
 // operands: (-1) x (-1) = 1, so the integer dot product of two such rows is popc(e AND f)).  Within a word's
 // 32 bytes the bits appear in the order 0 4 8 12, 1 5 9 13, 2 6 10 14, 3 7 11 15, then the same for the upper
 // half: a permutation of the contraction index, the same on both operands, that the sum does not see.
+__device__ __forceinline__ void expand_word_signed(uint32_t w, unsigned char* dst) {
+  uint4 lo, hi;
+  lo.x = select4(w);
+  lo.y = select4(w >> 1);
+  lo.z = select4(w >> 2);
+  lo.w = select4(w >> 3);
+  hi.x = select4(w >> 16);
+  hi.y = select4(w >> 17);
+  hi.z = select4(w >> 18);
+  hi.w = select4(w >> 19);
+  *reinterpret_cast<uint4*>(dst) = lo;
+  *reinterpret_cast<uint4*>(dst + 128) = hi;
+}
+
+// One 16-byte piece (four mask words) of one row -> eight 16-byte K chunks.
 __device__ __forceinline__ void expand_words_signed(uint4 q, unsigned char* dst) {
-  const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    uint4 lo, hi;
-    lo.x = select4(w[m]);
-    lo.y = select4(w[m] >> 1);
-    lo.z = select4(w[m] >> 2);
-    lo.w = select4(w[m] >> 3);
-    hi.x = select4(w[m] >> 16);
-    hi.y = select4(w[m] >> 17);
-    hi.z = select4(w[m] >> 18);
-    hi.w = select4(w[m] >> 19);
-    *reinterpret_cast<uint4*>(dst + (2 * m) * 128) = lo;
-    *reinterpret_cast<uint4*>(dst + (2 * m + 1) * 128) = hi;
-  }
+  expand_word_signed(q.x, dst);
+  expand_word_signed(q.y, dst + 256);
+  expand_word_signed(q.z, dst + 512);
+  expand_word_signed(q.w, dst + 768);
 }
 
 }  // namespace tc

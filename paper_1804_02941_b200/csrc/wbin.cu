@@ -10,14 +10,21 @@
 // accumulators per output in tensor memory; M1 = a3 2^24 + a2 2^16 + a1 2^8 + a0 (times 2^-sexp).  The only
 // error is the rounding of x_i to q_i: at most 2^-32 of the row's largest magnitude per element.
 //
-// A CTA owns a tile of TH x TW output positions of one image (at most 128 = the lanes of tensor memory; of
-// several images when a whole image is smaller than that) and 64 filters.  It never forms patches in global memory: for each group of 128 patch elements it stages the
-// channels they come from in shared memory, and every thread gathers 16 consecutive elements of its row,
-// converts them and stores one 16-byte K chunk per byte plane in the operand layout of tc.cuh.
+// A CTA owns up to 128 output positions (the lanes of tensor memory) and 64 or 128 filters (4 accumulators each: 512 columns).
+// Positions are consecutive in a strip of at most 32 output columns that runs through all images, so that a tile is full
+// whatever the image size.  Patches are never formed in global memory: for each group of JS mask words (32 JS patch elements)
+// the CTA stages the channels they come from in shared memory, and every thread gathers 16 elements of its row at a time,
+// converts them and stores one 16-byte K chunk per byte plane in the operand layout of tc.cuh.  Both the staged channels and
+// the operands are double-buffered: while the tensor cores work on one stage the threads convert the next.
+//
+// Bound by shared memory: per stage of 128 elements and 128 filters the tensor cores read 128 KB of operands, the gather
+// 64 KB of values (twice where lanes of a warp lie in different output rows) and writes 64 KB.  The conversion, some 8
+// instructions per element, is what a CTA of 128 filters halves over one of 64.
 #include <algorithm>
 #include <climits>
 
 #include "common.cuh"
+#include "rowcode.cuh"
 #include "tc.cuh"
 
 namespace dab {
@@ -27,21 +34,16 @@ using namespace tc;
 
 __device__ unsigned int g_wbin_wait_timeouts;
 
-constexpr int WB_THREADS = 256;
-constexpr int WB_JS = 4;                         // mask words (k-steps of 32 elements) per stage
-constexpr int WB_KS = WB_JS * 32;                // patch elements per stage
-constexpr int WB_KC = WB_JS * 2;                 // 16-byte K chunks per stage
-constexpr int WB_NT = 64;                        // filters per CTA
-constexpr uint32_t WB_SBO = WB_KC * 128;         // bytes between groups of 8 rows
-constexpr uint32_t WB_PLANE = kLanes * WB_KS;    // bytes of one byte plane of the activation stage
-constexpr uint32_t WB_BSTAGE = WB_NT * WB_KS;    // bytes of the filter stage
+constexpr int WB_THREADS = 512;
 
 struct WbinArgs {
   dab_conv_desc d;
   int32_t Ho, Wo, n, words, khw;
-  int32_t TH, TW, TI, tiles_h, tiles_w;  // tile: TI images x TH x TW output positions (TI > 1 only when one tile covers an image)
-  int32_t in_h, in_w, pitch, ch_words, max_ch;
-  uint32_t magic_npix, magic_in_w, magic_khw, magic_kw;  // ceil(2^32 / d): floor(i / d) = umulhi(i, magic); 0 if d == 1
+  int32_t R, TW, strips;       // positions per tile; columns per strip; strips
+  int32_t in_w, pitch;         // staged columns; words per staged row
+  int32_t ch_words, max_ch;    // words per staged channel, channels per stage (both at most)
+  int32_t row_slots;           // 64 or 128: rows that the threads are spread over
+  uint32_t magic_khw, magic_kw;  // ceil(2^32 / d): floor(i / d) = umulhi(i, magic); 0 if d == 1
   const float* x;
   const uint32_t* pixmax;  // N x H x W: largest magnitude over the channels, as a bit pattern
   const uint32_t* wmask;
@@ -65,22 +67,26 @@ __device__ __forceinline__ void byte_planes(uint32_t q0, uint32_t q1, uint32_t q
   out[3] = __byte_perm(b, d, 0x7632);
 }
 
-// Sixteen consecutive elements (K chunk kc of the stage) of one row: gathered through the offset table, scaled
+// Place of a stage's element in its operand row: the order of expand_word_signed within a mask word.
+__device__ __forceinline__ int element_of_place(int i) { return (i & ~15) + ((i & 15) >> 2) + 4 * (i & 3); }
+
+// Sixteen elements (K chunk kc of the stage) of one row: gathered through the offset table, scaled
 // by 2^sexp in two exact steps, rounded to 32-bit integers, split into byte planes and stored as one 16-byte K
 // chunk per plane; the byte sums of the planes accumulate in psum.  kChecked: elements from `limit` on are 0.
 // kTwoStep: the scale is beyond one fp32 factor (patches whose largest magnitude is below 2^-70).
-template <bool kChecked, bool kTwoStep>
-__device__ __forceinline__ void gather_chunk(const float* src, const uint16_t* off, int kc, int limit, float fac,
+template <uint32_t kPlane, bool kChecked, bool kTwoStep>
+__device__ __forceinline__ void gather_chunk(const unsigned char* src, const int32_t* off, int kc, int limit, float fac,
                                              float fac2, unsigned char* dst0, int (&psum)[4]) {
   uint32_t pl[4][4];
 #pragma unroll
   for (int g4 = 0; g4 < 4; ++g4) {
+    const int4 o4 = *reinterpret_cast<const int4*>(off + kc * 16 + g4 * 4);
+    const int o[4] = {o4.x, o4.y, o4.z, o4.w};
     uint32_t q[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const int kk = kc * 16 + g4 * 4 + e;
-      float v = src[off[kk]];
-      if (kChecked && kk >= limit) v = 0.0f;
+      float v = *reinterpret_cast<const float*>(src + o[e]);
+      if (kChecked && kc * 16 + element_of_place(g4 * 4 + e) >= limit) v = 0.0f;
       v = __fmul_rn(v, fac);
       if (kTwoStep) v = __fmul_rn(v, fac2);
       q[e] = (uint32_t)__float2int_rn(v);
@@ -97,220 +103,276 @@ __device__ __forceinline__ void gather_chunk(const float* src, const uint16_t* o
   unsigned char* dst = dst0 + (uint32_t)kc * 128;
 #pragma unroll
   for (int p = 0; p < 4; ++p)
-    *reinterpret_cast<uint4*>(dst + p * WB_PLANE) = make_uint4(pl[p][0], pl[p][1], pl[p][2], pl[p][3]);
+    *reinterpret_cast<uint4*>(dst + p * kPlane) = make_uint4(pl[p][0], pl[p][1], pl[p][2], pl[p][3]);
 }
 
-__global__ void __launch_bounds__(WB_THREADS, 2) wbin_conv_kernel(const WbinArgs a) {
+// Exact for |v| < 2^31, without the conversion unit.
+__device__ __forceinline__ double signed_to_double(int v) {
+  return __dsub_rn(__hiloint2double(0x43300000, (int)((uint32_t)v ^ 0x80000000u)), 4503601774854144.0);  // 2^52 + 2^31
+}
+
+// Bytes of shared memory for the operands of one stage.
+constexpr size_t operand_bytes(int nt, int js) { return (size_t)(4 * kLanes + nt) * js * 32; }
+
+// The rows of input under a tile are staged one after another, those of an image together.  Row of output row `g` (counted
+// over all images) in the staging area, and what a staged row holds.
+struct TileRows {
+  int64_t img0;
+  int ho0, first, full, stride, Ho;  // rows staged for the first image (at most) and for a whole one
+  __device__ __forceinline__ TileRows(const WbinArgs& a, int64_t g0) : stride(a.d.stride_h), Ho(a.Ho) {
+    img0 = g0 / a.Ho;
+    ho0 = (int)(g0 - img0 * a.Ho);
+    first = (a.Ho - 1 - ho0) * stride + a.d.kh;
+    full = (a.Ho - 1) * stride + a.d.kh;
+  }
+  __device__ __forceinline__ int staged(int dg, int& di, int& ho) const {  // dg: output rows behind the tile's first one
+    di = (ho0 + dg) / Ho;
+    ho = ho0 + dg - di * Ho;
+    return di == 0 ? (ho - ho0) * stride : first + (di - 1) * full + ho * stride;
+  }
+  __device__ __forceinline__ void source(int q, int& di, int& h) const {  // (h before the padding is taken off)
+    if (q < first) { di = 0; h = ho0 * stride + q; return; }
+    di = 1 + (q - first) / full;
+    h = (q - first) % full;
+  }
+};
+
+template <int NT, int JS>
+__global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs a) {
+  constexpr int KS = JS * 32, KC = JS * 2;        // patch elements and 16-byte K chunks per stage
+  constexpr uint32_t SBO = KC * 128;              // bytes between groups of 8 rows
+  constexpr uint32_t PLANE = kLanes * KS;         // bytes of one byte plane of the activations
+  constexpr uint32_t STAGE = 4 * PLANE + NT * KS;
+  static_assert(NT * JS <= WB_THREADS, "a mask word per thread and stage");
   extern __shared__ __align__(128) unsigned char dyn_mem[];
-  __shared__ __align__(8) uint64_t s_bar;
+  __shared__ __align__(8) uint64_t s_bar[2];
   __shared__ uint32_t s_tmem;
-  __shared__ int s_rowsexp[kLanes];      // scale exponent of a row; INT_MIN: row not in the image; INT_MAX: non-finite
-  __shared__ int s_rowsum[2][kLanes][4]; // byte-plane sums of q over the row, one set per gathering thread
-  __shared__ double s_alpha[WB_NT], s_beta[WB_NT];
-  __shared__ uint16_t s_off[2][WB_KS];
+  __shared__ int s_rowsexp[kLanes];               // scale exponent of a row; INT_MIN: not in the image; INT_MAX: non-finite
+  __shared__ double s_alpha[NT], s_beta[NT];
+  __shared__ __align__(16) int32_t s_off[2][KS];  // byte offsets of a stage's elements in the staged channels
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t mem0 = (smem_u32(dyn_mem) + 127u) & ~127u;
-  unsigned char* const stage_a = dyn_mem + (mem0 - smem_u32(dyn_mem));
-  unsigned char* const stage_b = stage_a + 4 * WB_PLANE;
-  // two input tiles: the next group of channels arrives while the current one is gathered
-  const int img_words = a.max_ch * a.ch_words;  // staged words of one image of the tile
-  const int tile_words = a.TI * img_words;
-  float* const tiles = reinterpret_cast<float*>(stage_b + WB_BSTAGE);
-  uint32_t* const pixmax = reinterpret_cast<uint32_t*>(tiles + 2 * (size_t)tile_words);
-  const uint32_t bar = smem_u32(&s_bar);
+  unsigned char* const operands = dyn_mem + (mem0 - smem_u32(dyn_mem));
+  const int tile_words = a.max_ch * a.ch_words;
+  float* const tiles = reinterpret_cast<float*>(operands + 2 * STAGE);
+  int32_t* const goff = reinterpret_cast<int32_t*>(tiles + 2 * (size_t)tile_words);  // [pixel] place in x; -1: outside
+  uint32_t* const pixmax = reinterpret_cast<uint32_t*>(tiles);                        // [pixel]; until channels are staged
+  int4* const rowsum = reinterpret_cast<int4*>(operands);  // [thread] byte-plane sums of q over its part of the row; at the end
+  const uint32_t bar0 = smem_u32(&s_bar[0]), bar1 = smem_u32(&s_bar[1]);
 
-  // tile of this CTA
-  const int tiles_per_img = a.tiles_h * a.tiles_w;
-  const int img0 = (blockIdx.x / tiles_per_img) * a.TI, trem = blockIdx.x % tiles_per_img;
-  const int imgs = min(a.TI, a.d.N - img0);  // images of this tile
-  const int ho0 = (trem / a.tiles_w) * a.TH, wo0 = (trem % a.tiles_w) * a.TW;
-  const int h0 = ho0 * a.d.stride_h - a.d.pad_h, w0 = wo0 * a.d.stride_w - a.d.pad_w;
-  const int j0 = blockIdx.y * WB_NT;
-  const int64_t img_stride = (int64_t)a.d.C * a.d.H * a.d.W;
-  const float* const x0 = a.x + (int64_t)img0 * img_stride;
-  const int npix = a.in_h * a.in_w;
+  // tile of this CTA: positions f0 .. f0 + R - 1 of its strip
+  const int strip = blockIdx.x % a.strips, wo0 = strip * a.TW;
+  const int64_t f0 = (int64_t)(blockIdx.x / a.strips) * a.R, total = (int64_t)a.d.N * a.Ho * a.TW;
+  const int rows = (int)min((int64_t)a.R, total - f0);
+  const int64_t g0 = f0 / a.TW;
+  const int lead = (int)(f0 - g0 * a.TW);  // positions of the first output row before the tile
+  const TileRows map(a, g0);
+  const int w0 = wo0 * a.d.stride_w - a.d.pad_w;
+  const int j0 = blockIdx.y * NT;
+  const int plane_in = a.d.H * a.d.W;
+  const int64_t img_stride = (int64_t)a.d.C * plane_in;
+  const float* const x0 = a.x + map.img0 * img_stride;
+  int pixels;  // staged words per channel
+  {
+    int di, ho;
+    pixels = (map.staged((lead + rows - 1) / a.TW, di, ho) + a.d.kh) * a.pitch;
+  }
 
-  if (warp == 0) tmem_alloc(smem_u32(&s_tmem), 4 * WB_NT);
+  if (warp == 0) tmem_alloc(smem_u32(&s_tmem), 4 * NT);
   if (tid == 0) {
-    mbar_init(bar, 1);
+    mbar_init(bar0, 1);
+    mbar_init(bar1, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int j = tid; j < WB_NT; j += WB_THREADS) {
+  for (int j = tid; j < NT; j += WB_THREADS) {
     const bool in = j0 + j < a.d.Cout;
     s_alpha[j] = in ? (double)a.walpha[j0 + j] : 0.0;
     s_beta[j] = in ? (double)a.wbeta[j0 + j] : 0.0;
   }
-  // per-pixel maxima of the staged region (0 outside the image)
-  for (int idx = tid; idx < imgs * npix; idx += WB_THREADS) {
-    const int ti = fast_div(idx, a.magic_npix), pix = idx - ti * npix;
-    const int r = fast_div(pix, a.magic_in_w), s = pix - r * a.in_w;
-    const int h = h0 + r, w = w0 + s;
-    uint32_t m = 0u;
-    if ((unsigned)h < (unsigned)a.d.H && (unsigned)w < (unsigned)a.d.W)
-      m = __ldg(a.pixmax + ((int64_t)(img0 + ti) * a.d.H + h) * a.d.W + w);
-    pixmax[idx] = m;
+  // where the staged words come from, and the per-pixel maxima (0 outside the image)
+  for (int i = tid; i < pixels; i += WB_THREADS) {
+    const int q = i / a.pitch, s = i - q * a.pitch, w = w0 + s;
+    int di, h;
+    map.source(q, di, h);
+    h -= a.d.pad_h;
+    const bool in = s < a.in_w && (unsigned)h < (unsigned)a.d.H && (unsigned)w < (unsigned)a.d.W && map.img0 + di < a.d.N;
+    goff[i] = in ? di * (int)img_stride + h * a.d.W + w : -1;
+    pixmax[i] = in ? __ldg(a.pixmax + (map.img0 + di) * plane_in + (int64_t)h * a.d.W + w) : 0u;
   }
   __syncthreads();
 
-  // Row = output position (lh, lw) of the tile; its scale comes from the largest magnitude of its patch.
-  const int row = tid & (kLanes - 1), half = tid >> 7;
-  const int per_img = a.TH * a.TW;
-  const int rti = row / per_img, rrem = row - rti * per_img;  // image of the tile, position inside it
-  const int lh = rrem / a.TW, lw = rrem - lh * a.TW;
-  const bool row_in = rti < imgs && ho0 + lh < a.Ho && wo0 + lw < a.Wo;
-  const int origin = rti * img_words + lh * a.d.stride_h * a.pitch + lw * a.d.stride_w;
-  if (tid < kLanes) {
-    int sexp = INT_MIN;
-    if (row_in) {
-      uint32_t m = 0u;
-      for (int i = 0; i < a.d.kh; ++i)
-        for (int j = 0; j < a.d.kw; ++j)
-          m = max(m, pixmax[rti * npix + (lh * a.d.stride_h + i) * a.in_w + lw * a.d.stride_w + j]);
-      if (m >= 0x7F800000u) sexp = INT_MAX;
-      else if (m == 0u) sexp = 0;
-      else sexp = 30 - ((int)(m >> 23) - 127);  // -97 .. 157 (the largest for a subnormal maximum)
+  // Row = output position; its scale comes from the largest magnitude of its patch.
+  const int slots = a.row_slots, groups = WB_THREADS / slots;
+  auto locate = [&](int r, int64_t& img, int& ho, int& lw) {  // returns the first staged word of the row's window
+    const int dg = (lead + r) / a.TW;
+    lw = lead + r - dg * a.TW;
+    int di;
+    const int q = map.staged(dg, di, ho);
+    img = map.img0 + di;
+    return q * a.pitch + lw * a.d.stride_w;
+  };
+  const int row = tid & (slots - 1), group = tid / slots;
+  int origin = 0;
+  {
+    int64_t img;
+    int ho, lw = 0;
+    if (row < rows) origin = locate(row, img, ho, lw);
+    if (tid < kLanes) {
+      int sexp = INT_MIN;
+      if (tid < rows && wo0 + lw < a.Wo) {  // (rows <= slots: row = tid here)
+        uint32_t m = 0u;
+        for (int i = 0; i < a.d.kh; ++i)
+          for (int j = 0; j < a.d.kw; ++j) m = max(m, pixmax[origin + i * a.pitch + j]);
+        if (m >= 0x7F800000u) sexp = INT_MAX;
+        else if (m == 0u) sexp = 0;
+        else sexp = 30 - ((int)(m >> 23) - 127);  // -97 .. 157 (the largest for a subnormal maximum)
+      }
+      s_rowsexp[tid] = sexp;
     }
-    s_rowsexp[row] = sexp;
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = s_tmem;
   const int my_sexp = s_rowsexp[row];
-  const bool gather = row_in && my_sexp != INT_MAX;
+  const bool gather = my_sexp != INT_MIN && my_sexp != INT_MAX;
   // x * 2^sexp in two exact steps: 2^sexp itself is beyond fp32 for the smallest patches
   const int sexp1 = gather ? min(my_sexp, 100) : 0, sexp2 = gather ? my_sexp - sexp1 : 0;
   const float fac = __int_as_float((sexp1 + 127) << 23), fac2 = __int_as_float((sexp2 + 127) << 23);
-  const uint32_t idesc_u = instr_desc(WB_NT, false), idesc_s = instr_desc(WB_NT, true);
 
-  int psum[4] = {0, 0, 0, 0};
-  bool dead = false;
-  uint32_t parity = 0;
-  const int stages = (a.words + WB_JS - 1) / WB_JS;
+  const int stages = (a.words + JS - 1) / JS;
   // Asynchronous copy of the channels that stage `st` draws from into tile buffer st & 1, and the offsets of its
-  // elements inside that tile.
+  // elements inside that tile.  A thread keeps to one pixel where there are few.
+  const int copies = max(1, WB_THREADS / pixels);
+  const int pix0 = copies > 1 ? tid % pixels : tid, c_first = copies > 1 ? tid / pixels : 0;
   auto stage_in = [&](int st) {
-    const int k0 = st * WB_KS, k1 = min(a.n, k0 + WB_KS);
-    const int c_lo = fast_div(k0, a.magic_khw), c_hi = fast_div(k1 - 1, a.magic_khw) + 1;
-    for (int ti = 0; ti < imgs; ++ti) {
-      float* const tile = tiles + (st & 1) * tile_words + ti * img_words;
-      const float* const ximg = x0 + ti * img_stride;
-      for (int idx = tid; idx < (c_hi - c_lo) * npix; idx += WB_THREADS) {
-        const int c = fast_div(idx, a.magic_npix), pix = idx - c * npix;
-        const int r = fast_div(pix, a.magic_in_w), s = pix - r * a.in_w;
-        const int h = h0 + r, w = w0 + s;
-        const bool in = (unsigned)h < (unsigned)a.d.H && (unsigned)w < (unsigned)a.d.W;
-        const float* src = in ? ximg + ((int64_t)(c_lo + c) * a.d.H + h) * a.d.W + w : ximg;
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(tile + c * a.ch_words + r * a.pitch + s)),
-                     "l"(src), "r"(in ? 4 : 0)
-                     : "memory");  // source size 0: the word is filled with zeros
+    const int k0 = st * KS, k1 = min(a.n, k0 + KS);
+    const int c_lo = fast_div(k0, a.magic_khw), nch = fast_div(k1 - 1, a.magic_khw) + 1 - c_lo;
+    float* const tile = tiles + (st & 1) * tile_words;
+    if (c_first < copies)
+      for (int i = pix0; i < pixels; i += copies > 1 ? pixels : WB_THREADS) {
+        const int at = goff[i];
+        const float* src = at >= 0 ? x0 + at + (int64_t)(c_lo + c_first) * plane_in : x0;
+        const int64_t step = at >= 0 ? (int64_t)copies * plane_in : 0;
+        uint32_t dst = smem_u32(tile + c_first * a.ch_words + i);
+        for (int c = c_first; c < nch; c += copies) {
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(at >= 0 ? 4 : 0)
+                       : "memory");  // source size 0: the word is filled with zeros
+          src += step;
+          dst += (uint32_t)(copies * a.ch_words) * 4;
+        }
       }
-    }
     asm volatile("cp.async.commit_group;" ::: "memory");
-    if (tid < WB_KS) {
-      const int k = k0 + tid;
-      int o = 0;  // beyond the patch length: any staged word (the gather replaces it by 0)
+    if (tid < KS) {
+      const int k = k0 + element_of_place(tid);
+      int o = 0;  // beyond the patch length: any word of the patch (the gather replaces it by 0)
       if (k < a.n) {
         const int c = fast_div(k, a.magic_khw), rs = k - c * a.khw;
         const int r = fast_div(rs, a.magic_kw), s = rs - r * a.d.kw;
         o = (c - c_lo) * a.ch_words + r * a.pitch + s;
       }
-      s_off[st & 1][tid] = (uint16_t)o;
+      s_off[st & 1][tid] = 4 * o;
     }
   };
+  // mask word of this thread: filter tid % NT, word tid / NT of the stage
+  const int mrow = tid & (NT - 1), mword = tid / NT;
+  const uint32_t* const masks = a.wmask + (int64_t)min(j0 + mrow, a.d.Cout - 1) * a.ldw;
+  auto load_mask = [&](int st) {
+    const int w = st * JS + mword;
+    return mword < JS && w < a.words ? __ldg(masks + w) : 0u;
+  };
+  const uint32_t idesc_u = instr_desc(NT, false, true), idesc_s = instr_desc(NT, true, true);
+  auto multiply = [&](int st) {  // (one thread) the products of stage `st`
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t a_addr = mem0 + (st & 1) * STAGE, b_addr = a_addr + 4 * PLANE;
+    const int kw = min(JS, a.words - st * JS);
+    for (int t = 0; t < kw; ++t) {
+      const uint64_t db = smem_desc(b_addr + t * 256, 128, SBO);
+      for (int p = 0; p < 4; ++p)
+        mma_i8(tmem + (uint32_t)(p * NT), smem_desc(a_addr + p * PLANE + t * 256, 128, SBO), db,
+               p == 3 ? idesc_s : idesc_u, (st | t) != 0);
+    }
+    mma_commit(st & 1 ? bar1 : bar0);
+  };
 
+  int psum[4] = {0, 0, 0, 0};
+  bool dead = false;
+  uint32_t next_mask = load_mask(0);
   stage_in(0);
   for (int st = 0; st < stages; ++st) {
-    const int k0 = st * WB_KS;
-    // (1) start the copy for the next stage; wait for this stage's own
+    const int k0 = st * KS;
+    const uint32_t mask = next_mask;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy stores of the last stage -> tensor-core reads
+    __syncthreads();  // this stage's channels have arrived, the last stage's operands are complete
+    if (st > 0 && tid == 0) multiply(st - 1);
     if (st + 1 < stages) {
       stage_in(st + 1);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      next_mask = load_mask(st + 1);
     }
-    __syncthreads();
-    // (2) the tensor cores have finished reading the previous contents of the operand stages
-    if (st > 0) {
-      mbar_wait(bar, parity, dead, &g_wbin_wait_timeouts);
-      parity ^= 1;
-    }
-    // (3) gather, convert, split into byte planes: thread = (row, every other 16-element chunk)
+    // the tensor cores have finished reading what these buffers held two stages ago
+    if (st > 1) mbar_wait(st & 1 ? bar1 : bar0, (uint32_t)((st >> 1) - 1) & 1u, dead, &g_wbin_wait_timeouts);
+    unsigned char* const stage_a = operands + (st & 1) * STAGE;
     if (gather) {
-      const float* const src = tiles + (st & 1) * tile_words + origin;
-      const uint16_t* const off = s_off[st & 1];
-      unsigned char* const dst0 = stage_a + (uint32_t)(row >> 3) * WB_SBO + (row & 7) * 16;
-      if (k0 + WB_KS <= a.n && sexp2 == 0) {
-#pragma unroll
-        for (int t = 0; t < WB_KC / 2; ++t) gather_chunk<false, false>(src, off, half + 2 * t, 0, fac, fac2, dst0, psum);
-      } else {  // a row length that is not a multiple of 128 (elements beyond it count as 0) or a two-step scale
-        for (int t = 0; t < WB_KC / 2; ++t) {
-          const int kc = half + 2 * t;
-          if (k0 + kc * 16 >= a.n) break;
-          gather_chunk<true, true>(src, off, kc, a.n - k0, fac, fac2, dst0, psum);
-        }
+      const unsigned char* const src = reinterpret_cast<const unsigned char*>(tiles + (st & 1) * tile_words + origin);
+      const int32_t* const off = s_off[st & 1];
+      unsigned char* const dst0 = stage_a + (uint32_t)(row >> 3) * SBO + (row & 7) * 16;
+      if (k0 + KS <= a.n && sexp2 == 0) {
+        for (int kc = group; kc < KC; kc += groups) gather_chunk<PLANE, false, false>(src, off, kc, 0, fac, fac2, dst0, psum);
+      } else {  // a row length that is not a multiple of the stage (elements beyond it count as 0) or a two-step scale
+        for (int kc = group; kc < KC && k0 + kc * 16 < a.n; kc += groups)
+          gather_chunk<PLANE, true, true>(src, off, kc, a.n - k0, fac, fac2, dst0, psum);
       }
     }
-    // (4) the masks of the 64 filters: four words of a row -> eight K chunks of 0/1 bytes
-    if (tid < WB_NT) {
-      uint4 q = make_uint4(0, 0, 0, 0);
-      const int w0m = st * WB_JS;
-      if (j0 + tid < a.d.Cout && w0m < a.ldw)
-        q = *reinterpret_cast<const uint4*>(a.wmask + (int64_t)(j0 + tid) * a.ldw + w0m);
-      expand_words(q, stage_b + (uint32_t)(tid >> 3) * WB_SBO + (tid & 7) * 16);
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy stores -> tensor-core reads
-    __syncthreads();
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t b_addr = mem0 + 4 * WB_PLANE;
-      const int kw = min(WB_JS, a.words - st * WB_JS);
-      for (int t = 0; t < kw; ++t) {
-        const uint64_t db = smem_desc(b_addr + t * 256, 128, WB_SBO);
-        for (int p = 0; p < 4; ++p)
-          mma_i8(tmem + (uint32_t)(p * WB_NT), smem_desc(mem0 + p * WB_PLANE + t * 256, 128, WB_SBO), db,
-                 p == 3 ? idesc_s : idesc_u, (st | t) != 0);
-      }
-      mma_commit(bar);
-    }
+    if (mword < JS)
+      expand_word_signed(mask, stage_a + 4 * PLANE + (uint32_t)(mrow >> 3) * SBO + (mrow & 7) * 16 + mword * 256);
   }
-  s_rowsum[half][row][0] = psum[0];
-  s_rowsum[half][row][1] = psum[1];
-  s_rowsum[half][row][2] = psum[2];
-  s_rowsum[half][row][3] = psum[3];
-  mbar_wait(bar, parity, dead, &g_wbin_wait_timeouts);  // the last commit covers every instruction before it
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncthreads();
+  if (tid == 0) multiply(stages - 1);
+  // the last commit covers every instruction before it
+  mbar_wait((stages - 1) & 1 ? bar1 : bar0, (uint32_t)((stages - 1) >> 1) & 1u, dead, &g_wbin_wait_timeouts);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  rowsum[tid] = make_int4(psum[0], psum[1], psum[2], psum[3]);  // (a wait that ran out stores nothing to y)
   __syncthreads();
 
-  // Epilogue: thread = row (a warp reads the 32 lanes of its quarter), warps 0-3 the first 32 filters, 4-7 the rest.
+  // Epilogue: thread = row (a warp reads the 32 lanes of its quarter), a quarter of the filters per four warps.
+  // The filter bytes are 0 / -1: the accumulators hold the negative sums.
   {
     const int erow = (warp & 3) * 32 + lane;
-    const int eti = erow / per_img, erem = erow - eti * per_img;
-    const int elh = erem / a.TW, elw = erem - elh * a.TW;
     const int sexp = s_rowsexp[erow];
     const bool valid = sexp != INT_MIN && !dead;
     const bool bad = sexp == INT_MAX;
-    long long S = 0;
-    double inv = 0.0;
+    double Sd = 0.0, inv = 0.0;
+    int64_t obase = 0;
+    if (valid) {
+      int64_t img;
+      int ho, lw;
+      locate(erow, img, ho, lw);
+      obase = img * a.d.Cout * a.Ho * a.Wo + (int64_t)ho * a.Wo + wo0 + lw;
+    }
     if (valid && !bad) {
-      long long s4[4];
-#pragma unroll
-      for (int p = 0; p < 4; ++p) s4[p] = (long long)s_rowsum[0][erow][p] + (long long)s_rowsum[1][erow][p];
-      S = (s4[3] << 24) + (s4[2] << 16) + (s4[1] << 8) + s4[0];
+      long long s4[4] = {0, 0, 0, 0};
+      for (int g = 0; g < groups; ++g) {
+        const int4 part = rowsum[g * slots + erow];
+        s4[0] += part.x;
+        s4[1] += part.y;
+        s4[2] += part.z;
+        s4[3] += part.w;
+      }
+      Sd = (double)((s4[3] << 24) + (s4[2] << 16) + (s4[1] << 8) + s4[0]);
       inv = __hiloint2double((1023 - sexp) << 20, 0);
     }
-    const double Sd = (double)S;
     const int64_t plane_hw = (int64_t)a.Ho * a.Wo;
-    const int64_t obase = (int64_t)(img0 + eti) * a.d.Cout * plane_hw + (int64_t)(ho0 + elh) * a.Wo + (wo0 + elw);
-    const int cb = warp >> 2;
+    static_assert(DAB_MAX_N <= (1 << 14), "255 * 257 * n must stay below 2^31");
 #pragma unroll 1
-    for (int c8 = 0; c8 < 4; ++c8) {
-      const int col = cb * 32 + c8 * 8;
+    for (int c8 = 0; c8 < NT / 32; ++c8) {
+      const int col = (warp >> 2) * (NT / 4) + c8 * 8;
       uint32_t v[4][8];
       const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col;
 #pragma unroll
-      for (int p = 0; p < 4; ++p) tmem_load_8(taddr + (uint32_t)(p * WB_NT), v[p]);
+      for (int p = 0; p < 4; ++p) tmem_load_8(taddr + (uint32_t)(p * NT), v[p]);
       tmem_load_wait();
       if (!valid) continue;
 #pragma unroll
@@ -321,9 +383,9 @@ __global__ void __launch_bounds__(WB_THREADS, 2) wbin_conv_kernel(const WbinArgs
         if (bad) {
           out = __uint_as_float(0x7FC00000u);
         } else {
-          const long long M1 = ((long long)(int)v[3][jj] << 24) + ((long long)(int)v[2][jj] << 16) +
-                               ((long long)(int)v[1][jj] << 8) + (long long)(int)v[0][jj];
-          const double m1 = (double)M1, m0 = Sd - m1;  // exact: |.| < 2^45
+          const double hi = signed_to_double(-((int)v[3][jj] * 256 + (int)v[2][jj]));
+          const double lo = signed_to_double(-((int)v[1][jj] * 256 + (int)v[0][jj]));
+          const double m1 = __fma_rn(hi, 65536.0, lo), m0 = Sd - m1;  // exact: |.| < 2^45
           const double y = __dadd_rn(__dmul_rn(s_alpha[j], m1), __dmul_rn(s_beta[j], m0));
           out = (float)__dmul_rn(y, inv);
         }
@@ -333,30 +395,67 @@ __global__ void __launch_bounds__(WB_THREADS, 2) wbin_conv_kernel(const WbinArgs
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, 4 * WB_NT);
+  if (warp == 0) tmem_dealloc(tmem, 4 * NT);
 }
 
 // Largest magnitude over the channels of every pixel, as a bit pattern (NaN > Inf > finite): what the
-// convolution kernel derives the scale of a patch from.  One thread per pixel, coalesced along the image.
-__global__ void __launch_bounds__(256) wbin_pixmax_kernel(const float* __restrict__ x, uint32_t* __restrict__ out,
-                                                          int C, int64_t HW, int64_t total) {
-  const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (idx >= total) return;
-  const int64_t img = idx / HW, p = idx - img * HW;
-  const float* src = x + img * C * HW + p;
-  uint32_t m0 = 0u, m1 = 0u, m2 = 0u, m3 = 0u;
-  int c = 0;
-  for (; c + 4 <= C; c += 4) {
-    m0 = max(m0, __float_as_uint(__ldg(src + (int64_t)c * HW)) & 0x7FFFFFFFu);
-    m1 = max(m1, __float_as_uint(__ldg(src + (int64_t)(c + 1) * HW)) & 0x7FFFFFFFu);
-    m2 = max(m2, __float_as_uint(__ldg(src + (int64_t)(c + 2) * HW)) & 0x7FFFFFFFu);
-    m3 = max(m3, __float_as_uint(__ldg(src + (int64_t)(c + 3) * HW)) & 0x7FFFFFFFu);
+// convolution kernel derives the scale of a patch from.  A CTA takes 32 pixels, its warps a share of the channels each: bound
+// by the one read of x (a thread per pixel had too few loads in flight: 35 us for 51 MB).
+constexpr int PM_WARPS = 8;
+__global__ void __launch_bounds__(32 * PM_WARPS) wbin_pixmax_kernel(const float* __restrict__ x, uint32_t* __restrict__ out,
+                                                                    int C, int64_t HW, int64_t total) {
+  __shared__ uint32_t part[PM_WARPS][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t idx = (int64_t)blockIdx.x * 32 + lane;
+  uint32_t m = 0u;
+  if (idx < total) {
+    const int64_t img = idx / HW, p = idx - img * HW;
+    const float* src = x + img * C * HW + p;
+#pragma unroll 8
+    for (int c = warp; c < C; c += PM_WARPS) m = max(m, __float_as_uint(__ldg(src + (int64_t)c * HW)) & 0x7FFFFFFFu);
   }
-  for (; c < C; ++c) m0 = max(m0, __float_as_uint(__ldg(src + (int64_t)c * HW)) & 0x7FFFFFFFu);
-  out[idx] = max(max(m0, m1), max(m2, m3));
+  part[warp][lane] = m;
+  __syncthreads();
+  if (warp == 0 && idx < total) {
+#pragma unroll
+    for (int w = 1; w < PM_WARPS; ++w) m = max(m, part[w][lane]);
+    out[idx] = m;
+  }
 }
 
 uint32_t magic_for(uint32_t d) { return d > 1 ? (uint32_t)((0x100000000ull + d - 1) / d) : 0u; }
+
+constexpr size_t kSmemLimit = 227 * 1024 - 5 * 1024;  // (static shared memory aside)
+
+// Sets the tile: strips of at most `tw` columns, R positions.  Returns the shared memory it takes with operands of the given size.
+size_t set_tile(WbinArgs* a, int tw, int R, int nt, int js) {
+  const dab_conv_desc& d = a->d;
+  a->strips = (a->Wo + tw - 1) / tw;
+  a->TW = (a->Wo + a->strips - 1) / a->strips;
+  const int64_t total = (int64_t)d.N * a->Ho * a->TW;
+  a->R = (int)std::min<int64_t>(R, total);
+  a->in_w = (a->TW - 1) * d.stride_w + d.kw;
+  a->pitch = a->in_w | 1;
+  // output rows a tile touches, the images they lie in, and the rows of input under them (all at most)
+  const int64_t all_rows = (int64_t)d.N * a->Ho;
+  const int64_t rows = std::min<int64_t>(a->R % a->TW == 0 ? a->R / a->TW : (a->R + 2 * a->TW - 2) / a->TW, all_rows);
+  const int64_t images = std::min<int64_t>(1 + (rows - 1 + a->Ho - 1) / a->Ho, d.N);
+  const int64_t staged = rows * d.stride_h + images * std::max(0, d.kh - d.stride_h);
+  a->max_ch = std::min(d.C, (js * 32 + a->khw - 2) / a->khw + 1);
+  if (staged * a->pitch > 1 << 20 || images * d.C * d.H * d.W > 0x7FFFFFFF) return SIZE_MAX;  // (32-bit places)
+  a->ch_words = (int)(staged * a->pitch);
+  return 128 + 2 * operand_bytes(nt, js) + sizeof(float) * (2 * (size_t)a->max_ch + 1) * a->ch_words;
+}
+
+template <int NT, int JS>
+cudaError_t launch_tiles(const WbinArgs& a, size_t smem, cudaStream_t stream) {
+  const int64_t gx = ((int64_t)a.d.N * a.Ho * a.TW + a.R - 1) / a.R * a.strips, gy = (a.d.Cout + NT - 1) / NT;
+  if (gx > 0x7FFFFFFF || gy > 65535) return cudaErrorInvalidValue;
+  cudaError_t e = ensure_dynamic_smem(wbin_conv_kernel<NT, JS>, smem);
+  if (e != cudaSuccess) return e;
+  wbin_conv_kernel<NT, JS><<<dim3((unsigned)gx, (unsigned)gy), WB_THREADS, smem, stream>>>(a);
+  return cudaGetLastError();
+}
 
 }  // namespace
 
@@ -370,54 +469,35 @@ cudaError_t launch_wbin_conv(const dab_conv_desc& d, int32_t Ho, int32_t Wo, con
   a.n = d.C * a.khw;
   a.words = (a.n + 31) / 32;
   a.x = x; a.wmask = wmask; a.ldw = ldw; a.walpha = walpha; a.wbeta = wbeta; a.y = y;
-  // Tile: rows of at most 16 output positions, as many rows as fit the 128 lanes, both evened out over the image.
-  const int tw_tiles = (Wo + 15) / 16;
-  a.TW = (Wo + tw_tiles - 1) / tw_tiles;
-  int TH = std::min(Ho, kLanes / a.TW);
-  const size_t fixed = 4 * (size_t)WB_PLANE + WB_BSTAGE + 128;
-  const size_t limit2 = 110 * 1024, limit1 = 227 * 1024 - 8 * 1024;  // two CTAs per SM / one
-  a.max_ch = std::min(d.C, (WB_KS + a.khw - 1) / a.khw + 1);
-  size_t smem = 0;
-  for (;;) {
-    const int th_tiles = (Ho + TH - 1) / TH;
-    a.TH = (Ho + th_tiles - 1) / th_tiles;
-    a.in_h = (a.TH - 1) * d.stride_h + d.kh;
-    a.in_w = (a.TW - 1) * d.stride_w + d.kw;
-    a.pitch = a.in_w | 1;
-    a.ch_words = a.in_h * a.pitch;
-    smem = fixed + 2 * sizeof(float) * (size_t)a.max_ch * a.ch_words + sizeof(uint32_t) * (size_t)a.in_h * a.in_w;
-    const bool offsets_fit = (size_t)a.max_ch * a.ch_words <= 65535;
-    if ((smem <= limit2 && offsets_fit) || TH == 1) break;
-    TH = a.TH - 1;
-  }
-  if (smem > limit1 || (size_t)a.max_ch * a.ch_words > 65535) return cudaErrorInvalidValue;
-  a.tiles_h = (Ho + a.TH - 1) / a.TH;
-  a.tiles_w = (Wo + a.TW - 1) / a.TW;
-  // Small images (one tile each, e.g. fully connected layers as 1x1 outputs): a tile takes as many images as
-  // fit the 128 lanes and shared memory, so that the expansion of the filter masks is shared by more rows.
-  a.TI = 1;
-  if (a.tiles_h == 1 && a.tiles_w == 1) {
-    const size_t per_img = 2 * sizeof(float) * (size_t)a.max_ch * a.ch_words + sizeof(uint32_t) * (size_t)a.in_h * a.in_w;
-    int ti = std::min<int64_t>(d.N, kLanes / (a.TH * a.TW));
-    while (ti > 1 && fixed + ti * per_img > limit1) --ti;
-    a.TI = ti;
-    smem = fixed + ti * per_img;
-  }
-  a.magic_npix = magic_for((uint32_t)(a.in_h * a.in_w));
-  a.magic_in_w = magic_for((uint32_t)a.in_w);
   a.magic_khw = magic_for((uint32_t)a.khw);
   a.magic_kw = magic_for((uint32_t)d.kw);
-  const int64_t gx = (int64_t)((d.N + a.TI - 1) / a.TI) * a.tiles_h * a.tiles_w;
-  const int64_t gy = (d.Cout + WB_NT - 1) / WB_NT;
-  if (gx > 0x7FFFFFFF || gy > 65535) return cudaErrorInvalidValue;
+  // 128 filters per CTA share one conversion; 64 where there are no more, or where 128 leave SMs idle.  With 64 rows a tile
+  // converts in half the time: for layers that do not fill the device with them either.
+  const int64_t positions = (int64_t)d.N * Ho * Wo, sms = sm_count();
+  int nt = d.Cout > 64 && (positions + 127) / 128 * ((d.Cout + 127) / 128) >= sms ? 128 : 64;
+  const int rows = (positions + 63) / 64 * ((d.Cout + nt - 1) / nt) <= sms ? 64 : kLanes;
+  // Stages of 128 elements where shared memory allows, else of 64; the fewest strips, then the most rows that fit.
+  int js = 0;
+  size_t smem = 0;
+  auto fits = [&](int tw, int R, int stage_words) {
+    smem = set_tile(&a, tw, R, nt, stage_words);
+    if (smem <= kSmemLimit) js = stage_words;
+    return js != 0;
+  };
+  for (;; nt = 64) {
+    for (int tw = 32; tw >= 1 && !js; tw >>= 1)
+      for (int R = rows; R >= (tw > 1 ? rows / 2 : 1) && !js; R -= R > 16 ? 16 : 1) fits(tw, R, 4) || fits(tw, R, 2);
+    if (js || nt == 64) break;
+  }
+  if (!js) return cudaErrorInvalidValue;
+  a.row_slots = a.R <= 64 ? 64 : kLanes;
   const int64_t HW = (int64_t)d.H * d.W, pixels = (int64_t)d.N * HW;
-  wbin_pixmax_kernel<<<(unsigned)((pixels + 255) / 256), 256, 0, stream>>>(x, pixmax, d.C, HW, pixels);
+  if ((pixels + 31) / 32 > 0x7FFFFFFF) return cudaErrorInvalidValue;
+  wbin_pixmax_kernel<<<(unsigned)((pixels + 31) / 32), 32 * PM_WARPS, 0, stream>>>(x, pixmax, d.C, HW, pixels);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  e = ensure_dynamic_smem(wbin_conv_kernel, smem);
-  if (e != cudaSuccess) return e;
-  wbin_conv_kernel<<<dim3((unsigned)gx, (unsigned)gy), WB_THREADS, smem, stream>>>(a);
-  return cudaGetLastError();
+  if (nt == 128) return js == 4 ? launch_tiles<128, 4>(a, smem, stream) : launch_tiles<128, 2>(a, smem, stream);
+  return js == 4 ? launch_tiles<64, 4>(a, smem, stream) : launch_tiles<64, 2>(a, smem, stream);
 }
 
 cudaError_t read_wbin_wait_timeouts(unsigned int* count) {
