@@ -19,13 +19,15 @@ std::atomic<int> g_contraction{(int)DAB_CONTRACT_AUTO};
 
 // The contraction kernel the process-wide setting names.  The tensor-core kernel tiles the column side
 // (weights when lanes_along_rows, activations otherwise) at least 64 rows per grid row; a launch too tall for
-// that takes the population-count kernel, and so does, under DAB_CONTRACT_AUTO, one with fewer 128 x 64 tiles
-// than a B200 has SMs: there the tensor-core kernel is a chain of dependent stage rounds on a few SMs.
+// that takes the population-count kernel, and so does, under DAB_CONTRACT_AUTO, one whose 128 x 64 tiles are
+// fewer than a third of the SMs: there the tensor-core kernel is a chain of dependent stage rounds on a few SMs, while the
+// other splits its rows.  Measured, population counts against tensor cores: 4096 x 32 of 9216 bits (32 tiles) 27 and 51 us,
+// 256 x 2000 of 1152 (64 tiles) 16.5 and 14.4, 512 x 1568 of 4608 (100 tiles) 39 and 31.
 cudaError_t contract(const GemmArgs& g, bool lanes_along_rows, cudaStream_t stream) {
   const int64_t lane_rows = lanes_along_rows ? g.M : g.N, column_rows = lanes_along_rows ? g.N : g.M;
   const int mode = g_contraction.load(std::memory_order_relaxed);
   bool tensor = mode != (int)DAB_CONTRACT_POPC && column_rows <= (int64_t)65535 * 64;
-  if (mode == (int)DAB_CONTRACT_AUTO && ((lane_rows + 127) / 128) * ((column_rows + 63) / 64) < sm_count()) tensor = false;
+  if (mode == (int)DAB_CONTRACT_AUTO && ((lane_rows + 127) / 128) * ((column_rows + 63) / 64) * 3 < sm_count()) tensor = false;
   return tensor ? launch_gemm_mma(g, lanes_along_rows, stream) : launch_gemm(g, lanes_along_rows, stream);
 }
 
