@@ -3,7 +3,7 @@
 #include <atomic>
 #include <mutex>
 
-#include "common.cuh"
+#include "contraction.cuh"
 
 using namespace dab;
 
@@ -182,10 +182,10 @@ dab_status dab_sign_binarize(const float* d_values, int64_t rows, int32_t n, int
                                     static_cast<cudaStream_t>(stream)));
 }
 
-dab_status dab_binary_conv_contract(const dab_conv_desc* desc, const uint32_t* d_pmask, int32_t ldp,
-                                    const int32_t* d_pK, const float* d_pgamma, const float* d_pdelta,
-                                    const uint32_t* d_wmask, int32_t ldw, const int32_t* d_wK, const float* d_walpha,
-                                    const float* d_wbeta, float* d_y, int32_t* d_p11, void* stream) {
+static dab_status conv_contract(const dab_conv_desc* desc, const uint32_t* d_pmask, int32_t ldp, const int32_t* d_pK,
+                                const float* d_pgamma, const float* d_pdelta, const uint32_t* d_wmask, int32_t ldw,
+                                const int32_t* d_wK, const float* d_walpha, const float* d_wbeta, float* d_y, int32_t* d_p11,
+                                const PostOps& post, void* stream) {
   ConvGeom g;
   if (!conv_geom(desc, &g)) return DAB_ERR_INVALID_ARG;
   if (!d_pmask || !d_pK || !d_pgamma || !d_pdelta || !d_wmask || !d_wK || !d_walpha || !d_wbeta || !d_y)
@@ -203,14 +203,23 @@ dab_status dab_binary_conv_contract(const dab_conv_desc* desc, const uint32_t* d
   a.map.inner = HoWo; a.map.outer_stride = (int64_t)desc->Cout * HoWo; a.map.row_stride = 1; a.map.col_stride = HoWo;
   a.c_extent = (int64_t)desc->N * desc->Cout * HoWo;
   a.p11 = d_p11; a.ldp = desc->Cout;
+  a.post = post;
   return from_cuda(contract(a, /*lanes_along_rows=*/true, static_cast<cudaStream_t>(stream)));
+}
+
+dab_status dab_binary_conv_contract(const dab_conv_desc* desc, const uint32_t* d_pmask, int32_t ldp,
+                                    const int32_t* d_pK, const float* d_pgamma, const float* d_pdelta,
+                                    const uint32_t* d_wmask, int32_t ldw, const int32_t* d_wK, const float* d_walpha,
+                                    const float* d_wbeta, float* d_y, int32_t* d_p11, void* stream) {
+  return conv_contract(desc, d_pmask, ldp, d_pK, d_pgamma, d_pdelta, d_wmask, ldw, d_wK, d_walpha, d_wbeta, d_y, d_p11, PostOps(),
+                       stream);
 }
 
 static dab_status conv_with_coder(bool sign, const dab_conv_desc* desc, const float* d_x, const uint32_t* d_wmask, int32_t ldw,
                            const int32_t* d_wK, const float* d_walpha, const float* d_wbeta, float* d_y,
                            void* d_workspace, size_t workspace_bytes, int32_t* d_pK, float* d_pgamma,
                            float* d_pdelta, uint32_t* d_pmask, int32_t ldp, uint32_t* d_pflags, int32_t* d_p11,
-                           void* stream) {
+                           const PostOps& post, void* stream) {
   if (!desc) return DAB_ERR_INVALID_ARG;
   if (desc->C > 0 && desc->kh > 0 && desc->kw > 0 && (int64_t)desc->C * desc->kh * desc->kw > DAB_MAX_N)
     return DAB_ERR_UNSUPPORTED;
@@ -229,7 +238,7 @@ static dab_status conv_with_coder(bool sign, const dab_conv_desc* desc, const fl
   int32_t ldm = d_pmask ? ldp : g.ld;
   dab_status s = code_patches(sign, desc, d_x, pK, pg, pd, pm, ldm, d_pflags, stream);
   if (s != DAB_OK) return s;
-  return dab_binary_conv_contract(desc, pm, ldm, pK, pg, pd, d_wmask, ldw, d_wK, d_walpha, d_wbeta, d_y, d_p11, stream);
+  return conv_contract(desc, pm, ldm, pK, pg, pd, d_wmask, ldw, d_wK, d_walpha, d_wbeta, d_y, d_p11, post, stream);
 }
 
 dab_status dab_binary_conv(const dab_conv_desc* desc, const float* d_x, const uint32_t* d_wmask, int32_t ldw,
@@ -238,7 +247,7 @@ dab_status dab_binary_conv(const dab_conv_desc* desc, const float* d_x, const ui
                            float* d_pdelta, uint32_t* d_pmask, int32_t ldp, uint32_t* d_pflags, int32_t* d_p11,
                            void* stream) {
   return conv_with_coder(false, desc, d_x, d_wmask, ldw, d_wK, d_walpha, d_wbeta, d_y, d_workspace, workspace_bytes,
-                         d_pK, d_pgamma, d_pdelta, d_pmask, ldp, d_pflags, d_p11, stream);
+                         d_pK, d_pgamma, d_pdelta, d_pmask, ldp, d_pflags, d_p11, PostOps(), stream);
 }
 
 dab_status dab_binary_conv_sign(const dab_conv_desc* desc, const float* d_x, const uint32_t* d_wmask, int32_t ldw,
@@ -247,7 +256,7 @@ dab_status dab_binary_conv_sign(const dab_conv_desc* desc, const float* d_x, con
                                 float* d_pdelta, uint32_t* d_pmask, int32_t ldp, uint32_t* d_pflags, int32_t* d_p11,
                                 void* stream) {
   return conv_with_coder(true, desc, d_x, d_wmask, ldw, d_wK, d_walpha, d_wbeta, d_y, d_workspace, workspace_bytes,
-                         d_pK, d_pgamma, d_pdelta, d_pmask, ldp, d_pflags, d_p11, stream);
+                         d_pK, d_pgamma, d_pdelta, d_pmask, ldp, d_pflags, d_p11, PostOps(), stream);
 }
 
 // ---------------------------------------------------------------------------------------------------------
@@ -520,3 +529,12 @@ dab_status dab_binarize_backward(const float* d_Wc, int64_t rows, int32_t n, int
 
 
 }  // extern "C"
+
+namespace dab {
+dab_status binary_conv(const dab_conv_desc* desc, const float* d_x, const uint32_t* d_wmask, int32_t ldw, const int32_t* d_wK,
+                       const float* d_walpha, const float* d_wbeta, float* d_y, void* d_workspace, size_t workspace_bytes,
+                       const PostOps& post, void* stream) {
+  return conv_with_coder(false, desc, d_x, d_wmask, ldw, d_wK, d_walpha, d_wbeta, d_y, d_workspace, workspace_bytes, nullptr,
+                         nullptr, nullptr, nullptr, 0, nullptr, nullptr, post, stream);
+}
+}  // namespace dab

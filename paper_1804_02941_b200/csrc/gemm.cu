@@ -9,7 +9,7 @@
 
 #include <algorithm>
 
-#include "common.cuh"
+#include "contraction.cuh"
 
 namespace dab {
 
@@ -130,8 +130,9 @@ __global__ void __launch_bounds__(GEMM_THREADS) binary_gemm_kernel(const GemmArg
       if (gi >= g.M || gj >= g.N) continue;
       const int64_t to = (gi / g.map.inner) * g.map.outer_stride + (gi % g.map.inner) * g.map.row_stride + gj * g.map.col_stride;
       if (DAB_IN_BOUNDS(to, g.c_extent))
-        g.C[to] = rescale(p11, g.KB[DAB_IDX(gj, g.N)], g.KA[DAB_IDX(gi, g.M)], g.n, (double)g.alpha[DAB_IDX(gj, g.N)],
-                          (double)g.beta[DAB_IDX(gj, g.N)], (double)g.gamma[DAB_IDX(gi, g.M)], (double)g.delta[DAB_IDX(gi, g.M)]);
+        g.C[to] = apply_post(g.post, rescale(p11, g.KB[DAB_IDX(gj, g.N)], g.KA[DAB_IDX(gi, g.M)], g.n,
+                                             (double)g.alpha[DAB_IDX(gj, g.N)], (double)g.beta[DAB_IDX(gj, g.N)],
+                                             (double)g.gamma[DAB_IDX(gi, g.M)], (double)g.delta[DAB_IDX(gi, g.M)]), (int)gj, to);
       if (g.p11 && DAB_IN_BOUNDS(gi * g.ldp + gj, (g.M - 1) * g.ldp + g.N)) g.p11[gi * g.ldp + gj] = p11;
     }
     cluster.sync();  // a member's counts are read until here
@@ -161,7 +162,8 @@ __global__ void __launch_bounds__(GEMM_THREADS) binary_gemm_kernel(const GemmArg
       if (gj >= g.N) continue;
       int p11 = ones[i][j] + 2 * twos[i][j];
       if (DAB_IN_BOUNDS(base + gj * g.map.col_stride, g.c_extent))
-        g.C[base + gj * g.map.col_stride] = rescale(p11, Ke[j], Kf, g.n, al[j], be[j], gam, del);
+        g.C[base + gj * g.map.col_stride] =
+            apply_post(g.post, rescale(p11, Ke[j], Kf, g.n, al[j], be[j], gam, del), (int)gj, base + gj * g.map.col_stride);
       if (g.p11 && DAB_IN_BOUNDS(gi * g.ldp + gj, (g.M - 1) * g.ldp + g.N)) g.p11[gi * g.ldp + gj] = p11;
     }
   }

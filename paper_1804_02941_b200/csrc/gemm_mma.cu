@@ -12,7 +12,7 @@
 // word is 32 K bytes = two K chunks = the K extent of one kind::i8 instruction.
 #include <algorithm>
 
-#include "common.cuh"
+#include "contraction.cuh"
 #include "tc.cuh"
 
 namespace dab {
@@ -56,7 +56,7 @@ struct __align__(16) ColumnParams {
 // kLanesAreActivations: the rows that ride the 128 lanes of tensor memory (and the threads of the epilogue)
 // are activation rows, the columns weight rows: coalesced stores when the output is contiguous along the
 // activation rows (NCHW).  Otherwise the roles are exchanged: coalesced for a row-major M x N output.
-template <int THREADS, int KQ, int MIN_CTAS, int NT_MAX, bool kLanesAreActivations>
+template <int THREADS, int KQ, int MIN_CTAS, int NT_MAX, bool kLanesAreActivations, bool kPost>
 __global__ void __launch_bounds__(THREADS, MIN_CTAS) binary_gemm_mma_kernel(const GemmArgs g, const int tile_cols) {
   constexpr int KC = 8 * KQ;            // 16-byte K chunks per stage (two per mask word)
   constexpr uint32_t SBO = KC * 128;    // bytes between groups of 8 rows
@@ -222,8 +222,28 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS) binary_gemm_mma_kernel(cons
           y = __dadd_rn(y, __dmul_rn(__dmul_rn(l0, cp.v1), pc));
         }
         y = __dadd_rn(y, __dmul_rn(__dmul_rn(cp.v0, l0), p00));
-        if (DAB_IN_BOUNDS(off + cp.off, g.c_extent)) crow[cp.off] = (float)y;
+        const bool stored = DAB_IN_BOUNDS(off + cp.off, g.c_extent);
+        if (stored && !kPost) crow[cp.off] = (float)y;
         if (want_p11 && DAB_IN_BOUNDS(pblock + jj * pstep, (g.M - 1) * g.ldp + g.N)) g.p11[pblock + jj * pstep] = (int)v[jj];
+        if (kPost) v[jj] = __float_as_uint((float)y);
+      }
+      if (kPost) {  // the layers behind a convolution, one after another over the 32 columns
+        const int64_t step = g.map.col_stride;
+        const int j_first = (int)j0 + cb * 32;
+        const int64_t at = off + j_first * step;
+        for (int k = 0; k < g.post.count; ++k) {
+          const PostOp o = g.post.op[k];
+#pragma unroll
+          for (int jj = 0; jj < 32; ++jj) {
+            if (jj >= left) break;
+            v[jj] = __float_as_uint(apply_post_op(o, __uint_as_float(v[jj]), j_first + jj, at + jj * step));
+          }
+        }
+#pragma unroll
+        for (int jj = 0; jj < 32; ++jj) {
+          if (jj >= left) break;
+          if (DAB_IN_BOUNDS(at + jj * step, g.c_extent)) g.C[at + jj * step] = __uint_as_float(v[jj]);
+        }
       }
     }
   }
@@ -237,16 +257,16 @@ inline size_t dynamic_bytes(int kq, int ncap) {
   return (size_t)(MMA_M + ncap) * (8 * kq) * 16 + (size_t)ncap * sizeof(ColumnParams) + 128;
 }
 
-template <int THREADS, int KQ, int MIN_CTAS, int NT_MAX, bool kLanesAreActivations>
+template <int THREADS, int KQ, int MIN_CTAS, int NT_MAX, bool kLanesAreActivations, bool kPost>
 cudaError_t launch_shape(const GemmArgs& args, dim3 grid, int tile_cols, int ncap, cudaStream_t stream) {
-  auto kernel = binary_gemm_mma_kernel<THREADS, KQ, MIN_CTAS, NT_MAX, kLanesAreActivations>;
+  auto kernel = binary_gemm_mma_kernel<THREADS, KQ, MIN_CTAS, NT_MAX, kLanesAreActivations, kPost>;
   cudaError_t e = ensure_dynamic_smem(kernel, dynamic_bytes(KQ, NT_MAX));
   if (e != cudaSuccess) return e;
   kernel<<<grid, THREADS, dynamic_bytes(KQ, ncap), stream>>>(args, tile_cols);
   return cudaGetLastError();
 }
 
-template <bool kLanesAreActivations>
+template <bool kLanesAreActivations, bool kPost>
 cudaError_t launch_side(const GemmArgs& args, cudaStream_t stream) {
   const int64_t lane_rows = kLanesAreActivations ? args.M : args.N, col_rows = kLanesAreActivations ? args.N : args.M;
   // Column tile: the full 256 columns of an accumulator unless that leaves most SMs without a CTA.
@@ -260,18 +280,19 @@ cudaError_t launch_side(const GemmArgs& args, cudaStream_t stream) {
   // CTA shape by tile width, from timings of the four layer shapes of the ResNet-18-like stack: narrow tiles
   // run best as many small CTAs (six of 128 threads per SM), wider ones as fewer CTAs of 256 threads with
   // longer stages (two per SM at the full 256 columns, where shared memory is the limit).
-  if (ncap <= 64) return launch_shape<128, 1, 6, 64, kLanesAreActivations>(args, grid, tile_cols, ncap, stream);
+  if (ncap <= 64) return launch_shape<128, 1, 6, 64, kLanesAreActivations, kPost>(args, grid, tile_cols, ncap, stream);
   if (ncap <= 128 && args.words >= 64)  // long rows: eight words per stage halve the dependent stage rounds
-    return launch_shape<256, 2, 3, 128, kLanesAreActivations>(args, grid, tile_cols, ncap, stream);
-  if (ncap <= 128) return launch_shape<256, 1, 4, 128, kLanesAreActivations>(args, grid, tile_cols, ncap, stream);
-  return launch_shape<256, 2, 2, MMA_NMAX, kLanesAreActivations>(args, grid, tile_cols, ncap, stream);
+    return launch_shape<256, 2, 3, 128, kLanesAreActivations, kPost>(args, grid, tile_cols, ncap, stream);
+  if (ncap <= 128) return launch_shape<256, 1, 4, 128, kLanesAreActivations, kPost>(args, grid, tile_cols, ncap, stream);
+  return launch_shape<256, 2, 2, MMA_NMAX, kLanesAreActivations, kPost>(args, grid, tile_cols, ncap, stream);
 }
 
 }  // namespace
 
 cudaError_t launch_gemm_mma(const GemmArgs& args, bool lanes_along_rows, cudaStream_t stream) {
   if (args.words < 1 || args.M < 1 || args.N < 1) return cudaErrorInvalidValue;
-  return lanes_along_rows ? launch_side<true>(args, stream) : launch_side<false>(args, stream);
+  if (!lanes_along_rows) return launch_side<false, false>(args, stream);
+  return args.post.count > 0 ? launch_side<true, true>(args, stream) : launch_side<true, false>(args, stream);
 }
 
 cudaError_t read_mma_wait_timeouts(unsigned int* count) {

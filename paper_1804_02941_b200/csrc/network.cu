@@ -2,9 +2,11 @@
 // layer binarized): the full-precision layers around the binarized ones as small kernels of their own, and
 // dab_network_forward, which queues every layer of a chain on one stream without synchronising.
 //
-// The elementwise layers and pooling are the layer's plain definition, one thread per output.  The dense convolution sums its products in fp64 in element order (c, kh, kw), each product and sum
+// Elementwise layers (per-channel affine, ReLU, shortcuts and the copies that remember them) run in the kernel of the layer before
+// them, on its outputs; what has no such layer before it runs as one pass.  Pooling is its plain definition, one thread per
+// output.  The dense convolution sums its products in fp64 in element order (c, kh, kw), each product and sum
 // rounded on its own, and rounds once to fp32, so that its result does not depend on the launch shape.
-#include "common.cuh"
+#include "contraction.cuh"
 
 namespace dab {
 
@@ -36,7 +38,7 @@ struct __align__(16) DenseTap {
 template <int PX, int CO, int TAPS>
 __global__ void __launch_bounds__(256, 2) conv_dense_kernel(dab_conv_desc d, int Ho, int Wo, int co_tiles, const float* __restrict__ x,
                                                          const float* __restrict__ w, const float* __restrict__ bias,
-                                                         float* __restrict__ y) {
+                                                         float* __restrict__ y, const PostOps post) {
   constexpr int PT = 32 * PX, CT = 8 * CO;                 // positions and filters of a CTA
   constexpr int XL = TAPS * PT / 256;                // staged values per thread and chunk: positions ...
   constexpr int WL = (TAPS * CT + 255) / 256;        // ... and weights
@@ -147,15 +149,24 @@ __global__ void __launch_bounds__(256, 2) conv_dense_kernel(dab_conv_desc d, int
   for (int i = 0; i < PX; ++i) {
     const int64_t p = p0 + i * 32 + lane;
     if (p >= positions) continue;
-    float* const out = y + (p / HoWo) * d.Cout * HoWo + p % HoWo;
+    const int64_t at = (p / HoWo) * d.Cout * HoWo + p % HoWo;
+    const int first = co0 + warp * CO;
+    float out[CO];
 #pragma unroll
     for (int j = 0; j < CO; ++j) {
-      const int co = co0 + warp * CO + j;
-      if (co >= d.Cout) break;
       double v = acc[i][j];
-      if (bias) v = __dadd_rn(v, (double)__ldg(bias + co));
-      out[(int64_t)co * HoWo] = (float)v;
+      if (bias && first + j < d.Cout) v = __dadd_rn(v, (double)__ldg(bias + first + j));
+      out[j] = (float)v;
     }
+    for (int k = 0; k < post.count; ++k) {
+      const PostOp o = post.op[k];
+#pragma unroll
+      for (int j = 0; j < CO; ++j)
+        if (first + j < d.Cout) out[j] = apply_post_op(o, out[j], first + j, at + (first + j) * HoWo);
+    }
+#pragma unroll
+    for (int j = 0; j < CO; ++j)
+      if (first + j < d.Cout) y[at + (first + j) * HoWo] = out[j];
   }
 }
 
@@ -163,7 +174,7 @@ __global__ void __launch_bounds__(256, 2) conv_dense_kernel(dab_conv_desc d, int
 // (batch 1, fully connected layers, where a chain of n dependent additions is what counts) 32 positions x 16 filters in
 // chunks of 64 taps, one memory latency each.
 cudaError_t launch_conv_dense(const dab_conv_desc& d, int Ho, int Wo, const float* x, const float* w, const float* bias, float* y,
-                              cudaStream_t stream) {
+                              const PostOps& post, cudaStream_t stream) {
   const int64_t positions = (int64_t)d.N * Ho * Wo;
   const bool large = ((positions + 127) / 128) * ((d.Cout + 63) / 64) >= sm_count();
   const bool by48 = (d.Cout + 47) / 48 * 48 < (d.Cout + 63) / 64 * 64;
@@ -171,36 +182,61 @@ cudaError_t launch_conv_dense(const dab_conv_desc& d, int Ho, int Wo, const floa
   const int co_tiles = (d.Cout + ct - 1) / ct;
   const int64_t blocks = (positions + pt - 1) / pt * co_tiles;
   if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
-  if (!large) conv_dense_kernel<1, 2, 64><<<(unsigned)blocks, 256, 0, stream>>>(d, Ho, Wo, co_tiles, x, w, bias, y);
-  else if (by48) conv_dense_kernel<4, 6, 16><<<(unsigned)blocks, 256, 0, stream>>>(d, Ho, Wo, co_tiles, x, w, bias, y);
-  else conv_dense_kernel<4, 8, 16><<<(unsigned)blocks, 256, 0, stream>>>(d, Ho, Wo, co_tiles, x, w, bias, y);
+  if (!large) conv_dense_kernel<1, 2, 64><<<(unsigned)blocks, 256, 0, stream>>>(d, Ho, Wo, co_tiles, x, w, bias, y, post);
+  else if (by48) conv_dense_kernel<4, 6, 16><<<(unsigned)blocks, 256, 0, stream>>>(d, Ho, Wo, co_tiles, x, w, bias, y, post);
+  else conv_dense_kernel<4, 8, 16><<<(unsigned)blocks, 256, 0, stream>>>(d, Ho, Wo, co_tiles, x, w, bias, y, post);
   return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(kGlueThreads) affine_kernel(const float* __restrict__ x, int64_t total, int C, int64_t HW,
-                                                              const float* __restrict__ scale, const float* __restrict__ shift,
-                                                              float* __restrict__ y) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)((i / HW) % C);
-    y[i] = (float)__dadd_rn(__dmul_rn((double)__ldg(scale + c), (double)x[i]), (double)__ldg(shift + c));
+// Elementwise layers with no layer before them that could take them along: one pass, four elements a thread (VEC) where the
+// planes and pointers allow.  magic: ceil(2^32 / units of a plane), 0 where a 32-bit quotient would not be exact.
+template <int VEC>
+__global__ void __launch_bounds__(kGlueThreads) glue_kernel(const float* __restrict__ x, int64_t units, int C, int64_t plane_units,
+                                                            uint32_t magic, const PostOps post, float* __restrict__ y) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < units; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t plane = magic ? (int64_t)__umulhi((unsigned)i, magic) : i / plane_units;
+    const int channel = magic ? (int)((unsigned)plane % (unsigned)C) : (int)(plane % C);
+    float v[VEC];
+    if (VEC == 4) {
+      const float4 f = *reinterpret_cast<const float4*>(x + 4 * i);
+      v[0] = f.x; v[VEC > 1 ? 1 : 0] = f.y; v[VEC > 2 ? 2 : 0] = f.z; v[VEC > 3 ? 3 : 0] = f.w;
+    } else {
+      v[0] = x[i];
+    }
+    for (int k = 0; k < post.count; ++k) {
+      const PostOp o = post.op[k];
+      if (VEC == 4 && o.kind == kPostStore) {
+        *reinterpret_cast<float4*>(o.to + 4 * i) = make_float4(v[0], v[VEC > 1 ? 1 : 0], v[VEC > 2 ? 2 : 0], v[VEC > 3 ? 3 : 0]);
+      } else if (VEC == 4 && o.kind == kPostAdd) {
+        const float4 f = *reinterpret_cast<const float4*>(o.a + 4 * i);
+        const float w[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) v[j] = __fadd_rn(v[j], w[j]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) v[j] = apply_post_op(o, v[j], channel, VEC * i + j);
+      }
+    }
+    if (VEC == 4) *reinterpret_cast<float4*>(y + 4 * i) = make_float4(v[0], v[VEC > 1 ? 1 : 0], v[VEC > 2 ? 2 : 0], v[VEC > 3 ? 3 : 0]);
+    else y[i] = v[0];
   }
 }
 
-__global__ void __launch_bounds__(kGlueThreads) relu_kernel(const float* __restrict__ x, int64_t total, float* __restrict__ y) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const float v = x[i];
-    y[i] = v > 0.0f ? v : 0.0f;
-  }
-}
-
-__global__ void __launch_bounds__(kGlueThreads) add_kernel(const float* __restrict__ a, const float* __restrict__ b, int64_t total,
-                                                           float* __restrict__ y) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x)
-    y[i] = __fadd_rn(a[i], b[i]);
+cudaError_t launch_glue(const float* x, int32_t N, int32_t C, int64_t plane, const PostOps& post, float* y, cudaStream_t stream) {
+  uintptr_t bits = reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y);
+  for (int k = 0; k < post.count; ++k)
+    bits |= post.op[k].kind == kPostAdd ? reinterpret_cast<uintptr_t>(post.op[k].a) : reinterpret_cast<uintptr_t>(post.op[k].to);
+  const int vec = plane % 4 == 0 && (bits & 15) == 0 ? 4 : 1;
+  const int64_t per_plane = plane / vec, units = (int64_t)N * C * per_plane;
+  // floor(i / d) = umulhi(i, ceil(2^32 / d)) for i * d < 2^32
+  const uint32_t magic = per_plane > 1 && units * per_plane < 0x100000000ll ? (uint32_t)((0x100000000ull + per_plane - 1) / per_plane) : 0u;
+  if (vec == 4) glue_kernel<4><<<glue_blocks(units), kGlueThreads, 0, stream>>>(x, units, C, per_plane, magic, post, y);
+  else glue_kernel<1><<<glue_blocks(units), kGlueThreads, 0, stream>>>(x, units, C, per_plane, magic, post, y);
+  return cudaGetLastError();
 }
 
 __global__ void __launch_bounds__(kGlueThreads) maxpool_kernel(dab_conv_desc d, int Ho, int Wo, const float* __restrict__ x,
-                                                               float* __restrict__ y) {
+                                                               const PostOps post, float* __restrict__ y) {
   const int64_t outputs = (int64_t)d.N * d.C * Ho * Wo;
   for (int64_t oi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; oi < outputs; oi += (int64_t)gridDim.x * blockDim.x) {
     const int wo = (int)(oi % Wo);
@@ -218,6 +254,7 @@ __global__ void __launch_bounds__(kGlueThreads) maxpool_kernel(dab_conv_desc d, 
           seen = true;
         }
       }
+    if (post.count > 0) best = apply_post(post, best, (int)(plane % d.C), oi);
     y[oi] = best;
   }
 }
@@ -341,68 +378,83 @@ dab_status dab_network_forward(const dab_layer* layers, int32_t count, int32_t N
   const float* saved = nullptr;
   int cur_next = 0, saved_next = 2;
   Shape cs_shape{C, H, W}, sv_shape{0, 0, 0};
-  for (int32_t i = 0; i < count; ++i) {
+  auto kept = [&](int32_t i) { return h_layer_outputs ? h_layer_outputs[i] : nullptr; };  // the caller wants this layer's output
+  auto to_saved = [&]() {
+    float* const slot = pool[saved_next];
+    saved_next = saved_next == 2 ? 3 : 2;
+    return slot;
+  };
+  for (int32_t i = 0; i < count;) {
     const dab_layer& L = layers[i];
-    float* keep = h_layer_outputs ? h_layer_outputs[i] : nullptr;  // the caller wants this layer's output
-    if (L.kind == DAB_LAYER_SAVE) {
-      // the remembered tensor is a copy (the running buffers are overwritten two layers on); the running tensor stays
-      float* slot = pool[saved_next];
-      saved_next = saved_next == 2 ? 3 : 2;
-      const size_t bytes = (size_t)cs_shape.count(N) * sizeof(float);
-      if (cudaMemcpyAsync(slot, cur, bytes, cudaMemcpyDeviceToDevice, cs) != cudaSuccess) return DAB_ERR_CUDA;
-      if (keep && cudaMemcpyAsync(keep, cur, bytes, cudaMemcpyDeviceToDevice, cs) != cudaSuccess) return DAB_ERR_CUDA;
-      saved = slot;
-      sv_shape = cs_shape;
-      continue;
-    }
-    Shape& shp = L.on_saved ? sv_shape : cs_shape;
-    const float* src = L.on_saved ? saved : cur;
-    float* dst;
-    if (keep) dst = keep;
-    else if (L.on_saved) { dst = pool[saved_next]; saved_next = saved_next == 2 ? 3 : 2; }
-    else if (i == count - 1) dst = d_y;
-    else { dst = pool[cur_next]; cur_next ^= 1; }
+    const bool on_saved = L.on_saved != 0;
+    Shape& shp = on_saved ? sv_shape : cs_shape;
+    const float* const src = on_saved ? saved : cur;
+    const bool own_kernel = L.kind == DAB_LAYER_CONV_DENSE || L.kind == DAB_LAYER_CONV_BINARY || L.kind == DAB_LAYER_MAXPOOL;
     dab_conv_desc d;
     Shape out = shp;
+    if (own_kernel) layer_desc(L, N, shp, &d, &out);
+    // the elementwise layers that follow on the same tensor (or that begin here), as far as they fit
+    PostOps post;
+    auto add = [&](int32_t kind, const float* a, const float* b, float* to) { post.op[post.count++] = PostOp{kind, a, b, to}; };
+    int32_t last = own_kernel ? i : i - 1;
+    while (last + 1 < count && post.count + 3 <= kMaxPostOps) {
+      const dab_layer& E = layers[last + 1];
+      if ((E.on_saved != 0) != on_saved || E.kind < DAB_LAYER_AFFINE || E.kind == DAB_LAYER_MAXPOOL) break;
+      // (a SAVE's kept output is stored with it)
+      if (last >= i && layers[last].kind != DAB_LAYER_SAVE && kept(last)) add(kPostStore, nullptr, nullptr, kept(last));
+      ++last;
+      if (E.kind == DAB_LAYER_AFFINE) add(kPostAffine, E.d_scale, E.d_shift, nullptr);
+      else if (E.kind == DAB_LAYER_RELU) add(kPostRelu, nullptr, nullptr, nullptr);
+      else if (E.kind == DAB_LAYER_ADD) add(kPostAdd, saved, nullptr, nullptr);
+      else {
+        // the remembered tensor is a copy (the running buffers are overwritten two layers on)
+        float* const slot = to_saved();
+        add(kPostStore, nullptr, nullptr, slot);
+        saved = slot;
+        sv_shape = out;
+        if (kept(last)) break;
+      }
+    }
+    const bool ends_saved = layers[last].kind == DAB_LAYER_SAVE;
+    if (ends_saved && kept(last)) add(kPostStore, nullptr, nullptr, kept(last));
     cudaError_t e = cudaSuccess;
-    switch (L.kind) {
+    bool copies = !own_kernel;  // nothing but a SAVE: the running tensor stays where it is
+    for (int32_t k = 0; k < post.count; ++k) copies = copies && post.op[k].kind == kPostStore;
+    if (copies) {
+      const size_t bytes = (size_t)shp.count(N) * sizeof(float);
+      for (int32_t k = 0; k < post.count && e == cudaSuccess; ++k) e = cudaMemcpyAsync(post.op[k].to, src, bytes, cudaMemcpyDeviceToDevice, cs);
+      if (e != cudaSuccess) return DAB_ERR_CUDA;
+      i = last + 1;
+      continue;
+    }
+    float* dst;
+    if (!ends_saved && kept(last)) dst = kept(last);
+    else if (on_saved) dst = to_saved();
+    else if (last == count - 1) dst = d_y;
+    else { dst = pool[cur_next]; cur_next ^= 1; }
+    switch (own_kernel ? L.kind : DAB_LAYER_RELU) {
       case DAB_LAYER_CONV_DENSE:
-        layer_desc(L, N, shp, &d, &out);
-        e = launch_conv_dense(d, out.H, out.W, src, L.d_weights, L.d_bias, dst, cs);
+        e = launch_conv_dense(d, out.H, out.W, src, L.d_weights, L.d_bias, dst, post, cs);
         break;
       case DAB_LAYER_CONV_BINARY: {
-        layer_desc(L, N, shp, &d, &out);
-        dab_status s = dab_binary_conv(&d, src, L.d_wmask, L.ldw, L.d_wK, L.d_walpha, L.d_wbeta, dst, scratch,
-                                       round_up(plan.conv_scratch, kAlign), nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr,
-                                       stream);
+        const dab_status s = binary_conv(&d, src, L.d_wmask, L.ldw, L.d_wK, L.d_walpha, L.d_wbeta, dst, scratch,
+                                         round_up(plan.conv_scratch, kAlign), post, stream);
         if (s != DAB_OK) return s;
         break;
       }
-      case DAB_LAYER_AFFINE:
-        affine_kernel<<<glue_blocks(shp.count(N)), kGlueThreads, 0, cs>>>(src, shp.count(N), shp.C, (int64_t)shp.H * shp.W, L.d_scale,
-                                                                          L.d_shift, dst);
-        e = cudaGetLastError();
-        break;
-      case DAB_LAYER_RELU:
-        relu_kernel<<<glue_blocks(shp.count(N)), kGlueThreads, 0, cs>>>(src, shp.count(N), dst);
-        e = cudaGetLastError();
-        break;
       case DAB_LAYER_MAXPOOL:
-        layer_desc(L, N, shp, &d, &out);
-        maxpool_kernel<<<glue_blocks(out.count(N)), kGlueThreads, 0, cs>>>(d, out.H, out.W, src, dst);
-        e = cudaGetLastError();
-        break;
-      case DAB_LAYER_ADD:
-        add_kernel<<<glue_blocks(shp.count(N)), kGlueThreads, 0, cs>>>(cur, saved, shp.count(N), dst);
+        maxpool_kernel<<<glue_blocks(out.count(N)), kGlueThreads, 0, cs>>>(d, out.H, out.W, src, post, dst);
         e = cudaGetLastError();
         break;
       default:
-        return DAB_ERR_INVALID_ARG;
+        e = launch_glue(src, N, out.C, (int64_t)out.H * out.W, post, dst, cs);
+        break;
     }
     if (e != cudaSuccess) return DAB_ERR_CUDA;
     shp = out;
-    if (L.on_saved) saved = dst;
+    if (on_saved) saved = dst;
     else cur = dst;
+    i = last + 1;
   }
   if (cur != d_y &&
       cudaMemcpyAsync(d_y, cur, (size_t)cs_shape.count(N) * sizeof(float), cudaMemcpyDeviceToDevice, cs) != cudaSuccess)

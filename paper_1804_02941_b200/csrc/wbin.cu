@@ -24,7 +24,6 @@
 #include <climits>
 
 #include "common.cuh"
-#include "rowcode.cuh"
 #include "tc.cuh"
 
 namespace dab {
@@ -104,11 +103,6 @@ __device__ __forceinline__ void gather_chunk(const unsigned char* src, const int
 #pragma unroll
   for (int p = 0; p < 4; ++p)
     *reinterpret_cast<uint4*>(dst + p * kPlane) = make_uint4(pl[p][0], pl[p][1], pl[p][2], pl[p][3]);
-}
-
-// Exact for |v| < 2^31, without the conversion unit.
-__device__ __forceinline__ double signed_to_double(int v) {
-  return __dsub_rn(__hiloint2double(0x43300000, (int)((uint32_t)v ^ 0x80000000u)), 4503601774854144.0);  // 2^52 + 2^31
 }
 
 // Bytes of shared memory for the operands of one stage.
@@ -383,8 +377,8 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
         if (bad) {
           out = __uint_as_float(0x7FC00000u);
         } else {
-          const double hi = signed_to_double(-((int)v[3][jj] * 256 + (int)v[2][jj]));
-          const double lo = signed_to_double(-((int)v[1][jj] * 256 + (int)v[0][jj]));
+          const double hi = int_to_double(-((int)v[3][jj] * 256 + (int)v[2][jj]));
+          const double lo = int_to_double(-((int)v[1][jj] * 256 + (int)v[0][jj]));
           const double m1 = __fma_rn(hi, 65536.0, lo), m0 = Sd - m1;  // exact: |.| < 2^45
           const double y = __dadd_rn(__dmul_rn(s_alpha[j], m1), __dmul_rn(s_beta[j], m0));
           out = (float)__dmul_rn(y, inv);
