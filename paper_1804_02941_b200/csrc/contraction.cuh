@@ -40,14 +40,27 @@ __device__ __forceinline__ float apply_post(const PostOps& ops, float v, int cha
   return v;
 }
 
-// Four-term rescale in fp64, one rounding to fp32.  Term order is part of the contract.
-__device__ __forceinline__ float rescale(int p11, int Ke, int Kf, int n, double a, double b, double g, double d) {
-  int p10 = Ke - p11, p01 = Kf - p11, p00 = n - Ke - Kf + p11;
-  double y = __dmul_rn(__dmul_rn(a, g), int_to_double(p11));
-  y = __dadd_rn(y, __dmul_rn(__dmul_rn(a, d), int_to_double(p10)));
-  y = __dadd_rn(y, __dmul_rn(__dmul_rn(b, g), int_to_double(p01)));
-  y = __dadd_rn(y, __dmul_rn(__dmul_rn(b, d), int_to_double(p00)));
-  return (float)y;
+// The sum of the four terms alpha gamma p11 + alpha delta p10 + beta gamma p01 + beta delta p00 of the four counts
+// (p10 = Ke - p11, p01 = Kf - p11, p00 = n - Ke - Kf + p11) in fp64, one rounding to fp32, gathered by what depends on the pair:
+//   (gamma - delta) ((alpha - beta) p11 + beta Kf) + delta (alpha Ke + beta (n - Ke))
+// Five fp64 operations per output instead of the fifteen of the four terms, which kept the fp64 pipe busy longer than the
+// counting where rows are short.  A product of a value and a count is exact in fp64 and the fused additions round once, so what
+// is rounded on the way stays below 2^-50 of the terms, as before.  Every kernel that rescales does it in exactly these operations.
+struct RescaleSide {  // of a weight row: d = alpha - beta, b = beta, c = alpha Ke + beta (n - Ke); of an activation row: d = gamma -
+  double d, b, c;     // delta, b = Kf, c = delta
+};
+__device__ __forceinline__ RescaleSide rescale_weight(double alpha, double beta, int Ke, int n) {
+  return {__dsub_rn(alpha, beta), beta, __dadd_rn(__dmul_rn(alpha, int_to_double(Ke)), __dmul_rn(beta, int_to_double(n - Ke)))};
+}
+__device__ __forceinline__ RescaleSide rescale_activation(double gamma, double delta, int Kf) {
+  return {__dsub_rn(gamma, delta), int_to_double(Kf), delta};
+}
+__device__ __forceinline__ float rescale(int p11, double wd, double wb, double wc, double ad, double ab, double ac) {
+  const double t = __fma_rn(wd, int_to_double(p11), __dmul_rn(wb, ab));
+  return (float)__fma_rn(ad, t, __dmul_rn(ac, wc));
+}
+__device__ __forceinline__ float rescale(int p11, const RescaleSide& w, const RescaleSide& a) {
+  return rescale(p11, w.d, w.b, w.c, a.d, a.b, a.c);
 }
 
 // Where an output element (row i of the activation side, column j of the weight side) is stored:

@@ -101,6 +101,12 @@ __global__ void __launch_bounds__(GEMM_THREADS) binary_gemm_kernel(const GemmArg
     __syncthreads();
   }
 
+  auto weight = [&](int64_t gj) {
+    return rescale_weight((double)g.alpha[DAB_IDX(gj, g.N)], (double)g.beta[DAB_IDX(gj, g.N)], g.KB[DAB_IDX(gj, g.N)], g.n);
+  };
+  auto activation = [&](int64_t gi) {
+    return rescale_activation((double)g.gamma[DAB_IDX(gi, g.M)], (double)g.delta[DAB_IDX(gi, g.M)], g.KA[DAB_IDX(gi, g.M)]);
+  };
   if (kSplit) {
     // The counts meet in shared memory, [column][row] or [row][column] as the lanes of the stores run; a member finishes
     // every splits-th line of the tile.
@@ -130,31 +136,24 @@ __global__ void __launch_bounds__(GEMM_THREADS) binary_gemm_kernel(const GemmArg
       if (gi >= g.M || gj >= g.N) continue;
       const int64_t to = (gi / g.map.inner) * g.map.outer_stride + (gi % g.map.inner) * g.map.row_stride + gj * g.map.col_stride;
       if (DAB_IN_BOUNDS(to, g.c_extent))
-        g.C[to] = apply_post(g.post, rescale(p11, g.KB[DAB_IDX(gj, g.N)], g.KA[DAB_IDX(gi, g.M)], g.n,
-                                             (double)g.alpha[DAB_IDX(gj, g.N)], (double)g.beta[DAB_IDX(gj, g.N)],
-                                             (double)g.gamma[DAB_IDX(gi, g.M)], (double)g.delta[DAB_IDX(gi, g.M)]), (int)gj, to);
+        g.C[to] = apply_post(g.post, rescale(p11, weight(gj), activation(gi)), (int)gj, to);
       if (g.p11 && DAB_IN_BOUNDS(gi * g.ldp + gj, (g.M - 1) * g.ldp + g.N)) g.p11[gi * g.ldp + gj] = p11;
     }
     cluster.sync();  // a member's counts are read until here
     return;
   }
 
-  double al[TN], be[TN];
-  int Ke[TN];
+  RescaleSide side[TN];
 #pragma unroll
   for (int j = 0; j < TN; ++j) {
-    int64_t gj = j0 + b_t * TN + j;
-    const bool in = gj < g.N;
-    al[j] = in ? (double)g.alpha[DAB_IDX(gj, g.N)] : 0.0;
-    be[j] = in ? (double)g.beta[DAB_IDX(gj, g.N)] : 0.0;
-    Ke[j] = in ? g.KB[DAB_IDX(gj, g.N)] : 0;
+    const int64_t gj = j0 + b_t * TN + j;
+    side[j] = gj < g.N ? weight(gj) : RescaleSide{0.0, 0.0, 0.0};
   }
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
     int64_t gi = i0 + a_t * TM + i;
     if (gi >= g.M) continue;
-    int Kf = g.KA[DAB_IDX(gi, g.M)];
-    double gam = (double)g.gamma[DAB_IDX(gi, g.M)], del = (double)g.delta[DAB_IDX(gi, g.M)];
+    const RescaleSide act = activation(gi);
     int64_t base = (gi / g.map.inner) * g.map.outer_stride + (gi % g.map.inner) * g.map.row_stride;
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
@@ -163,7 +162,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) binary_gemm_kernel(const GemmArg
       int p11 = ones[i][j] + 2 * twos[i][j];
       if (DAB_IN_BOUNDS(base + gj * g.map.col_stride, g.c_extent))
         g.C[base + gj * g.map.col_stride] =
-            apply_post(g.post, rescale(p11, Ke[j], Kf, g.n, al[j], be[j], gam, del), (int)gj, base + gj * g.map.col_stride);
+            apply_post(g.post, rescale(p11, side[j], act), (int)gj, base + gj * g.map.col_stride);
       if (g.p11 && DAB_IN_BOUNDS(gi * g.ldp + gj, (g.M - 1) * g.ldp + g.N)) g.p11[gi * g.ldp + gj] = p11;
     }
   }

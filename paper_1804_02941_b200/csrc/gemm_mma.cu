@@ -2,8 +2,8 @@
 // coded rows).  popc(e AND f) over a row of n bits is the dot product of the two rows written as 0/1 bytes,
 // so each CTA expands mask words to bytes in shared memory and lets the fifth-generation tensor cores
 // (tcgen05.mma, kind::i8, 32-bit integer accumulators in tensor memory) form a 128 x NT block of exact integer
-// counts.  The bytes are 0 / -1 (signed operands on both sides: one byte permutation per four bits makes them,
-// and (-1) x (-1) = 1), in an order of the row's bits that is permuted within each word, alike on both sides.  The four-term rescale then runs on the counts as they are read
+// counts.  The bytes are single bits left where they stand in the mask word, mirrored on one side, so that an AND
+// makes four of them and every product of two set bits is 128.  The four-term rescale then runs on the counts as they are read
 // back from tensor memory, with the same arithmetic as the population-count kernel.
 //
 // Shared-memory operand layout (K-major, no swizzle): 8 rows x 16 bytes form one contiguous 128-byte core
@@ -34,15 +34,82 @@ struct Side {
   const float* v1;  // value of the set bits
   const float* v0;  // value of the clear bits
   int64_t rows;
+  bool weights;
+  __device__ __forceinline__ RescaleSide rescaled(int64_t row, int n) const {
+    const double a = (double)v1[DAB_IDX(row, rows)], b = (double)v0[DAB_IDX(row, rows)];
+    const int k = K[DAB_IDX(row, rows)];
+    return weights ? rescale_weight(a, b, k, n) : rescale_activation(a, b, k);
+  }
 };
 
-// What the epilogue needs of one column-side row: its two values, its popcount K and n - K as doubles, and
-// its part of the output offset.
+// What the epilogue needs of one column-side row: its part of the rescale and of the output offset.
 struct __align__(16) ColumnParams {
-  double v1, v0, K, nK;
+  RescaleSide r;
   int64_t off;
-  int64_t pad;
 };
+
+// Where activation row i and weight row j meet in the output: act_offset(i) + j * col_stride.
+__device__ __forceinline__ int64_t act_offset(const GemmArgs& g, int64_t i) {
+  return (i / g.map.inner) * g.map.outer_stride + (i % g.map.inner) * g.map.row_stride;
+}
+
+// Outputs of one lane-side row and up to 32 columns from column `first` (counted over the whole matrix) on.  v: their counts.
+template <bool kLanesAreActivations, bool kPost>
+__device__ __forceinline__ void store_columns(const GemmArgs& g, uint32_t (&v)[32], int left, const ColumnParams* col, int64_t first,
+                                              int64_t gl, const RescaleSide& lane_side, int64_t off) {
+  // this row's counts: element (gl, column) when the lanes are activation rows, (column, gl) otherwise
+  const int64_t pblock = kLanesAreActivations ? gl * g.ldp + first : first * g.ldp + gl;
+  const int64_t pstep = kLanesAreActivations ? 1 : g.ldp;
+#pragma unroll
+  for (int jj = 0; jj < 32; ++jj) v[jj] >>= kBitProductLog;
+  if (!kPost && left >= 32 && !g.p11) {  // the usual case
+    float* const row = g.C + off;
+#pragma unroll
+    for (int jj = 0; jj < 32; ++jj) {
+      const ColumnParams cp = col[jj];
+      const float y = kLanesAreActivations ? rescale((int)v[jj], cp.r, lane_side) : rescale((int)v[jj], lane_side, cp.r);
+      if (DAB_IN_BOUNDS(off + cp.off, g.c_extent)) row[cp.off] = y;
+    }
+    return;
+  }
+#pragma unroll
+  for (int jj = 0; jj < 32; ++jj) {
+    if (jj >= left) break;
+    const ColumnParams cp = col[jj];
+    const float y = kLanesAreActivations ? rescale((int)v[jj], cp.r, lane_side) : rescale((int)v[jj], lane_side, cp.r);
+    if (!kPost && DAB_IN_BOUNDS(off + cp.off, g.c_extent)) g.C[off + cp.off] = y;
+    if (g.p11 && DAB_IN_BOUNDS(pblock + jj * pstep, (g.M - 1) * g.ldp + g.N)) g.p11[pblock + jj * pstep] = (int)v[jj];
+    if (kPost) v[jj] = __float_as_uint(y);
+  }
+  if (kPost) {  // the layers behind a convolution, one after another over the 32 columns
+    const int64_t step = g.map.col_stride, at = off + first * step;
+    for (int k = 0; k < g.post.count; ++k) {
+      const PostOp o = g.post.op[k];
+#pragma unroll
+      for (int jj = 0; jj < 32; ++jj) {
+        if (jj >= left) break;
+        v[jj] = __float_as_uint(apply_post_op(o, __uint_as_float(v[jj]), (int)first + jj, at + jj * step));
+      }
+    }
+#pragma unroll
+    for (int jj = 0; jj < 32; ++jj) {
+      if (jj >= left) break;
+      if (DAB_IN_BOUNDS(at + jj * step, g.c_extent)) g.C[at + jj * step] = __uint_as_float(v[jj]);
+    }
+  }
+}
+
+template <bool kLanesAreActivations>
+__device__ __forceinline__ void both_sides(const GemmArgs& g, Side& L, Side& S) {
+  const Side act{g.A, g.lda, g.KA, g.gamma, g.delta, g.M, false}, wgt{g.B, g.ldb, g.KB, g.alpha, g.beta, g.N, true};
+  L = kLanesAreActivations ? act : wgt;  // lane side
+  S = kLanesAreActivations ? wgt : act;  // column side
+}
+
+template <bool kLanesAreActivations>
+__device__ __forceinline__ ColumnParams column_params(const GemmArgs& g, const Side& S, int64_t j) {
+  return {S.rescaled(j, g.n), kLanesAreActivations ? j * g.map.col_stride : act_offset(g, j)};
+}
 
 // The pieces one thread expands per stage: unit u covers row (u>>3)/KQ*8 + (u&7), 16-byte piece (u>>3)%KQ.
 // Eight consecutive lanes hold the eight rows of one core matrix, so their 16-byte stores are one
@@ -65,9 +132,8 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS) binary_gemm_mma_kernel(cons
   __shared__ __align__(8) uint64_t s_bar;
   __shared__ uint32_t s_tmem;
 
-  const Side act{g.A, g.lda, g.KA, g.gamma, g.delta, g.M}, wgt{g.B, g.ldb, g.KB, g.alpha, g.beta, g.N};
-  const Side L = kLanesAreActivations ? act : wgt;  // lane side
-  const Side S = kLanesAreActivations ? wgt : act;  // column side
+  Side L, S;
+  both_sides<kLanesAreActivations>(g, L, S);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t i0 = (int64_t)blockIdx.x * MMA_M;
@@ -94,26 +160,12 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS) binary_gemm_mma_kernel(cons
     mbar_init(bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // where activation row i and weight row j meet in the output: act_offset(i) + j * col_stride
-  auto act_offset = [&](int64_t i) {
-    return (i / g.map.inner) * g.map.outer_stride + (i % g.map.inner) * g.map.row_stride;
-  };
-  for (int j = tid; j < nrows; j += THREADS) {
-    ColumnParams cp;
-    const int K = S.K[DAB_IDX(j0 + j, S.rows)];
-    cp.v1 = (double)S.v1[DAB_IDX(j0 + j, S.rows)];
-    cp.v0 = (double)S.v0[DAB_IDX(j0 + j, S.rows)];
-    cp.K = (double)K;
-    cp.nK = (double)(g.n - K);
-    cp.off = kLanesAreActivations ? (j0 + j) * g.map.col_stride : act_offset(j0 + j);
-    cp.pad = 0;
-    s_col[j] = cp;
-  }
+  for (int j = tid; j < nrows; j += THREADS) s_col[j] = column_params<kLanesAreActivations>(g, S, j0 + j);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = s_tmem;
-  const uint32_t idesc = instr_desc(NT, true, true);  // both operands signed: bytes 0 / -1
+  const uint32_t idesc = instr_desc(NT);
 
   // units of this thread: lane-side pieces first, then column-side pieces
   const int l_units = MMA_M * KQ, units = l_units + NT * KQ;
@@ -161,7 +213,12 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS) binary_gemm_mma_kernel(cons
       if (c * 4 * KQ + 4 * piece >= g.words) continue;  // no instruction reads this part of the stage
       unsigned char* dst =
           stage + (isL ? 0u : a_bytes) + (uint32_t)group * SBO + (uint32_t)(8 * piece) * 128 + (v & 7) * 16;
-      expand_words_signed(q[t], dst);
+      const uint32_t w[4] = {q[t].x, q[t].y, q[t].z, q[t].w};
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        if (isL) expand_word_bits<false>(w[m], dst + 256 * m);
+        else expand_word_bits<true>(w[m], dst + 256 * m);
+      }
     }
     if (c + 1 < chunks) fetch(c + 1);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy stores -> tensor-core reads
@@ -183,74 +240,136 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS) binary_gemm_mma_kernel(cons
   {
     const int64_t gl = i0 + (warp & 3) * 32 + lane;
     const bool valid = gl < L.rows && !dead;
-    double Kl = 0.0, l1 = 0.0, l0 = 0.0;
+    RescaleSide lane_side{0.0, 0.0, 0.0};
     int64_t off = 0;
     if (valid) {
-      Kl = (double)L.K[DAB_IDX(gl, L.rows)];
-      l1 = (double)L.v1[DAB_IDX(gl, L.rows)];
-      l0 = (double)L.v0[DAB_IDX(gl, L.rows)];
-      off = kLanesAreActivations ? act_offset(gl) : gl * g.map.col_stride;
+      lane_side = L.rescaled(gl, g.n);
+      off = kLanesAreActivations ? act_offset(g, gl) : gl * g.map.col_stride;
     }
-    const bool want_p11 = g.p11 != nullptr;
-    float* const crow = g.C + off;
-    // this row's counts: element (gl, j0 + j) when the lanes are activation rows, (j0 + j, gl) otherwise
-    const int64_t p0 = kLanesAreActivations ? gl * g.ldp + j0 : j0 * g.ldp + gl;
-    const int64_t pstep = kLanesAreActivations ? 1 : g.ldp;
     for (int cb = warp >> 2; cb * 32 < NT; cb += THREADS / 128) {
       uint32_t v[32];
       tmem_load_32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(cb * 32), v);
-      if (!valid) continue;
-      const int left = nrows - cb * 32;  // columns of this block that exist
-      const ColumnParams* const col = s_col + cb * 32;
-      const int64_t pblock = p0 + (int64_t)(cb * 32) * pstep;
-#pragma unroll
-      for (int jj = 0; jj < 32; ++jj) {
-        if (jj >= left) break;
-        const ColumnParams cp = col[jj];
-        // The four counts as doubles (small integers: every difference is exact, so these are the values
-        // rescale() converts from int), then its four terms in its order: alpha gamma p11, alpha delta p10,
-        // beta gamma p01, beta delta p00, with p10 the count on the weight side only.
-        const double p11 = int_to_double((int)v[jj]);
-        const double pc = __dsub_rn(cp.K, p11), pl = __dsub_rn(Kl, p11);  // set on the column / lane side only
-        const double p00 = __dsub_rn(cp.nK, pl);
-        double y = __dmul_rn(__dmul_rn(cp.v1, l1), p11);
-        if (kLanesAreActivations) {
-          y = __dadd_rn(y, __dmul_rn(__dmul_rn(cp.v1, l0), pc));
-          y = __dadd_rn(y, __dmul_rn(__dmul_rn(cp.v0, l1), pl));
-        } else {
-          y = __dadd_rn(y, __dmul_rn(__dmul_rn(l1, cp.v0), pl));
-          y = __dadd_rn(y, __dmul_rn(__dmul_rn(l0, cp.v1), pc));
-        }
-        y = __dadd_rn(y, __dmul_rn(__dmul_rn(cp.v0, l0), p00));
-        const bool stored = DAB_IN_BOUNDS(off + cp.off, g.c_extent);
-        if (stored && !kPost) crow[cp.off] = (float)y;
-        if (want_p11 && DAB_IN_BOUNDS(pblock + jj * pstep, (g.M - 1) * g.ldp + g.N)) g.p11[pblock + jj * pstep] = (int)v[jj];
-        if (kPost) v[jj] = __float_as_uint((float)y);
-      }
-      if (kPost) {  // the layers behind a convolution, one after another over the 32 columns
-        const int64_t step = g.map.col_stride;
-        const int j_first = (int)j0 + cb * 32;
-        const int64_t at = off + j_first * step;
-        for (int k = 0; k < g.post.count; ++k) {
-          const PostOp o = g.post.op[k];
-#pragma unroll
-          for (int jj = 0; jj < 32; ++jj) {
-            if (jj >= left) break;
-            v[jj] = __float_as_uint(apply_post_op(o, __uint_as_float(v[jj]), j_first + jj, at + jj * step));
-          }
-        }
-#pragma unroll
-        for (int jj = 0; jj < 32; ++jj) {
-          if (jj >= left) break;
-          if (DAB_IN_BOUNDS(at + jj * step, g.c_extent)) g.C[at + jj * step] = __uint_as_float(v[jj]);
-        }
-      }
+      if (valid) store_columns<kLanesAreActivations, kPost>(g, v, nrows - cb * 32, s_col + cb * 32, j0 + cb * 32, gl, lane_side, off);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
+}
+
+// The form for long rows: 128 x 128 outputs per CTA, two CTAs per SM.  The lane side never passes through shared memory: every
+// thread writes four words of its row, expanded, into tensor memory, from where the tensor cores take their first operand.
+// What is left there is the column side, written and read once: in the kernel above 24 KB pass through shared memory per 32 bits
+// of 128 x 256 outputs, 192 cycles, where the products take 128; here it is 16 KB, 128 cycles.  Two stages of eight words, one
+// barrier each.  Bound by the load and shared-memory pipe (0.79 busy; tensor cores 0.46): a warp's load of 16 bytes per row takes it 32 cycles.
+// 8192 x 8192 x 4608 bits: 346 us in the kernel above, 287 here (369 with stages of four words and loads of 8 bytes; 310 with
+// the words staged in shared memory by 16-byte asynchronous copies, 418 by bulk copies of 64 bytes per row).
+constexpr int WIDE_THREADS = 256, WIDE_COLS = 128, WIDE_WORDS = 8, WIDE_BUFFERS = 2;
+constexpr uint32_t WIDE_SBO = 2 * WIDE_WORDS * 128, WIDE_STAGE = WIDE_COLS * WIDE_WORDS * 32;  // bytes
+constexpr uint32_t WIDE_ACOLS = WIDE_WORDS * 8;            // columns of a lane-side stage: 4 bytes each; behind the accumulator
+constexpr uint32_t WIDE_TMEM = WIDE_COLS + WIDE_BUFFERS * WIDE_ACOLS;
+static_assert(WIDE_TMEM == 256, "two CTAs share the 512 columns");
+constexpr size_t WIDE_BYTES = WIDE_BUFFERS * WIDE_STAGE + WIDE_COLS * sizeof(ColumnParams) + 128;
+
+template <bool kLanesAreActivations, bool kPost>
+__global__ void __launch_bounds__(WIDE_THREADS, 2) binary_gemm_wide_kernel(const GemmArgs g) {
+  extern __shared__ __align__(128) unsigned char dyn_mem[];  // [two column-side stages][ColumnParams]
+  __shared__ __align__(8) uint64_t s_bar[WIDE_BUFFERS];
+  __shared__ uint32_t s_tmem;
+  Side L, S;
+  both_sides<kLanesAreActivations>(g, L, S);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t i0 = (int64_t)blockIdx.x * MMA_M, j0 = (int64_t)blockIdx.y * WIDE_COLS;
+  const int nrows = (int)min((int64_t)WIDE_COLS, S.rows - j0);
+  const uint32_t mem0 = (smem_u32(dyn_mem) + 127u) & ~127u;
+  unsigned char* const stages = dyn_mem + (mem0 - smem_u32(dyn_mem));
+  ColumnParams* const s_col = reinterpret_cast<ColumnParams*>(stages + WIDE_BUFFERS * WIDE_STAGE);
+  const uint32_t bars = smem_u32(s_bar);
+
+  if (warp == 0) tmem_alloc(smem_u32(&s_tmem), WIDE_TMEM);
+  if (tid == 0) {
+    for (int b = 0; b < WIDE_BUFFERS; ++b) mbar_init(bars + 8 * b, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  for (int j = tid; j < nrows; j += WIDE_THREADS) s_col[j] = column_params<kLanesAreActivations>(g, S, j0 + j);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = s_tmem;
+  const uint32_t idesc = instr_desc((nrows + 15) & ~15);
+
+  // lane side: thread = row (a warp reaches the 32 lanes of its quarter) and half of the stage's words
+  const int quarter = warp & 3, half = warp >> 2;
+  const int64_t gl = i0 + quarter * 32 + lane;
+  const bool row_in = gl < L.rows;
+  const uint32_t* const row = L.mask + (row_in ? gl : 0) * (int64_t)L.ld + 4 * half;
+  const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
+  // column side: thread = row and two words; eight neighbouring threads write 128 contiguous bytes
+  const int crow = (tid >> 4) * 8 + (tid & 7), piece = (tid >> 3) & 1;
+  const bool col_in = crow < nrows;
+  const uint32_t* const column = S.mask + (j0 + (col_in ? crow : 0)) * (int64_t)S.ld + 4 * piece;
+  const int chunks = (g.words + WIDE_WORDS - 1) / WIDE_WORDS, real_words = (g.n + 31) >> 5;
+
+  uint4 qa, qb;
+  auto fetch = [&](int c) {
+    const int w = c * WIDE_WORDS;
+    qa = row_in && w + 4 * half < g.words ? __ldg(reinterpret_cast<const uint4*>(row + w)) : make_uint4(0, 0, 0, 0);
+    qb = col_in && w + 4 * piece < g.words ? __ldg(reinterpret_cast<const uint4*>(column + w)) : make_uint4(0, 0, 0, 0);
+  };
+  bool dead = false;
+  fetch(0);
+  for (int c = 0; c < chunks; ++c) {
+    const uint32_t buffer = c % WIDE_BUFFERS, bar = bars + 8 * buffer;
+    // the products that read this buffer last are done
+    if (c >= WIDE_BUFFERS) mbar_wait(bar, (uint32_t)(c / WIDE_BUFFERS - 1) & 1u, dead, &g_mma_wait_timeouts);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    uint32_t e[32];
+    expand_bits(qa.x, e);
+    expand_bits(qa.y, e + 8);
+    expand_bits(qa.z, e + 16);
+    expand_bits(qa.w, e + 24);
+    tmem_store_32(tmem + lanes + WIDE_COLS + buffer * WIDE_ACOLS + half * 32, e);
+    unsigned char* const dst = stages + buffer * WIDE_STAGE + (uint32_t)(crow >> 3) * WIDE_SBO + (uint32_t)(8 * piece) * 128 + (crow & 7) * 16;
+    expand_word_bits<true>(qb.x, dst);
+    expand_word_bits<true>(qb.y, dst + 256);
+    expand_word_bits<true>(qb.z, dst + 512);
+    expand_word_bits<true>(qb.w, dst + 768);
+    if (c + 1 < chunks) fetch(c + 1);
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy stores -> tensor-core reads
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (tid == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t b_addr = mem0 + buffer * WIDE_STAGE, a_col = tmem + WIDE_COLS + buffer * WIDE_ACOLS;
+      const int kw = min(WIDE_WORDS, real_words - c * WIDE_WORDS);
+      for (int t = 0; t < kw; ++t)
+        mma_i8_tmem(tmem, a_col + 8 * t, smem_desc(b_addr + t * 256, 128, WIDE_SBO), idesc, (c | t) != 0);
+      mma_commit(bar);
+    }
+  }
+  // the last commit covers every instruction issued before it
+  mbar_wait(bars + 8 * ((chunks - 1) % WIDE_BUFFERS), (uint32_t)((chunks - 1) / WIDE_BUFFERS) & 1u, dead, &g_mma_wait_timeouts);
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  {
+    const bool valid = row_in && !dead;
+    RescaleSide lane_side{0.0, 0.0, 0.0};
+    int64_t off = 0;
+    if (valid) {
+      lane_side = L.rescaled(gl, g.n);
+      off = kLanesAreActivations ? act_offset(g, gl) : gl * g.map.col_stride;
+    }
+#pragma unroll 1
+    for (int cb = 2 * half; cb < 2 * half + 2 && cb * 32 < nrows; ++cb) {
+      uint32_t v[32];
+      tmem_load_32(tmem + lanes + cb * 32, v);
+      if (valid) store_columns<kLanesAreActivations, kPost>(g, v, nrows - cb * 32, s_col + cb * 32, j0 + cb * 32, gl, lane_side, off);
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tmem, WIDE_TMEM);
 }
 
 inline size_t dynamic_bytes(int kq, int ncap) {
@@ -270,6 +389,17 @@ template <bool kLanesAreActivations, bool kPost>
 cudaError_t launch_side(const GemmArgs& args, cudaStream_t stream) {
   const int64_t lane_rows = kLanesAreActivations ? args.M : args.N, col_rows = kLanesAreActivations ? args.N : args.M;
   // Column tile: the full 256 columns of an accumulator unless that leaves most SMs without a CTA.
+  const int64_t wide_x = (lane_rows + MMA_M - 1) / MMA_M, wide_y = (col_rows + WIDE_COLS - 1) / WIDE_COLS;
+  // Rows of 32 words or more, tiles for every SM: measured, the other form against this one, 256 images of 128 x 28 x 28 (36 words)
+  // 60 and 58 us, 256 x 14 x 14 (72) 47 and 39, 512 x 7 x 7 (144) 47 and 37; but 64 x 56 x 56 (18) 95 and 136, where the store
+  // of the outputs is most of it and narrow tiles keep more CTAs in flight.
+  if (args.words >= 32 && col_rows > 64 && wide_x * wide_y >= sm_count() && wide_x <= 0x7FFFFFFF && wide_y <= 65535) {
+    auto kernel = binary_gemm_wide_kernel<kLanesAreActivations, kPost>;
+    cudaError_t e = ensure_dynamic_smem(kernel, WIDE_BYTES);
+    if (e != cudaSuccess) return e;
+    kernel<<<dim3((unsigned)wide_x, (unsigned)wide_y), WIDE_THREADS, WIDE_BYTES, stream>>>(args);
+    return cudaGetLastError();
+  }
   const int64_t gx = (lane_rows + MMA_M - 1) / MMA_M;
   int tile_cols = MMA_NMAX;
   while (tile_cols > 64 && gx * ((col_rows + tile_cols - 1) / tile_cols) < 2 * sm_count()) tile_cols >>= 1;

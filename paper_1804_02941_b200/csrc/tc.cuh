@@ -72,6 +72,17 @@ __device__ __forceinline__ void mma_i8(uint32_t tmem_d, uint64_t desc_a, uint64_
       : "memory");
 }
 
+// The same with the first operand in tensor memory: row i in lane i, four consecutive K bytes per column.
+__device__ __forceinline__ void mma_i8_tmem(uint32_t tmem_d, uint32_t tmem_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, {%5, %6, %7, %8}, p;\n\t}"
+      :
+      : "r"(tmem_d), "r"(tmem_a), "l"(desc_b), "r"(idesc), "r"(accumulate), "r"(0u), "r"(0u), "r"(0u), "r"(0u)
+      : "memory");
+}
+
 // Arrives on the barrier once every tcgen05.mma issued by this thread so far has completed.
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -101,6 +112,20 @@ __device__ __forceinline__ void tmem_load_32(uint32_t taddr, uint32_t (&v)[32]) 
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// 32 consecutive columns of this warp's 32 lanes (no wait: follow with tcgen05.wait::st).
+__device__ __forceinline__ void tmem_store_32(uint32_t taddr, const uint32_t (&v)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};"
+      :
+      : "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
+        "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]),
+        "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]),
+        "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31]), "r"(taddr)
+      : "memory");
+}
+
 // Eight consecutive columns of this warp's 32 lanes (no wait: follow with tmem_load_wait).
 __device__ __forceinline__ void tmem_load_8(uint32_t taddr, uint32_t (&v)[8]) {
   asm volatile(
@@ -122,9 +147,8 @@ __device__ __forceinline__ uint32_t select4(uint32_t selector) {
 }
 
 // One mask word of one row -> two 16-byte K chunks of 0 / -1 bytes (signed 8-bit
-// operands: (-1) x (-1) = 1, so the integer dot product of two such rows is popc(e AND f)).  Within a word's
-// 32 bytes the bits appear in the order 0 4 8 12, 1 5 9 13, 2 6 10 14, 3 7 11 15, then the same for the upper
-// half: a permutation of the contraction index, the same on both operands, that the sum does not see.
+// operands).  Within a word's 32 bytes the bits appear in the order 0 4 8 12, 1 5 9 13, 2 6 10 14, 3 7 11 15, then the
+// same for the upper half.
 __device__ __forceinline__ void expand_word_signed(uint32_t w, unsigned char* dst) {
   uint4 lo, hi;
   lo.x = select4(w);
@@ -139,12 +163,28 @@ __device__ __forceinline__ void expand_word_signed(uint32_t w, unsigned char* ds
   *reinterpret_cast<uint4*>(dst + 128) = hi;
 }
 
-// One 16-byte piece (four mask words) of one row -> eight 16-byte K chunks.
-__device__ __forceinline__ void expand_words_signed(uint4 q, unsigned char* dst) {
-  expand_word_signed(q.x, dst);
-  expand_word_signed(q.y, dst + 256);
-  expand_word_signed(q.z, dst + 512);
-  expand_word_signed(q.w, dst + 768);
+// Mask words as unsigned bytes for the contraction of two such rows.  Register j of a word holds its bits j, j + 8, j + 16 and
+// j + 24, one per byte and where they stand: 2^j or 0.  The other side's are mirrored, 2^(7-j) or 0, so that every product of two set
+// bits is 128: the integer dot product of the rows is kBitProduct * popc(e AND f), and an AND per four bits is all it takes.
+constexpr int kBitProductLog = 7;
+__device__ __forceinline__ void expand_bits(uint32_t w, uint32_t* out) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j) out[j] = w & (0x01010101u << j);
+}
+__device__ __forceinline__ void expand_bits_mirrored(uint32_t w, uint32_t* out) {
+  const uint32_t m = __byte_perm(__brev(w), 0u, 0x0123);  // the bits of every byte in reverse order
+#pragma unroll
+  for (int j = 0; j < 8; ++j) out[j] = m & (0x80808080u >> j);
+}
+
+// A mask word of one row -> its two 16-byte K chunks, 128 bytes apart.
+template <bool kMirrored>
+__device__ __forceinline__ void expand_word_bits(uint32_t w, unsigned char* dst) {
+  uint32_t b[8];
+  if (kMirrored) expand_bits_mirrored(w, b);
+  else expand_bits(w, b);
+  *reinterpret_cast<uint4*>(dst) = make_uint4(b[0], b[1], b[2], b[3]);
+  *reinterpret_cast<uint4*>(dst + 128) = make_uint4(b[4], b[5], b[6], b[7]);
 }
 
 }  // namespace tc
