@@ -74,7 +74,7 @@ struct Grid {
   double elo[kMaxBuckets];       // signed start of the bucket's octave and signed unit of the mantissas there:
   double ulp[kMaxBuckets];       // sum of a bucket = count * elo + sum of the mantissas * ulp
   float edge[kMaxBuckets + 1];   // ascending; edge[B0] = 0
-  uint32_t hist[kMaxCells];      // sampled values per cell
+  uint32_t hist[kTileWarps * 32];  // sampled values per cell; once the grid is chosen, 32 words for each warp's search
   uint8_t lut[kMaxSteps + 2];    // bucket of a step
   float part[2][kTileWarps];     // per-warp partial sums
   uint32_t ipart[kTileWarps];
@@ -561,7 +561,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) binarize_patches_tile_kernel(
   uint16_t* const map = reinterpret_cast<uint16_t*>(invert + a.TH * a.TW);        // [window] slot of a pixel under the tile
   uint16_t* const win = map + window;                                             // [kh*kw] offsets of the window
   __shared__ Grid grid;
-  __shared__ float hulls[WARPS][32];
+  static_assert(kMaxCells <= kTileWarps * 32, "cells");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
   int t = blockIdx.x;
@@ -723,7 +723,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) binarize_patches_tile_kernel(
   // ---- the search: a warp per patch ----
   for (int p = warp; p < npatch; p += WARPS) {
     PatchCode code{0, 0.0f, 0.0f, __uint_as_float(0x7FC00000u), false};
-    if (top != 0u) code = search_patch<KHW, BPL>(a, grid, map, win, window_at(p), sums, counts, list, tile, hulls[warp], lane);
+    if (top != 0u) code = search_patch<KHW, BPL>(a, grid, map, win, window_at(p), sums, counts, list, tile, reinterpret_cast<float*>(grid.hist) + 32 * warp, lane);
     __syncwarp();
     if (lane == 0) store(p, code);
   }
@@ -831,7 +831,7 @@ size_t tile_bytes(TileArgs* t) {
   return a.tile_at + sizeof(float) * slots * a.pitch + 4 * slots + 8 * patches + 2 * ((size_t)a.in_h * a.in_w + khw);
 }
 
-constexpr size_t kSmemPerSm = 228 * 1024, kSmemCtaMax = 227 * 1024, kTileStatic = sizeof(Grid) + kTileWarps * 32 * sizeof(float) + 64;
+constexpr size_t kSmemPerSm = 228 * 1024, kSmemCtaMax = 227 * 1024, kTileStatic = sizeof(Grid) + 64;
 
 // The tile whose estimated time over the whole layer is least, in cycles.  From phase timings on 64 x 56 x 56 (7 x 14 tiles,
 // two CTAs per SM): per tile a fixed part, 4.3 per staged value and 6200 per round of 16 patches (a warp each); a CTA alone
