@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS) binary_gemm_mma_kernel(cons
   Side L, S;
   both_sides<kLanesAreActivations>(g, L, S);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = (int)uniform(tid >> 5), lane = tid & 31;
   const int64_t i0 = (int64_t)blockIdx.x * MMA_M;
   const int64_t j0 = (int64_t)blockIdx.y * tile_cols;        // tile_cols: 64, 128 or 256 column-side rows per CTA
   const int nrows = (int)min((int64_t)tile_cols, S.rows - j0);  // column-side rows of this tile
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS) binary_gemm_mma_kernel(cons
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = s_tmem;
+  const uint32_t tmem = uniform(s_tmem);
   const uint32_t idesc = instr_desc(NT);
 
   // units of this thread: lane-side pieces first, then column-side pieces
@@ -223,13 +223,13 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS) binary_gemm_mma_kernel(cons
     if (c + 1 < chunks) fetch(c + 1);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy stores -> tensor-core reads
     __syncthreads();
-    if (tid == 0) {
+    if (warp == 0 && elect_one()) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t a_addr = mem0, b_addr = mem0 + a_bytes;
+      const uint64_t da = smem_desc(mem0, 128, SBO), db = smem_desc(mem0 + a_bytes, 128, SBO);
       const int kw = min(4 * KQ, real_words - c * 4 * KQ);
-      for (int t = 0; t < kw; ++t)  // one mask word = 32 K bytes = two K chunks per instruction
-        mma_i8(tmem, smem_desc(a_addr + t * 256, 128, SBO), smem_desc(b_addr + t * 256, 128, SBO), idesc,
-               (c | t) != 0);
+#pragma unroll
+      for (int t = 0; t < 4 * KQ; ++t)  // one mask word = 32 K bytes = two K chunks per instruction
+        if (t < kw) mma_i8(tmem, desc_at(da, t * 256), desc_at(db, t * 256), idesc, (c | t) != 0);
       mma_commit(bar);
     }
   }
@@ -262,10 +262,11 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS) binary_gemm_mma_kernel(cons
 // thread writes four words of its row, expanded, into tensor memory, from where the tensor cores take their first operand.
 // What is left there is the column side, written and read once: in the kernel above 24 KB pass through shared memory per 32 bits
 // of 128 x 256 outputs, 192 cycles, where the products take 128; here it is 16 KB, 128 cycles.  Two stages of eight words, one
-// barrier each.  Bound by the load and shared-memory pipe (0.79 busy; tensor cores 0.46): a warp's load of 16 bytes per row takes it 32 cycles.
-// 8192 x 8192 x 4608 bits: 346 us in the kernel above, 287 here (369 with stages of four words and loads of 8 bytes; 310 with
+// barrier each, on which the workers only arrive: a warp of its own issues the products.  Bound by the load and shared-memory
+// pipe (0.79 busy; tensor cores 0.46): a warp's load of 16 bytes per row takes it 32 cycles.  8192 x 8192 x 4608 bits: 346 us in
+// the kernel above, 278 here (287 with a worker issuing; 369 with stages of four words and loads of 8 bytes; 310 with
 // the words staged in shared memory by 16-byte asynchronous copies, 418 by bulk copies of 64 bytes per row).
-constexpr int WIDE_THREADS = 256, WIDE_COLS = 128, WIDE_WORDS = 8, WIDE_BUFFERS = 2;
+constexpr int WIDE_WORKERS = 256, WIDE_THREADS = WIDE_WORKERS + 32, WIDE_COLS = 128, WIDE_WORDS = 8, WIDE_BUFFERS = 2;
 constexpr uint32_t WIDE_SBO = 2 * WIDE_WORDS * 128, WIDE_STAGE = WIDE_COLS * WIDE_WORDS * 32;  // bytes
 constexpr uint32_t WIDE_ACOLS = WIDE_WORDS * 8;            // columns of a lane-side stage: 4 bytes each; behind the accumulator
 constexpr uint32_t WIDE_TMEM = WIDE_COLS + WIDE_BUFFERS * WIDE_ACOLS;
@@ -279,7 +280,7 @@ __global__ void __launch_bounds__(WIDE_THREADS, 2) binary_gemm_wide_kernel(const
   __shared__ uint32_t s_tmem;
   Side L, S;
   both_sides<kLanesAreActivations>(g, L, S);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = (int)uniform(tid >> 5), lane = tid & 31;
   const int64_t i0 = (int64_t)blockIdx.x * MMA_M, j0 = (int64_t)blockIdx.y * WIDE_COLS;
   const int nrows = (int)min((int64_t)WIDE_COLS, S.rows - j0);
   const uint32_t mem0 = (smem_u32(dyn_mem) + 127u) & ~127u;
@@ -296,7 +297,7 @@ __global__ void __launch_bounds__(WIDE_THREADS, 2) binary_gemm_wide_kernel(const
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = s_tmem;
+  const uint32_t tmem = uniform(s_tmem);
   const uint32_t idesc = instr_desc((nrows + 15) & ~15);
 
   // lane side: thread = row (a warp reaches the 32 lanes of its quarter) and half of the stage's words
@@ -318,42 +319,53 @@ __global__ void __launch_bounds__(WIDE_THREADS, 2) binary_gemm_wide_kernel(const
     qb = col_in && w + 4 * piece < g.words ? __ldg(reinterpret_cast<const uint4*>(column + w)) : make_uint4(0, 0, 0, 0);
   };
   bool dead = false;
-  fetch(0);
-  for (int c = 0; c < chunks; ++c) {
-    const uint32_t buffer = c % WIDE_BUFFERS, bar = bars + 8 * buffer;
-    // the products that read this buffer last are done
-    if (c >= WIDE_BUFFERS) mbar_wait(bar, (uint32_t)(c / WIDE_BUFFERS - 1) & 1u, dead, &g_mma_wait_timeouts);
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    uint32_t e[32];
-    expand_bits(qa.x, e);
-    expand_bits(qa.y, e + 8);
-    expand_bits(qa.z, e + 16);
-    expand_bits(qa.w, e + 24);
-    tmem_store_32(tmem + lanes + WIDE_COLS + buffer * WIDE_ACOLS + half * 32, e);
-    unsigned char* const dst = stages + buffer * WIDE_STAGE + (uint32_t)(crow >> 3) * WIDE_SBO + (uint32_t)(8 * piece) * 128 + (crow & 7) * 16;
-    expand_word_bits<true>(qb.x, dst);
-    expand_word_bits<true>(qb.y, dst + 256);
-    expand_word_bits<true>(qb.z, dst + 512);
-    expand_word_bits<true>(qb.w, dst + 768);
-    if (c + 1 < chunks) fetch(c + 1);
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy stores -> tensor-core reads
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (tid == 0) {
+  if (warp == WIDE_WORKERS / 32) {  // the last warp issues the products
+    const uint64_t b_desc = smem_desc(mem0, 128, WIDE_SBO);
+    for (int c = 0; c < chunks; ++c) {
+      const uint32_t buffer = c % WIDE_BUFFERS;
+      bar_sync(1 + buffer, WIDE_THREADS);
+      if (elect_one()) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint64_t db = desc_at(b_desc, buffer * WIDE_STAGE);
+        const uint32_t a_col = tmem + WIDE_COLS + buffer * WIDE_ACOLS;
+        const int kw = min(WIDE_WORDS, real_words - c * WIDE_WORDS);
+#pragma unroll
+        for (int t = 0; t < WIDE_WORDS; ++t)
+          if (t < kw) mma_i8_tmem(tmem, a_col + 8 * t, desc_at(db, t * 256), idesc, (c | t) != 0);
+        mma_commit(bars + 8 * buffer);
+      }
+      __syncwarp();
+    }
+  } else {
+    fetch(0);
+    for (int c = 0; c < chunks; ++c) {
+      const uint32_t buffer = c % WIDE_BUFFERS, bar = bars + 8 * buffer;
+      // the products that read this buffer last are done
+      if (c >= WIDE_BUFFERS) mbar_wait(bar, (uint32_t)(c / WIDE_BUFFERS - 1) & 1u, dead, &g_mma_wait_timeouts);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t b_addr = mem0 + buffer * WIDE_STAGE, a_col = tmem + WIDE_COLS + buffer * WIDE_ACOLS;
-      const int kw = min(WIDE_WORDS, real_words - c * WIDE_WORDS);
-      for (int t = 0; t < kw; ++t)
-        mma_i8_tmem(tmem, a_col + 8 * t, smem_desc(b_addr + t * 256, 128, WIDE_SBO), idesc, (c | t) != 0);
-      mma_commit(bar);
+      uint32_t e[32];
+      expand_bits(qa.x, e);
+      expand_bits(qa.y, e + 8);
+      expand_bits(qa.z, e + 16);
+      expand_bits(qa.w, e + 24);
+      tmem_store_32(tmem + lanes + WIDE_COLS + buffer * WIDE_ACOLS + half * 32, e);
+      unsigned char* const dst = stages + buffer * WIDE_STAGE + (uint32_t)(crow >> 3) * WIDE_SBO + (uint32_t)(8 * piece) * 128 + (crow & 7) * 16;
+      expand_word_bits<true>(qb.x, dst);
+      expand_word_bits<true>(qb.y, dst + 256);
+      expand_word_bits<true>(qb.z, dst + 512);
+      expand_word_bits<true>(qb.w, dst + 768);
+      if (c + 1 < chunks) fetch(c + 1);
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy stores -> tensor-core reads
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      bar_arrive(1 + buffer, WIDE_THREADS);  // (the buffer's next use waits for the products, which wait for this barrier)
     }
   }
   // the last commit covers every instruction issued before it
   mbar_wait(bars + 8 * ((chunks - 1) % WIDE_BUFFERS), (uint32_t)((chunks - 1) / WIDE_BUFFERS) & 1u, dead, &g_mma_wait_timeouts);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   {
-    const bool valid = row_in && !dead;
+    const bool valid = row_in && !dead && warp < WIDE_WORKERS / 32;
     RescaleSide lane_side{0.0, 0.0, 0.0};
     int64_t off = 0;
     if (valid) {
@@ -361,7 +373,7 @@ __global__ void __launch_bounds__(WIDE_THREADS, 2) binary_gemm_wide_kernel(const
       off = kLanesAreActivations ? act_offset(g, gl) : gl * g.map.col_stride;
     }
 #pragma unroll 1
-    for (int cb = 2 * half; cb < 2 * half + 2 && cb * 32 < nrows; ++cb) {
+    for (int cb = 2 * half; cb < 2 * half + 2 && cb * 32 < nrows && warp < WIDE_WORKERS / 32; ++cb) {
       uint32_t v[32];
       tmem_load_32(tmem + lanes + cb * 32, v);
       if (valid) store_columns<kLanesAreActivations, kPost>(g, v, nrows - cb * 32, s_col + cb * 32, j0 + cb * 32, gl, lane_side, off);
@@ -391,7 +403,7 @@ cudaError_t launch_side(const GemmArgs& args, cudaStream_t stream) {
   // Column tile: the full 256 columns of an accumulator unless that leaves most SMs without a CTA.
   const int64_t wide_x = (lane_rows + MMA_M - 1) / MMA_M, wide_y = (col_rows + WIDE_COLS - 1) / WIDE_COLS;
   // Rows of 32 words or more, tiles for every SM: measured, the other form against this one, 256 images of 128 x 28 x 28 (36 words)
-  // 60 and 58 us, 256 x 14 x 14 (72) 47 and 39, 512 x 7 x 7 (144) 47 and 37; but 64 x 56 x 56 (18) 95 and 136, where the store
+  // 60 and 56 us, 256 x 14 x 14 (72) 47 and 37, 512 x 7 x 7 (144) 47 and 35; but 64 x 56 x 56 (18) 95 and 136, where the store
   // of the outputs is most of it and narrow tiles keep more CTAs in flight.
   if (args.words >= 32 && col_rows > 64 && wide_x * wide_y >= sm_count() && wide_x <= 0x7FFFFFFF && wide_y <= 65535) {
     auto kernel = binary_gemm_wide_kernel<kLanesAreActivations, kPost>;

@@ -25,6 +25,13 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes,
          ((uint64_t)(sbo_bytes >> 4) << 32) | (1ull << 46);
 }
 
+// The descriptor of the same operand `bytes` (a multiple of 16) further on.
+__device__ __forceinline__ uint64_t desc_at(uint64_t desc, uint32_t bytes) { return desc + (bytes >> 4); }
+
+// Named barriers: `threads` threads in all, of which some only arrive.
+__device__ __forceinline__ void bar_arrive(int id, int threads) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
+__device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
+
 // Instruction descriptor of kind::i8: D format S32 (2 at bit 4), A format at bit 7 and B format at bit 10
 // (0: unsigned 8-bit, 1: signed 8-bit), both K-major (0 at bits 15 and 16), N / 8 at bit 17, M / 16 at bit 24.
 __device__ __forceinline__ uint32_t instr_desc(int nt, bool a_signed = false, bool b_signed = false) {
@@ -61,14 +68,18 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, bool& d
   }
 }
 
+// The operands of an instruction live in uniform registers.  Issued under a branch on the thread, with operands the compiler
+// cannot tell are the warp's, one took 175 cycles to issue, whatever it multiplied (128 x 128 x 32: 64 cycles of tensor-core
+// time).  So: a warp's number and the tensor-memory address go through uniform(), the loops over instructions are unrolled,
+// and elect_one() picks the thread inside a branch that the whole warp takes.
 __device__ __forceinline__ void mma_i8(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc,
                                        uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, {%5, %6, %7, %8}, p;\n\t}"
+      "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
       :
-      : "r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate), "r"(0u), "r"(0u), "r"(0u), "r"(0u)
+      : "r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 
@@ -77,10 +88,19 @@ __device__ __forceinline__ void mma_i8_tmem(uint32_t tmem_d, uint32_t tmem_a, ui
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, {%5, %6, %7, %8}, p;\n\t}"
+      "tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, p;\n\t}"
       :
-      : "r"(tmem_d), "r"(tmem_a), "l"(desc_b), "r"(idesc), "r"(accumulate), "r"(0u), "r"(0u), "r"(0u), "r"(0u)
+      : "r"(tmem_d), "r"(tmem_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
       : "memory");
+}
+
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __shfl_sync(0xFFFFFFFFu, v, 0); }
+
+// True in one thread of the (converged) warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(e));
+  return e != 0u;
 }
 
 // Arrives on the barrier once every tcgen05.mma issued by this thread so far has completed.
