@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
   __shared__ double s_alpha[NT], s_beta[NT];
   __shared__ __align__(16) int32_t s_off[2][KS];  // byte offsets of a stage's elements in the staged channels
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = (int)uniform(tid >> 5), lane = tid & 31;
   const uint32_t mem0 = (smem_u32(dyn_mem) + 127u) & ~127u;
   unsigned char* const operands = dyn_mem + (mem0 - smem_u32(dyn_mem));
   const int tile_words = a.max_ch * a.ch_words;
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = s_tmem;
+  const uint32_t tmem = uniform(s_tmem);
   const int my_sexp = s_rowsexp[row];
   const bool gather = my_sexp != INT_MIN && my_sexp != INT_MAX;
   // x * 2^sexp in two exact steps: 2^sexp itself is beyond fp32 for the smallest patches
@@ -279,14 +279,15 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
   const uint32_t idesc_u = instr_desc(NT, false, true), idesc_s = instr_desc(NT, true, true);
   auto multiply = [&](int st) {  // (one thread) the products of stage `st`
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t a_addr = mem0 + (st & 1) * STAGE, b_addr = a_addr + 4 * PLANE;
+    const uint64_t da = smem_desc(mem0 + (st & 1) * STAGE, 128, SBO), db = desc_at(da, 4 * PLANE);
     const int kw = min(JS, a.words - st * JS);
-    for (int t = 0; t < kw; ++t) {
-      const uint64_t db = smem_desc(b_addr + t * 256, 128, SBO);
-      for (int p = 0; p < 4; ++p)
-        mma_i8(tmem + (uint32_t)(p * NT), smem_desc(a_addr + p * PLANE + t * 256, 128, SBO), db,
-               p == 3 ? idesc_s : idesc_u, (st | t) != 0);
-    }
+#pragma unroll
+    for (int t = 0; t < JS; ++t)
+      if (t < kw)
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+          mma_i8(tmem + (uint32_t)(p * NT), desc_at(da, p * PLANE + t * 256), desc_at(db, t * 256), p == 3 ? idesc_s : idesc_u,
+                 (st | t) != 0);
     mma_commit(st & 1 ? bar1 : bar0);
   };
 
@@ -300,7 +301,7 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy stores of the last stage -> tensor-core reads
     __syncthreads();  // this stage's channels have arrived, the last stage's operands are complete
-    if (st > 0 && tid == 0) multiply(st - 1);
+    if (st > 0 && warp == 0 && elect_one()) multiply(st - 1);
     if (st + 1 < stages) {
       stage_in(st + 1);
       next_mask = load_mask(st + 1);
@@ -324,7 +325,7 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
-  if (tid == 0) multiply(stages - 1);
+  if (warp == 0 && elect_one()) multiply(stages - 1);
   // the last commit covers every instruction before it
   mbar_wait((stages - 1) & 1 ? bar1 : bar0, (uint32_t)((stages - 1) >> 1) & 1u, dead, &g_wbin_wait_timeouts);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
