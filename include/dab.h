@@ -351,7 +351,7 @@ dab_status dab_network_forward(const dab_layer* layers, int32_t count, int32_t N
  *                        tcgen05.mma kind::i8 into tensor memory;
  *   DAB_CONTRACT_POPC    AND, carry-save adders and population counts on the integer pipes;
  *   DAB_CONTRACT_AUTO    (default) the tensor-core kernel, except for problems so small (fewer 128 x 64
- *                        output tiles than a third of the SMs) that its per-tile latency is all there is.
+ *                        output tiles than a third of the SMs, rows not short) that its per-tile latency is all there is.
  * Both kernels give the same counts and the same outputs bit for bit.  The setting is process-wide and read at
  * each call; the two forced values exist so that the kernels can be tested and measured against each other.
  */

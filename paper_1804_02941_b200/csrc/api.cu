@@ -21,13 +21,15 @@ std::atomic<int> g_contraction{(int)DAB_CONTRACT_AUTO};
 // (weights when lanes_along_rows, activations otherwise) at least 64 rows per grid row; a launch too tall for
 // that takes the population-count kernel, and so does, under DAB_CONTRACT_AUTO, one whose 128 x 64 tiles are
 // fewer than a third of the SMs: there the tensor-core kernel is a chain of dependent stage rounds on a few SMs, while the
-// other splits its rows.  Measured, population counts against tensor cores: 4096 x 32 of 9216 bits (32 tiles) 27 and 51 us,
-// 256 x 2000 of 1152 (64 tiles) 16.5 and 14.4, 512 x 1568 of 4608 (100 tiles) 39 and 31.
+// other splits its rows; rows of 24 words or less are no chain.  Measured, population counts against tensor cores: 4096 x 32 of
+// 128 words (32 tiles) 12.7 and 19.0 us, 128 x 961 of 50 (16 tiles) 8.1 and 10.3; 101 x 3952 of 31 (62 tiles) 9.4 and 8.4,
+// 300 x 1000 of 16 (48 tiles) 7.7 and 6.1, 64 x 1024 of 18 (16 tiles) 7.7 and 6.3, 67 x 128 of 24 (2 tiles) 6.8 and 6.8.
 cudaError_t contract(const GemmArgs& g, bool lanes_along_rows, cudaStream_t stream) {
   const int64_t lane_rows = lanes_along_rows ? g.M : g.N, column_rows = lanes_along_rows ? g.N : g.M;
   const int mode = g_contraction.load(std::memory_order_relaxed);
   bool tensor = mode != (int)DAB_CONTRACT_POPC && column_rows <= (int64_t)65535 * 64;
-  if (mode == (int)DAB_CONTRACT_AUTO && ((lane_rows + 127) / 128) * ((column_rows + 63) / 64) * 3 < sm_count()) tensor = false;
+  const int64_t tiles = ((lane_rows + 127) / 128) * ((column_rows + 63) / 64);
+  if (mode == (int)DAB_CONTRACT_AUTO && tiles * 3 < sm_count() && (g.words > 24 || tiles < 8)) tensor = false;
   return tensor ? launch_gemm_mma(g, lanes_along_rows, stream) : launch_gemm(g, lanes_along_rows, stream);
 }
 

@@ -3,8 +3,8 @@
 //
 // A launch of few tiles splits the row length over the CTAs of a cluster: each counts its share of the words, then
 // finishes its share of the tile's outputs from the counts of all of them (distributed shared memory).  Bound by the chain
-// of slices and by POPC (16 a clock and SM): 1 x 512 outputs of 392 words took 65 us on 8 CTAs of 64 x 64 outputs and less
-// than 15 on 64 of 16 x 64; the five such layers of a sketch classified alone 132 us, now 55.
+// of slices and by POPC (16 a clock and SM): 1 x 512 outputs of 392 words took 65 us on 8 CTAs of 64 x 64 outputs and
+// 7 on 64 of 16 x 64; the five such layers of a sketch classified alone 132 us, now 55.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -174,9 +174,13 @@ template <bool kLanesAlongRows, int TM>
 cudaError_t launch_rows(const GemmArgs& args, cudaStream_t stream) {
   const dim3 grid((unsigned)((args.M + 16 * TM - 1) / (16 * TM)), (unsigned)((args.N + BN - 1) / BN));
   if (grid.y > 65535) return cudaErrorInvalidValue;
-  // Split until there are two CTAs per SM, shares of no less than 12 words (a quarter of a slice).
+  // Split up to eight ways while the CTAs fit the SMs once and a member has six words.  The cluster and its two barriers cost 3 us,
+  // so two ways pay only for long rows.  Measured, whole and split: 225 x 256 of 72 words 14.5 and 7.9 us (eight ways), of 36 words
+  // 9.4 and 7.3 (four), 10.4 (two); 32 x 4096 of 128 words 21.9 and 12.7 (two), 17.5 (eight, four waves of CTAs).
+  const int64_t tiles = (int64_t)grid.x * grid.y;
   int splits = 1;
-  while (splits < kMaxSplit && (int64_t)grid.x * grid.y * splits < 2 * sm_count() && args.words >= 24 * splits) splits *= 2;
+  while (splits < kMaxSplit && tiles * 2 * splits <= sm_count() && args.words >= 12 * splits) splits *= 2;
+  if (splits == 2 && args.words < 96) splits = 1;
   if (splits == 1) {
     binary_gemm_kernel<kLanesAlongRows, TM, false><<<grid, GEMM_THREADS, 0, stream>>>(args, args.words);
     return cudaGetLastError();
