@@ -235,7 +235,9 @@ def patch_launches(L, coder):
         return 1
     pixel = n <= 8192 and L.kh * L.kw >= 4 and L.patches >= 1024
     if coder == "pixel" or (coder == "auto" and pixel):
-        return 2                      # tile coder, then the kernel that codes the patches it marked
+        # tile coder, then the kernel that codes the patches it marked; long rows of strided windows, which share little, may go to
+        # a CTA per patch at once (a lower bound)
+        return 1 if coder == "auto" and L.stride > 1 and n > 2048 else 2
     if coder == "auto" and (L.kh * L.kw >= 4 or L.patches < 1024 or n > 8192):
         return 1                      # a CTA per patch
     if coder == "auto":

@@ -33,13 +33,15 @@ def main():
             d["bytes"] += v * {"byte": 1.0, "kbyte": 1e3, "mbyte": 1e6, "gbyte": 1e9}[unit]
     launches = [per_launch[k] for k in sorted(per_launch)]
     layers = configs.config5(256)
-    out, i = {}, 0
-    for L in layers:
-        n = bench.patch_launches(L, "auto")
-        out[L.name] = sum(x["bytes"] for x in launches[i:i + n])
-        i += n
-    if i != len(launches):
-        raise SystemExit("captured %d launches, one step has %d" % (len(launches), i))
+    per_layer = []  # a layer's main kernel, then the kernel that takes what it marked
+    for x in launches:
+        if "marked" in x["name"] and per_layer:
+            per_layer[-1] += x["bytes"]
+        else:
+            per_layer.append(x["bytes"])
+    if len(per_layer) != len(layers):
+        raise SystemExit("captured %d layers, one step has %d" % (len(per_layer), len(layers)))
+    out = {L.name: b for L, b in zip(layers, per_layer)}
     rec = {"source_sha256": bench.patch_coder_source_hash(), "batch": 256, "dense": False,
            "command": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none -k regex:binarize_patches "
                       "python bench.py --steps 1 --warmup 3 --no-e2e --no-wbin --no-cpu-baseline (the timed step's launches)",
