@@ -99,7 +99,10 @@ dab_status dab_pack(const uint8_t* d_bits, int64_t rows, int32_t n, int64_t ld_b
  * forward product of Section 4.3.2 expands over the four 0/1 indicator pairs:
  *   C[i,j] = alpha_j gamma_i p11 + alpha_j delta_i p10 + beta_j gamma_i p01 + beta_j delta_i p00,
  *   p11 = popc(e_j & f_i), p10 = K_e - p11, p01 = K_f - p11, p00 = n - K_e - K_f + p11
- * evaluated in fp64 from the fp32 scalars in exactly that order of terms, rounded once to fp32.
+ * evaluated in fp64 from the fp32 scalars and rounded once to fp32.  Pairs with |alpha_j| >= |beta_j| and
+ * |gamma_i| >= |delta_i|, all finite (every row that the coders write, flagged ones aside), may be summed in another
+ * order, with an error before the rounding below 2^-50 of the sum of the terms' magnitudes; every other pair in exactly
+ * the order above.
  *
  *   d_A, lda, d_KA, d_gamma, d_delta   activation side: M packed rows, their K_f, gamma, delta
  *   d_B, ldb, d_KB, d_alpha, d_beta    weight side: N packed rows, their K_e, alpha, beta

@@ -44,8 +44,12 @@ __device__ __forceinline__ float apply_post(const PostOps& ops, float v, int cha
 // (p10 = Ke - p11, p01 = Kf - p11, p00 = n - Ke - Kf + p11) in fp64, one rounding to fp32, gathered by what depends on the pair:
 //   (gamma - delta) ((alpha - beta) p11 + beta Kf) + delta (alpha Ke + beta (n - Ke))
 // Five fp64 operations per output instead of the fifteen of the four terms, which kept the fp64 pipe busy longer than the
-// counting where rows are short.  A product of a value and a count is exact in fp64 and the fused additions round once, so what
-// is rounded on the way stays below 2^-50 of the terms, as before.  Every kernel that rescales does it in exactly these operations.
+// counting where rows are short.  A product of a value and a count is exact in fp64 and the fused additions round once.  What is
+// rounded on the way stays below 2^-50 of the terms' magnitudes if |alpha| >= |beta| and |gamma| >= |delta|, as in every code that
+// the coders write: then no part of the gathered sum is larger than the terms.  Other scales (the contraction entry points take
+// any) could cancel in it: alpha = 1, beta = 0, gamma = 1e-12, delta = 3, p11 = Ke = 100 comes out 9e-5 off.  An output of which
+// either row is not gathers() is formed by rescale_terms, term by term.  Every kernel that rescales does it in exactly these
+// operations.
 struct RescaleSide {  // of a weight row: d = alpha - beta, b = beta, c = alpha Ke + beta (n - Ke); of an activation row: d = gamma -
   double d, b, c;     // delta, b = Kf, c = delta
 };
@@ -61,6 +65,15 @@ __device__ __forceinline__ float rescale(int p11, double wd, double wb, double w
 }
 __device__ __forceinline__ float rescale(int p11, const RescaleSide& w, const RescaleSide& a) {
   return rescale(p11, w.d, w.b, w.c, a.d, a.b, a.c);
+}
+// Values of the set and the clear bits of a row that the gathered form is good for: finite, the first no smaller in magnitude.
+__device__ __forceinline__ bool gathers(float set, float clear) { return fabsf(clear) <= fabsf(set) && !is_nonfinite(set); }
+// The four terms by themselves, every operation rounded, in the order above.
+__device__ __forceinline__ float rescale_terms(int p11, int Ke, int Kf, int n, double alpha, double beta, double gamma, double delta) {
+  double y = __dmul_rn(__dmul_rn(alpha, gamma), int_to_double(p11));
+  y = __dadd_rn(y, __dmul_rn(__dmul_rn(alpha, delta), int_to_double(Ke - p11)));
+  y = __dadd_rn(y, __dmul_rn(__dmul_rn(beta, gamma), int_to_double(Kf - p11)));
+  return (float)__dadd_rn(y, __dmul_rn(__dmul_rn(beta, delta), int_to_double(n - Ke - Kf + p11)));
 }
 
 // Where an output element (row i of the activation side, column j of the weight side) is stored:
@@ -91,6 +104,15 @@ struct GemmArgs {
   int64_t ldp;
   PostOps post;      // applied to every output (convolutions only: column j = channel j)
 };
+
+// Output of activation row i and weight row j with p11 common bits: gathered if both rows are, else term by term.
+__device__ __forceinline__ float rescale_any(const GemmArgs& g, int p11, int64_t i, int64_t j) {
+  const float alpha = g.alpha[DAB_IDX(j, g.N)], beta = g.beta[DAB_IDX(j, g.N)], gamma = g.gamma[DAB_IDX(i, g.M)], delta = g.delta[DAB_IDX(i, g.M)];
+  const int Ke = g.KB[DAB_IDX(j, g.N)], Kf = g.KA[DAB_IDX(i, g.M)];
+  if (gathers(alpha, beta) && gathers(gamma, delta))
+    return rescale(p11, rescale_weight((double)alpha, (double)beta, Ke, g.n), rescale_activation((double)gamma, (double)delta, Kf));
+  return rescale_terms(p11, Ke, Kf, g.n, (double)alpha, (double)beta, (double)gamma, (double)delta);
+}
 
 cudaError_t launch_gemm(const GemmArgs& args, bool lanes_along_rows, cudaStream_t stream);
 // Tensor-core contraction; lanes_along_rows as for launch_gemm.  See gemm_mma.cu.

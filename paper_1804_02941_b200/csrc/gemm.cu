@@ -107,6 +107,8 @@ __global__ void __launch_bounds__(GEMM_THREADS) binary_gemm_kernel(const GemmArg
   auto activation = [&](int64_t gi) {
     return rescale_activation((double)g.gamma[DAB_IDX(gi, g.M)], (double)g.delta[DAB_IDX(gi, g.M)], g.KA[DAB_IDX(gi, g.M)]);
   };
+  auto weight_gathers = [&](int64_t gj) { return gathers(g.alpha[DAB_IDX(gj, g.N)], g.beta[DAB_IDX(gj, g.N)]); };
+  auto activation_gathers = [&](int64_t gi) { return gathers(g.gamma[DAB_IDX(gi, g.M)], g.delta[DAB_IDX(gi, g.M)]); };
   if (kSplit) {
     // The counts meet in shared memory, [column][row] or [row][column] as the lanes of the stores run; a member finishes
     // every splits-th line of the tile.
@@ -126,34 +128,43 @@ __global__ void __launch_bounds__(GEMM_THREADS) binary_gemm_kernel(const GemmArg
     const int* member[kMaxSplit];
 #pragma unroll
     for (int z = 0; z < kMaxSplit; ++z) member[z] = cluster.map_shared_rank(counts, z < splits ? z : 0);
-    for (int t = tid; t < LINE * LINES / splits; t += GEMM_THREADS) {
-      const int line = t / LINE * splits + rank, at = t % LINE;
-      int p11 = 0;
+    bool gathered = true;
+    auto finish = [&](auto each_pair) {
+      for (int t = tid; t < LINE * LINES / splits; t += GEMM_THREADS) {
+        const int line = t / LINE * splits + rank, at = t % LINE;
+        int p11 = 0;
 #pragma unroll
-      for (int z = 0; z < kMaxSplit; ++z)
-        if (z < splits) p11 += member[z][line * PITCH + at];
-      const int64_t gi = i0 + (kLanesAlongRows ? at : line), gj = j0 + (kLanesAlongRows ? line : at);
-      if (gi >= g.M || gj >= g.N) continue;
-      const int64_t to = (gi / g.map.inner) * g.map.outer_stride + (gi % g.map.inner) * g.map.row_stride + gj * g.map.col_stride;
-      if (DAB_IN_BOUNDS(to, g.c_extent))
-        g.C[to] = apply_post(g.post, rescale(p11, weight(gj), activation(gi)), (int)gj, to);
-      if (g.p11 && DAB_IN_BOUNDS(gi * g.ldp + gj, (g.M - 1) * g.ldp + g.N)) g.p11[gi * g.ldp + gj] = p11;
-    }
+        for (int z = 0; z < kMaxSplit; ++z)
+          if (z < splits) p11 += member[z][line * PITCH + at];
+        const int64_t gi = i0 + (kLanesAlongRows ? at : line), gj = j0 + (kLanesAlongRows ? line : at);
+        if (gi >= g.M || gj >= g.N) continue;
+        const int64_t to = (gi / g.map.inner) * g.map.outer_stride + (gi % g.map.inner) * g.map.row_stride + gj * g.map.col_stride;
+        const float y = decltype(each_pair)::value ? rescale_any(g, p11, gi, gj) : rescale(p11, weight(gj), activation(gi));
+        if (!decltype(each_pair)::value) gathered = gathered && weight_gathers(gj) && activation_gathers(gi);
+        if (DAB_IN_BOUNDS(to, g.c_extent)) g.C[to] = apply_post(g.post, y, (int)gj, to);
+        if (g.p11 && DAB_IN_BOUNDS(gi * g.ldp + gj, (g.M - 1) * g.ldp + g.N)) g.p11[gi * g.ldp + gj] = p11;
+      }
+    };
+    finish(std::false_type());
+    if (!gathered) finish(std::true_type());
     cluster.sync();  // a member's counts are read until here
     return;
   }
 
   RescaleSide side[TN];
+  bool gathered = true;
 #pragma unroll
   for (int j = 0; j < TN; ++j) {
     const int64_t gj = j0 + b_t * TN + j;
     side[j] = gj < g.N ? weight(gj) : RescaleSide{0.0, 0.0, 0.0};
+    gathered = gathered && (gj >= g.N || weight_gathers(gj));
   }
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
     int64_t gi = i0 + a_t * TM + i;
     if (gi >= g.M) continue;
     const RescaleSide act = activation(gi);
+    gathered = gathered && activation_gathers(gi);
     int64_t base = (gi / g.map.inner) * g.map.outer_stride + (gi % g.map.inner) * g.map.row_stride;
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
@@ -164,6 +175,26 @@ __global__ void __launch_bounds__(GEMM_THREADS) binary_gemm_kernel(const GemmArg
         g.C[base + gj * g.map.col_stride] =
             apply_post(g.post, rescale(p11, side[j], act), (int)gj, base + gj * g.map.col_stride);
       if (g.p11 && DAB_IN_BOUNDS(gi * g.ldp + gj, (g.M - 1) * g.ldp + g.N)) g.p11[gi * g.ldp + gj] = p11;
+    }
+  }
+  if (!gathered) {  // rare: the counts wait in the outputs' own places for a loop that is not unrolled
+    auto place = [&](int64_t gi, int64_t gj) {
+      return (gi / g.map.inner) * g.map.outer_stride + (gi % g.map.inner) * g.map.row_stride + gj * g.map.col_stride;
+    };
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        const int64_t gi = i0 + a_t * TM + i, gj = j0 + b_t * TN + j;
+        if (gi < g.M && gj < g.N && DAB_IN_BOUNDS(place(gi, gj), g.c_extent)) g.C[place(gi, gj)] = __int_as_float(ones[i][j] + 2 * twos[i][j]);
+      }
+#pragma unroll 1
+    for (int t = 0; t < TM * TN; ++t) {
+      const int64_t gi = i0 + a_t * TM + t / TN, gj = j0 + b_t * TN + t % TN;
+      if (gi >= g.M || gj >= g.N) continue;
+      const int64_t to = place(gi, gj);
+      if (DAB_IN_BOUNDS(to, g.c_extent))
+        g.C[to] = apply_post(g.post, rescale_any(g, __float_as_int(g.C[to]), gi, gj), (int)gj, to);
     }
   }
 }

@@ -40,6 +40,7 @@ struct Side {
     const int k = K[DAB_IDX(row, rows)];
     return weights ? rescale_weight(a, b, k, n) : rescale_activation(a, b, k);
   }
+  __device__ __forceinline__ bool gathered(int64_t row) const { return gathers(v1[DAB_IDX(row, rows)], v0[DAB_IDX(row, rows)]); }
 };
 
 // What the epilogue needs of one column-side row: its part of the rescale and of the output offset.
@@ -54,14 +55,34 @@ __device__ __forceinline__ int64_t act_offset(const GemmArgs& g, int64_t i) {
 }
 
 // Outputs of one lane-side row and up to 32 columns from column `first` (counted over the whole matrix) on.  v: their counts.
+// gathered: every one of these rows and the lane's own gathers().
 template <bool kLanesAreActivations, bool kPost>
 __device__ __forceinline__ void store_columns(const GemmArgs& g, uint32_t (&v)[32], int left, const ColumnParams* col, int64_t first,
-                                              int64_t gl, const RescaleSide& lane_side, int64_t off) {
+                                              int64_t gl, const RescaleSide& lane_side, int64_t off, bool gathered) {
   // this row's counts: element (gl, column) when the lanes are activation rows, (column, gl) otherwise
   const int64_t pblock = kLanesAreActivations ? gl * g.ldp + first : first * g.ldp + gl;
   const int64_t pstep = kLanesAreActivations ? 1 : g.ldp;
 #pragma unroll
   for (int jj = 0; jj < 32; ++jj) v[jj] >>= kBitProductLog;
+  if (!gathered) {  // rare: the counts wait in the outputs' own places for a loop that is not unrolled
+#pragma unroll
+    for (int jj = 0; jj < 32; ++jj) {
+      if (jj >= left) break;
+      const int64_t to = off + col[jj].off;
+      if (DAB_IN_BOUNDS(to, g.c_extent)) g.C[to] = __int_as_float((int)v[jj]);
+    }
+    const int count = min(left, 32);
+#pragma unroll 1
+    for (int jj = 0; jj < count; ++jj) {
+      const int64_t to = off + col[jj].off, at = first + jj;
+      if (!DAB_IN_BOUNDS(to, g.c_extent)) continue;
+      const int p11 = __float_as_int(g.C[to]);
+      const float y = kLanesAreActivations ? rescale_any(g, p11, gl, at) : rescale_any(g, p11, at, gl);
+      g.C[to] = kPost ? apply_post(g.post, y, (int)at, to) : y;
+      if (g.p11 && DAB_IN_BOUNDS(pblock + jj * pstep, (g.M - 1) * g.ldp + g.N)) g.p11[pblock + jj * pstep] = p11;
+    }
+    return;
+  }
   if (!kPost && left >= 32 && !g.p11) {  // the usual case
     float* const row = g.C + off;
 #pragma unroll
@@ -160,9 +181,13 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS) binary_gemm_mma_kernel(cons
     mbar_init(bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int j = tid; j < nrows; j += THREADS) s_col[j] = column_params<kLanesAreActivations>(g, S, j0 + j);
+  bool gathered = true;
+  for (int j = tid; j < nrows; j += THREADS) {
+    s_col[j] = column_params<kLanesAreActivations>(g, S, j0 + j);
+    gathered = gathered && S.gathered(j0 + j);
+  }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
+  gathered = __syncthreads_and(gathered);  // of the tile's columns
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = uniform(s_tmem);
   const uint32_t idesc = instr_desc(NT);
@@ -244,12 +269,13 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS) binary_gemm_mma_kernel(cons
     int64_t off = 0;
     if (valid) {
       lane_side = L.rescaled(gl, g.n);
+      gathered = gathered && L.gathered(gl);
       off = kLanesAreActivations ? act_offset(g, gl) : gl * g.map.col_stride;
     }
     for (int cb = warp >> 2; cb * 32 < NT; cb += THREADS / 128) {
       uint32_t v[32];
       tmem_load_32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(cb * 32), v);
-      if (valid) store_columns<kLanesAreActivations, kPost>(g, v, nrows - cb * 32, s_col + cb * 32, j0 + cb * 32, gl, lane_side, off);
+      if (valid) store_columns<kLanesAreActivations, kPost>(g, v, nrows - cb * 32, s_col + cb * 32, j0 + cb * 32, gl, lane_side, off, gathered);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -293,9 +319,13 @@ __global__ void __launch_bounds__(WIDE_THREADS, 2) binary_gemm_wide_kernel(const
     for (int b = 0; b < WIDE_BUFFERS; ++b) mbar_init(bars + 8 * b, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int j = tid; j < nrows; j += WIDE_THREADS) s_col[j] = column_params<kLanesAreActivations>(g, S, j0 + j);
+  bool gathered = true;
+  for (int j = tid; j < nrows; j += WIDE_THREADS) {
+    s_col[j] = column_params<kLanesAreActivations>(g, S, j0 + j);
+    gathered = gathered && S.gathered(j0 + j);
+  }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
+  gathered = __syncthreads_and(gathered);  // of the tile's columns
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = uniform(s_tmem);
   const uint32_t idesc = instr_desc((nrows + 15) & ~15);
@@ -370,13 +400,14 @@ __global__ void __launch_bounds__(WIDE_THREADS, 2) binary_gemm_wide_kernel(const
     int64_t off = 0;
     if (valid) {
       lane_side = L.rescaled(gl, g.n);
+      gathered = gathered && L.gathered(gl);
       off = kLanesAreActivations ? act_offset(g, gl) : gl * g.map.col_stride;
     }
 #pragma unroll 1
     for (int cb = 2 * half; cb < 2 * half + 2 && cb * 32 < nrows && warp < WIDE_WORKERS / 32; ++cb) {
       uint32_t v[32];
       tmem_load_32(tmem + lanes + cb * 32, v);
-      if (valid) store_columns<kLanesAreActivations, kPost>(g, v, nrows - cb * 32, s_col + cb * 32, j0 + cb * 32, gl, lane_side, off);
+      if (valid) store_columns<kLanesAreActivations, kPost>(g, v, nrows - cb * 32, s_col + cb * 32, j0 + cb * 32, gl, lane_side, off, gathered);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
