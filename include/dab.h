@@ -367,13 +367,13 @@ dab_contraction dab_get_contraction(void);
  * in dab_binarize (Section 4.1 / Algorithm 1 per row; every choice gives the same codes bit for bit):
  *   DAB_PATCHES_SORT   every row is sorted in full (its exact zeros are only counted) and every split evaluated;
  *   DAB_PATCHES_PIXEL  patches of 257..8192 values: the values of every input pixel (its C channels) are counted once
- *                      per tile into buckets (ranges of bit patterns), with exact fp64 sums; a patch adds the tables of
- *                      its kh*kw pixels, which gives the split size and prefix sum at every bucket edge exactly.  The
+ *                      per tile into buckets (ranges of bit patterns), with their sums in fp64; a patch adds the tables of
+ *                      its kh*kw pixels, which gives the split size and prefix sum at every bucket edge.  The
  *                      objective is convex in (split size, prefix sum), so inside a bucket it is bounded by its values
  *                      at the corners of the region the bucket's count, sum and value bounds allow; only the few
  *                      buckets whose bound reaches the best edge value are searched exactly.  Work per pixel is
  *                      shared by the up to kh*kw patches that contain it.  Patches it cannot settle (a hull of more
- *                      than 1024 values, a constant row without zeros, magnitudes outside 2^-40..2^40, a NaN or an
+ *                      than 1023 values, a constant row without zeros, magnitudes outside 2^-40..2^40, a NaN or an
  *                      infinity in the tile) are coded by a second kernel, a CTA per patch.  At most 512 channels and 32
  *                      pixels per window;
  *   DAB_PATCHES_HIST   patches of 257..8192 values, one warp each: a histogram of the patch's own values

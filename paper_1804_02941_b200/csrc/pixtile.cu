@@ -6,7 +6,8 @@
 //   grid       value buckets chosen for the tile: one per octave of magnitude and sign, and more where a sample of the tile
 //              says that the best splits lie.  Buckets are ranges of bit patterns, so membership is exact;
 //   tables     per pixel and bucket the cumulative count and the cumulative fp64 sum (from the count and the sum of the
-//              mantissas: 32-bit shared-memory atomics, exact), and the channels in bucket order.
+//              mantissas: 32-bit shared-memory atomics, exact; below the grid's octaves a 64-bit fixed-point sum), and the
+//              channels in bucket order.
 // A patch is then searched by a warp, a lane per bucket:
 //   edges      the tables of its kh*kw pixels are added: split size and prefix sum at every bucket edge, exactly;
 //   prune      the objective is jointly convex in (split size, prefix sum); inside a bucket the pair stays within a
@@ -40,6 +41,9 @@ constexpr int kSampledUnits = 512; // of four values
 // activations: from 3 to 30 resp. 0.03 to 0.2 the coder's time moves by less than 10 %, networks by 20 % (local optima of a patch
 // differ from the tile's: broad is better there).
 constexpr float kSharp = 10.0f, kPrior = 0.2f;
+// Sums of at most 2048 values in 62 bits.  Values down to 2^-27 of the lowest resolved octave are exact; what smaller ones lose is
+// below the rounding of an fp64 sum with any resolved value in it, and patches without one are left to the other kernel.
+constexpr int kTinyBits = 51;
 constexpr int kHullCap = 1024;     // values the search of one patch takes at most
 // A bucket is kept if its bound reaches the best edge objective times this: edges and inner corners are formed in fp32 from
 // sums rounded once (1e-6 relative), the place of a corner to 4e-7 of the bucket's count.
@@ -499,6 +503,13 @@ __device__ __forceinline__ PatchCode search_patch(const TileArgs& a, const Grid&
   }
   const int size = c_end - c_lo, s_lo = c_lo + (seg_lo > B0 ? z : 0);
   if (size < 1 || size > kHullCap - 1 || (z == 0 && size == n)) return code;
+  if (b_lo >= B0 - 1 && b_end <= B0 + 1) {  // the two buckets next to zero: does the patch have no other values?
+    int below, upto;
+    double unused;
+    state_at(B0 - 1, below, unused);
+    state_at(B0 + 1, upto, unused);
+    if (upto - below == m) return code;
+  }
   // ---- their values, from the lists of the window's pixels ----
   int begin = 0, incl = 0;
   if (lane < wn) {
@@ -550,7 +561,9 @@ __global__ void __launch_bounds__(kTileThreads, 2) binarize_patches_tile_kernel(
   // dead once the patches are searched; the assembled masks then take their place
   double* const sums = reinterpret_cast<double*>(smem_raw);                       // [bucket][slot] cumulative sums ...
   uint32_t* const cells = reinterpret_cast<uint32_t*>(smem_raw);                  // ... in place of (count, sum of the mantissas)
-  double* const tiny = sums + (size_t)BUCKETS * slots;                            // [2][slot] sums of what the grid does not resolve
+  // [2][slot] sums of what the grid does not resolve: in units of 2^-kTinyBits of its lowest octave, so that they are the same
+  // whatever the order (an atomic fp64 sum rounds as the order falls)
+  unsigned long long* const tiny = reinterpret_cast<unsigned long long*>(sums + (size_t)BUCKETS * slots);
   uint16_t* const counts = reinterpret_cast<uint16_t*>(tiny + 2 * slots);         // [bucket][slot] cumulative counts
   ListT* const list = reinterpret_cast<ListT*>(counts + (size_t)BUCKETS * slots);  // [slot][4 * quads] channels by bucket
   // kept
@@ -632,7 +645,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) binarize_patches_tile_kernel(
   }
 
   if (top != 0u) {
-    // ---- the grid, from about a thousand values spread over the tile ----
+    // ---- the grid, from about two thousand values spread over the tile ----
     {
       const int side = a.octaves * kCells + 1, base = (((int)(top >> 23) - a.octaves + 1) << kCellBits) - 1;
       const int samples = min(units, kSampledUnits), step = units / samples;
@@ -651,6 +664,9 @@ __global__ void __launch_bounds__(kTileThreads, 2) binarize_patches_tile_kernel(
     }
     const int nb = grid.nb, B0 = grid.B0, base = grid.base, side = grid.side;
     const bool negatives = grid.signs & 1;
+    const int low = (int)(top >> 23) - 127 - a.octaves + 1;  // 2^low: what the unresolved values stay below
+    const float tiny_scale = __int_as_float((127 + kTinyBits - low) << 23);
+    const double tiny_unit = __hiloint2double((1023 + low - kTinyBits) << 20, 0);
     // ---- per pixel: count and sum of the mantissas per bucket ----
 #pragma unroll 2
     for (int u = tid; u < units; u += THREADS) {
@@ -664,7 +680,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) binarize_patches_tile_kernel(
           const int c = grid_step(m, base, side), slot = grid_bucket(grid, v[j], c, side) * slots + p;
           atomicAdd(&cells[2 * slot], 1u);
           if (c > 0) atomicAdd(&cells[2 * slot + 1], m & 0x7FFFFFu);
-          else atomicAdd(&tiny[(v[j] < 0.0f ? 0 : slots) + p], (double)v[j]);
+          else atomicAdd(&tiny[(v[j] < 0.0f ? 0 : slots) + p], (unsigned long long)__float2ll_rn(__fmul_rn(v[j], tiny_scale)));
         }
       }
     }
@@ -673,7 +689,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) binarize_patches_tile_kernel(
     for (int p = tid; p <= pixels; p += THREADS) {
       int run = 0;
       double sum = 0.0;
-      const double inner_neg = tiny[p], inner_pos = tiny[slots + p];
+      const double inner_neg = __dmul_rn((double)(long long)tiny[p], tiny_unit), inner_pos = __dmul_rn((double)(long long)tiny[slots + p], tiny_unit);
 #pragma unroll 4
       for (int b = 0; b < BUCKETS; ++b) {  // (the buckets beyond nb are empty)
         const uint2 cell = *reinterpret_cast<const uint2*>(cells + 2 * (b * slots + p));
