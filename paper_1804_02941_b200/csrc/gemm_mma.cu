@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS) binary_gemm_mma_kernel(cons
       mma_commit(bar);
     }
   }
-  mbar_wait(bar, parity, dead, &g_mma_wait_timeouts);  // the last commit covers every instruction issued before it
+  mbar_wait_last(bar, parity, dead, &g_mma_wait_timeouts);  // the last commit covers every instruction issued before it
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
   // Epilogue: thread = lane-side row (a warp reads the 32 lanes of its quarter), 32 columns at a time.
@@ -388,11 +388,11 @@ __global__ void __launch_bounds__(WIDE_THREADS, 2) binary_gemm_wide_kernel(const
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy stores -> tensor-core reads
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      bar_arrive(1 + buffer, WIDE_THREADS);  // (the buffer's next use waits for the products, which wait for this barrier)
+      stage_handover(1 + buffer, WIDE_THREADS, dead);  // (the buffer's next use waits for the products, which wait for this barrier)
     }
   }
   // the last commit covers every instruction issued before it
-  mbar_wait(bars + 8 * ((chunks - 1) % WIDE_BUFFERS), (uint32_t)((chunks - 1) / WIDE_BUFFERS) & 1u, dead, &g_mma_wait_timeouts);
+  mbar_wait_last(bars + 8 * ((chunks - 1) % WIDE_BUFFERS), (uint32_t)((chunks - 1) / WIDE_BUFFERS) & 1u, dead, &g_mma_wait_timeouts);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   {
     const bool valid = row_in && !dead && warp < WIDE_WORKERS / 32;

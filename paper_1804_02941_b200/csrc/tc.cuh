@@ -68,6 +68,22 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, bool& d
   }
 }
 
+// The wait for the last commit before tensor memory is given back: with a limit of its own, also after an earlier wait ran out.
+__device__ __forceinline__ void mbar_wait_last(uint32_t bar, uint32_t parity, bool& dead, unsigned int* failures,
+                                               long long limit = kWaitCycles) {
+  bool late = false;
+  mbar_wait(bar, parity, late, failures, limit);
+  dead = dead || late;
+}
+
+// A producer warp hands a stage to the warp that issues the products (which takes it with bar_sync).  It does not block: the wait
+// for the buffer's next use keeps the two in step.  A producer whose waits no longer hold (dead) waits here instead: running
+// ahead, it would arrive twice in one phase, and the issuing warp would wait for arrivals that have been spent.
+__device__ __forceinline__ void stage_handover(int id, int threads, bool dead) {
+  if (__any_sync(0xFFFFFFFFu, dead)) bar_sync(id, threads);
+  else bar_arrive(id, threads);
+}
+
 // The operands of an instruction live in uniform registers.  Issued under a branch on the thread, with operands the compiler
 // cannot tell are the warp's, one took 175 cycles to issue, whatever it multiplied (128 x 128 x 32: 64 cycles of tensor-core
 // time).  So: a warp's number and the tensor-memory address go through uniform(), the loops over instructions are unrolled,

@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
   __syncthreads();
   if (warp == 0 && elect_one()) multiply(stages - 1);
   // the last commit covers every instruction before it
-  mbar_wait((stages - 1) & 1 ? bar1 : bar0, (uint32_t)((stages - 1) >> 1) & 1u, dead, &g_wbin_wait_timeouts);
+  mbar_wait_last((stages - 1) & 1 ? bar1 : bar0, (uint32_t)((stages - 1) >> 1) & 1u, dead, &g_wbin_wait_timeouts);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   rowsum[tid] = make_int4(psum[0], psum[1], psum[2], psum[3]);  // (a wait that ran out stores nothing to y)
   __syncthreads();

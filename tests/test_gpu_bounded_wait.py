@@ -29,6 +29,8 @@ def probe(tmp_path_factory):
     lib = C.CDLL(out)
     lib.run_wait_timeout.argtypes = [C.c_longlong, C.c_int, C.c_void_p, C.c_void_p]
     lib.run_wait_timeout.restype = C.c_int
+    lib.run_handover_timeout.argtypes = [C.c_int, C.c_int, C.c_longlong, C.c_void_p, C.c_void_p]
+    lib.run_handover_timeout.restype = C.c_int
     return lib
 
 
@@ -43,6 +45,18 @@ def test_a_wait_that_nothing_ends_runs_out_and_is_counted(probe, threads):
     assert out.cpu().tolist() == [0, 0, 1, 1]              # both waits failed, the first only after the limit
     assert int(failures.item()) == threads                 # one count per waiting thread, none for the second wait
     assert float((torch.ones(8, device="cuda") * 2).sum().item()) == 16.0
+
+
+@pytest.mark.parametrize("warps,stages", [(1, 9), (8, 3), (8, 40)])
+def test_producers_whose_waits_ran_out_stay_in_step_with_the_issuing_warp(probe, warps, stages):
+    torch.cuda.init()
+    failures = torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = torch.full((stages,), -1, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    rc = probe.run_handover_timeout(warps, stages, 20000, C.c_void_p(failures.data_ptr()), C.c_void_p(out.data_ptr()))
+    assert rc == 0
+    assert out.cpu().tolist() == [warps] * stages
+    assert int(failures.item()) == 32 * warps
 
 
 def test_the_library_kernels_report_no_wait_that_ran_out():
