@@ -435,7 +435,7 @@ size_t set_tile(WbinArgs* a, int tw, int R, int nt, int js) {
   const int64_t all_rows = (int64_t)d.N * a->Ho;
   const int64_t rows = std::min<int64_t>(a->R % a->TW == 0 ? a->R / a->TW : (a->R + 2 * a->TW - 2) / a->TW, all_rows);
   const int64_t images = std::min<int64_t>(1 + (rows - 1 + a->Ho - 1) / a->Ho, d.N);
-  const int64_t staged = rows * d.stride_h + images * std::max(0, d.kh - d.stride_h);
+  const int64_t staged = rows * d.stride_h + (d.kh > d.stride_h ? images : 1) * (d.kh - d.stride_h);  // (rows between windows are not)
   a->max_ch = std::min(d.C, (js * 32 + a->khw - 2) / a->khw + 1);
   if (staged * a->pitch > 1 << 20 || images * d.C * d.H * d.W > 0x7FFFFFFF) return SIZE_MAX;  // (32-bit places)
   a->ch_words = (int)(staged * a->pitch);
