@@ -3,10 +3,10 @@
 //
 //   y[p][co] = alpha_co * M1 + beta_co * (S - M1),   M1 = sum_{i: e_co[i] = 1} x_p[i],   S = sum_i x_p[i]
 //
-// M1 is a dense contraction of the patch matrix with the 0/1 filter masks.  It is formed exactly in integers:
+// M1 is a dense contraction of the patch matrix with the 0/1 filter masks (stored as 0 / -1 bytes).  It is formed exactly in integers:
 // every patch row is written as 32-bit fixed point relative to its own largest magnitude
 // (q_i = rint(x_i * 2^sexp), |q_i| < 2^31), q is split into its four bytes (three unsigned, the top one
-// signed), and four tcgen05.mma kind::i8 products with the masks expanded to 0/1 bytes give four 32-bit
+// signed), and four tcgen05.mma kind::i8 products with the masks expanded to 0 / -1 bytes give four negated 32-bit
 // accumulators per output in tensor memory; M1 = a3 2^24 + a2 2^16 + a1 2^8 + a0 (times 2^-sexp).  The only
 // error is the rounding of x_i to q_i: at most 2^-32 of the row's largest magnitude per element.
 //
@@ -15,7 +15,8 @@
 // whatever the image size.  Patches are never formed in global memory: for each group of JS mask words (32 JS patch elements)
 // the CTA stages the channels they come from in shared memory, and every thread gathers 16 elements of its row at a time,
 // converts them and stores one 16-byte K chunk per byte plane in the operand layout of tc.cuh.  Both the staged channels and
-// the operands are double-buffered: while the tensor cores work on one stage the threads convert the next.
+// the operands are double-buffered: while the tensor cores work on one stage the threads convert the next.  (Where two CTAs share an
+// SM, or a wide window leaves no room, the operands are not: see launch_wbin_conv.)
 //
 // Bound by shared memory: per stage of 128 elements and 128 filters the tensor cores read 128 KB of operands, the gather
 // 64 KB of values (twice where lanes of a warp lie in different output rows) and writes 64 KB.  The conversion, some 8
@@ -33,8 +34,6 @@ using namespace tc;
 
 __device__ unsigned int g_wbin_wait_timeouts;
 
-constexpr int WB_THREADS = 512;
-
 struct WbinArgs {
   dab_conv_desc d;
   int32_t Ho, Wo, n, words, khw;
@@ -51,6 +50,11 @@ struct WbinArgs {
   const float* wbeta;
   float* y;
 };
+
+// a / b, both positive; a 64-bit division (some 100 instructions) only where it takes one.
+__device__ __forceinline__ int64_t quotient(int64_t a, int b) {
+  return a >> 32 ? a / b : (int64_t)((uint32_t)a / (uint32_t)b);
+}
 
 __device__ __forceinline__ int fast_div(int i, uint32_t magic) {
   return magic ? (int)__umulhi((unsigned)i, magic) : i;
@@ -105,8 +109,8 @@ __device__ __forceinline__ void gather_chunk(const unsigned char* src, const int
     *reinterpret_cast<uint4*>(dst + p * kPlane) = make_uint4(pl[p][0], pl[p][1], pl[p][2], pl[p][3]);
 }
 
-// Bytes of shared memory for the operands of one stage.
-constexpr size_t operand_bytes(int nt, int js) { return (size_t)(4 * kLanes + nt) * js * 32; }
+// Bytes of shared memory for the operands.
+constexpr size_t operand_bytes(int nt, int js, int buffers) { return (size_t)buffers * (4 * kLanes + nt) * js * 32; }
 
 // The rows of input under a tile are staged one after another, those of an image together.  Row of output row `g` (counted
 // over all images) in the staging area, and what a staged row holds.
@@ -114,7 +118,7 @@ struct TileRows {
   int64_t img0;
   int ho0, first, full, stride, Ho;  // rows staged for the first image (at most) and for a whole one
   __device__ __forceinline__ TileRows(const WbinArgs& a, int64_t g0) : stride(a.d.stride_h), Ho(a.Ho) {
-    img0 = g0 / a.Ho;
+    img0 = quotient(g0, a.Ho);
     ho0 = (int)(g0 - img0 * a.Ho);
     first = (a.Ho - 1 - ho0) * stride + a.d.kh;
     full = (a.Ho - 1) * stride + a.d.kh;
@@ -131,13 +135,15 @@ struct TileRows {
   }
 };
 
-template <int NT, int JS>
-__global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs a) {
+// THREADS 512: a CTA has the SM to itself; 256 (of 64 filters): two CTAs share it.  BUFFERS: operand stages, 1 or 2.
+template <int NT, int JS, int THREADS, int BUFFERS>
+__global__ void __launch_bounds__(THREADS, 512 / THREADS) wbin_conv_kernel(const WbinArgs a) {
   constexpr int KS = JS * 32, KC = JS * 2;        // patch elements and 16-byte K chunks per stage
   constexpr uint32_t SBO = KC * 128;              // bytes between groups of 8 rows
   constexpr uint32_t PLANE = kLanes * KS;         // bytes of one byte plane of the activations
   constexpr uint32_t STAGE = 4 * PLANE + NT * KS;
-  static_assert(NT * JS <= WB_THREADS, "a mask word per thread and stage");
+  constexpr int SHARE = NT / (THREADS / 128);     // filters per group of four warps in the epilogue
+  static_assert(NT * JS <= THREADS, "a mask word per thread and stage");
   extern __shared__ __align__(128) unsigned char dyn_mem[];
   __shared__ __align__(8) uint64_t s_bar[2];
   __shared__ uint32_t s_tmem;
@@ -149,7 +155,7 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
   const uint32_t mem0 = (smem_u32(dyn_mem) + 127u) & ~127u;
   unsigned char* const operands = dyn_mem + (mem0 - smem_u32(dyn_mem));
   const int tile_words = a.max_ch * a.ch_words;
-  float* const tiles = reinterpret_cast<float*>(operands + 2 * STAGE);
+  float* const tiles = reinterpret_cast<float*>(operands + BUFFERS * STAGE);
   int32_t* const goff = reinterpret_cast<int32_t*>(tiles + 2 * (size_t)tile_words);  // [pixel] place in x; -1: outside
   uint32_t* const pixmax = reinterpret_cast<uint32_t*>(tiles);                        // [pixel]; until channels are staged
   int4* const rowsum = reinterpret_cast<int4*>(operands);  // [thread] byte-plane sums of q over its part of the row; at the end
@@ -159,7 +165,7 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
   const int strip = blockIdx.x % a.strips, wo0 = strip * a.TW;
   const int64_t f0 = (int64_t)(blockIdx.x / a.strips) * a.R, total = (int64_t)a.d.N * a.Ho * a.TW;
   const int rows = (int)min((int64_t)a.R, total - f0);
-  const int64_t g0 = f0 / a.TW;
+  const int64_t g0 = quotient(f0, a.TW);
   const int lead = (int)(f0 - g0 * a.TW);  // positions of the first output row before the tile
   const TileRows map(a, g0);
   const int w0 = wo0 * a.d.stride_w - a.d.pad_w;
@@ -179,13 +185,13 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
     mbar_init(bar1, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int j = tid; j < NT; j += WB_THREADS) {
+  for (int j = tid; j < NT; j += THREADS) {
     const bool in = j0 + j < a.d.Cout;
     s_alpha[j] = in ? (double)a.walpha[j0 + j] : 0.0;
     s_beta[j] = in ? (double)a.wbeta[j0 + j] : 0.0;
   }
   // where the staged words come from, and the per-pixel maxima (0 outside the image)
-  for (int i = tid; i < pixels; i += WB_THREADS) {
+  for (int i = tid; i < pixels; i += THREADS) {
     const int q = i / a.pitch, s = i - q * a.pitch, w = w0 + s;
     int di, h;
     map.source(q, di, h);
@@ -197,7 +203,7 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
   __syncthreads();
 
   // Row = output position; its scale comes from the largest magnitude of its patch.
-  const int slots = a.row_slots, groups = WB_THREADS / slots;
+  const int slots = a.row_slots, groups = THREADS / slots;
   auto locate = [&](int r, int64_t& img, int& ho, int& lw) {  // returns the first staged word of the row's window
     const int dg = (lead + r) / a.TW;
     lw = lead + r - dg * a.TW;
@@ -238,14 +244,14 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
   const int stages = (a.words + JS - 1) / JS;
   // Asynchronous copy of the channels that stage `st` draws from into tile buffer st & 1, and the offsets of its
   // elements inside that tile.  A thread keeps to one pixel where there are few.
-  const int copies = max(1, WB_THREADS / pixels);
+  const int copies = max(1, THREADS / pixels);
   const int pix0 = copies > 1 ? tid % pixels : tid, c_first = copies > 1 ? tid / pixels : 0;
   auto stage_in = [&](int st) {
     const int k0 = st * KS, k1 = min(a.n, k0 + KS);
     const int c_lo = fast_div(k0, a.magic_khw), nch = fast_div(k1 - 1, a.magic_khw) + 1 - c_lo;
     float* const tile = tiles + (st & 1) * tile_words;
     if (c_first < copies)
-      for (int i = pix0; i < pixels; i += copies > 1 ? pixels : WB_THREADS) {
+      for (int i = pix0; i < pixels; i += copies > 1 ? pixels : THREADS) {
         const int at = goff[i];
         const float* src = at >= 0 ? x0 + at + (int64_t)(c_lo + c_first) * plane_in : x0;
         const int64_t step = at >= 0 ? (int64_t)copies * plane_in : 0;
@@ -279,7 +285,7 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
   const uint32_t idesc_u = instr_desc(NT, false, true), idesc_s = instr_desc(NT, true, true);
   auto multiply = [&](int st) {  // (one thread) the products of stage `st`
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint64_t da = smem_desc(mem0 + (st & 1) * STAGE, 128, SBO), db = desc_at(da, 4 * PLANE);
+    const uint64_t da = smem_desc(mem0 + st % BUFFERS * STAGE, 128, SBO), db = desc_at(da, 4 * PLANE);
     const int kw = min(JS, a.words - st * JS);
 #pragma unroll
     for (int t = 0; t < JS; ++t)
@@ -288,7 +294,7 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
         for (int p = 0; p < 4; ++p)
           mma_i8(tmem + (uint32_t)(p * NT), desc_at(da, p * PLANE + t * 256), desc_at(db, t * 256), p == 3 ? idesc_s : idesc_u,
                  (st | t) != 0);
-    mma_commit(st & 1 ? bar1 : bar0);
+    mma_commit(st % BUFFERS ? bar1 : bar0);
   };
 
   int psum[4] = {0, 0, 0, 0};
@@ -306,9 +312,9 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
       stage_in(st + 1);
       next_mask = load_mask(st + 1);
     }
-    // the tensor cores have finished reading what these buffers held two stages ago
-    if (st > 1) mbar_wait(st & 1 ? bar1 : bar0, (uint32_t)((st >> 1) - 1) & 1u, dead, &g_wbin_wait_timeouts);
-    unsigned char* const stage_a = operands + (st & 1) * STAGE;
+    // the tensor cores have finished reading what these buffers held before
+    if (st >= BUFFERS) mbar_wait(st % BUFFERS ? bar1 : bar0, (uint32_t)(st / BUFFERS - 1) & 1u, dead, &g_wbin_wait_timeouts);
+    unsigned char* const stage_a = operands + st % BUFFERS * STAGE;
     if (gather) {
       const unsigned char* const src = reinterpret_cast<const unsigned char*>(tiles + (st & 1) * tile_words + origin);
       const int32_t* const off = s_off[st & 1];
@@ -327,12 +333,12 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
   __syncthreads();
   if (warp == 0 && elect_one()) multiply(stages - 1);
   // the last commit covers every instruction before it
-  mbar_wait_last((stages - 1) & 1 ? bar1 : bar0, (uint32_t)((stages - 1) >> 1) & 1u, dead, &g_wbin_wait_timeouts);
+  mbar_wait_last((stages - 1) % BUFFERS ? bar1 : bar0, (uint32_t)((stages - 1) / BUFFERS) & 1u, dead, &g_wbin_wait_timeouts);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   rowsum[tid] = make_int4(psum[0], psum[1], psum[2], psum[3]);  // (a wait that ran out stores nothing to y)
   __syncthreads();
 
-  // Epilogue: thread = row (a warp reads the 32 lanes of its quarter), a quarter of the filters per four warps.
+  // Epilogue: thread = row (a warp reads the 32 lanes of its quarter), an equal share of the filters per four warps.
   // The filter bytes are 0 / -1: the accumulators hold the negative sums.
   {
     const int erow = (warp & 3) * 32 + lane;
@@ -362,8 +368,8 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
     const int64_t plane_hw = (int64_t)a.Ho * a.Wo;
     static_assert(DAB_MAX_N <= (1 << 14), "255 * 257 * n must stay below 2^31");
 #pragma unroll 1
-    for (int c8 = 0; c8 < NT / 32; ++c8) {
-      const int col = (warp >> 2) * (NT / 4) + c8 * 8;
+    for (int c8 = 0; c8 < SHARE / 8; ++c8) {
+      const int col = (warp >> 2) * SHARE + c8 * 8;
       uint32_t v[4][8];
       const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col;
 #pragma unroll
@@ -394,36 +400,48 @@ __global__ void __launch_bounds__(WB_THREADS, 1) wbin_conv_kernel(const WbinArgs
 }
 
 // Largest magnitude over the channels of every pixel, as a bit pattern (NaN > Inf > finite): what the
-// convolution kernel derives the scale of a patch from.  A CTA takes 32 pixels, its warps a share of the channels each: bound
-// by the one read of x (a thread per pixel had too few loads in flight: 35 us for 51 MB).
+// convolution kernel derives the scale of a patch from.  SHARES warps take a share of the channels of 32 pixels each: bound by
+// the one read of x (with a thread per pixel too few loads are in flight where there are many channels: 35 us for 51 MB; with
+// eight shares of three channels most warps have nothing to do).
 constexpr int PM_WARPS = 8;
+template <int SHARES>
 __global__ void __launch_bounds__(32 * PM_WARPS) wbin_pixmax_kernel(const float* __restrict__ x, uint32_t* __restrict__ out,
-                                                                    int C, int64_t HW, int64_t total) {
+                                                                    int C, int HW, int64_t total) {
   __shared__ uint32_t part[PM_WARPS][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t idx = (int64_t)blockIdx.x * 32 + lane;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, share = warp % SHARES;
+  const int64_t idx = ((int64_t)blockIdx.x * (PM_WARPS / SHARES) + warp / SHARES) * 32 + lane;
   uint32_t m = 0u;
   if (idx < total) {
-    const int64_t img = idx / HW, p = idx - img * HW;
-    const float* src = x + img * C * HW + p;
+    const int64_t img = quotient(idx, HW), p = idx - img * HW;
+    const float* src = x + img * C * (int64_t)HW + p;
 #pragma unroll 8
-    for (int c = warp; c < C; c += PM_WARPS) m = max(m, __float_as_uint(__ldg(src + (int64_t)c * HW)) & 0x7FFFFFFFu);
+    for (int c = share; c < C; c += SHARES) m = max(m, __float_as_uint(__ldg(src + (int64_t)c * HW)) & 0x7FFFFFFFu);
   }
-  part[warp][lane] = m;
-  __syncthreads();
-  if (warp == 0 && idx < total) {
+  if (SHARES > 1) {
+    part[warp][lane] = m;
+    __syncthreads();
 #pragma unroll
-    for (int w = 1; w < PM_WARPS; ++w) m = max(m, part[w][lane]);
-    out[idx] = m;
+    for (int w = 1; w < SHARES; ++w)
+      if (share == 0) m = max(m, part[warp + w][lane]);
   }
+  if (share == 0 && idx < total) out[idx] = m;
+}
+
+template <int SHARES>
+cudaError_t launch_pixmax(const float* x, uint32_t* out, int C, int HW, int64_t total, cudaStream_t stream) {
+  const int64_t blocks = (total + 32 * PM_WARPS / SHARES - 1) / (32 * PM_WARPS / SHARES);
+  if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
+  wbin_pixmax_kernel<SHARES><<<(unsigned)blocks, 32 * PM_WARPS, 0, stream>>>(x, out, C, HW, total);
+  return cudaGetLastError();
 }
 
 uint32_t magic_for(uint32_t d) { return d > 1 ? (uint32_t)((0x100000000ull + d - 1) / d) : 0u; }
 
 constexpr size_t kSmemLimit = 227 * 1024 - 5 * 1024;  // (static shared memory aside)
+constexpr size_t kSmemLimitOfTwo = 113 * 1024 - 3 * 1024;
 
 // Sets the tile: strips of at most `tw` columns, R positions.  Returns the shared memory it takes with operands of the given size.
-size_t set_tile(WbinArgs* a, int tw, int R, int nt, int js) {
+size_t set_tile(WbinArgs* a, int tw, int R, int nt, int js, int buffers) {
   const dab_conv_desc& d = a->d;
   a->strips = (a->Wo + tw - 1) / tw;
   a->TW = (a->Wo + a->strips - 1) / a->strips;
@@ -439,16 +457,16 @@ size_t set_tile(WbinArgs* a, int tw, int R, int nt, int js) {
   a->max_ch = std::min(d.C, (js * 32 + a->khw - 2) / a->khw + 1);
   if (staged * a->pitch > 1 << 20 || images * d.C * d.H * d.W > 0x7FFFFFFF) return SIZE_MAX;  // (32-bit places)
   a->ch_words = (int)(staged * a->pitch);
-  return 128 + 2 * operand_bytes(nt, js) + sizeof(float) * (2 * (size_t)a->max_ch + 1) * a->ch_words;
+  return 128 + operand_bytes(nt, js, buffers) + sizeof(float) * (2 * (size_t)a->max_ch + 1) * a->ch_words;
 }
 
-template <int NT, int JS>
+template <int NT, int JS, int THREADS, int BUFFERS>
 cudaError_t launch_tiles(const WbinArgs& a, size_t smem, cudaStream_t stream) {
   const int64_t gx = ((int64_t)a.d.N * a.Ho * a.TW + a.R - 1) / a.R * a.strips, gy = (a.d.Cout + NT - 1) / NT;
   if (gx > 0x7FFFFFFF || gy > 65535) return cudaErrorInvalidValue;
-  cudaError_t e = ensure_dynamic_smem(wbin_conv_kernel<NT, JS>, smem);
+  cudaError_t e = ensure_dynamic_smem(wbin_conv_kernel<NT, JS, THREADS, BUFFERS>, smem);
   if (e != cudaSuccess) return e;
-  wbin_conv_kernel<NT, JS><<<dim3((unsigned)gx, (unsigned)gy), WB_THREADS, smem, stream>>>(a);
+  wbin_conv_kernel<NT, JS, THREADS, BUFFERS><<<dim3((unsigned)gx, (unsigned)gy), THREADS, smem, stream>>>(a);
   return cudaGetLastError();
 }
 
@@ -471,28 +489,46 @@ cudaError_t launch_wbin_conv(const dab_conv_desc& d, int32_t Ho, int32_t Wo, con
   const int64_t positions = (int64_t)d.N * Ho * Wo, sms = sm_count();
   int nt = d.Cout > 64 && (positions + 127) / 128 * ((d.Cout + 127) / 128) >= sms ? 128 : 64;
   const int rows = (positions + 63) / 64 * ((d.Cout + nt - 1) / nt) <= sms ? 64 : kLanes;
-  // Stages of 128 elements where shared memory allows, else of 64; the fewest strips, then the most rows that fit.
-  int js = 0;
+  // The tile: the fewest strips, then the most rows that fit.  Tiles of 64 filters beyond the first wave go to CTAs of half the
+  // threads with one operand stage where 128 rows fit, two on an SM: short rows are mostly set-up, and one CTA's covers the other's.
+  // Measured, 512 threads and two stages -> this: 64 x 3 x 224 x 224 (27 elements, 64 filters) 1356 -> 806 us, 64 x 32 x 112 x 112
+  // (288, 32) 574 -> 392, 64 x 64 x 56 x 56 (576, 64) 198 -> 160, 64 x 64 x 28 x 28 7 x 7 (3136, 64) 170 -> 152; within the first
+  // wave 196 positions of 2304 elements, 64 filters 39 -> 51.  Rows of up to 96 elements, which are
+  // one stage, go there with more than 64 filters too: 3 x 2 x 141 x 141 1 x 1 (2, 177) 62 -> 45.
+  // All others: two stages of 128 elements, else of 64; for 64 filters and windows that reach over two channels at most whatever the
+  // stage, one of 128 instead: 16 x 2 x 80 x 80 31 x 31 104 -> 79 us, 64 x 1 x 120 x 120 64 x 64 1142 -> 770.
+  struct { int nt, js, buffers, threads; } form = {0, 0, 0, 0};
   size_t smem = 0;
-  auto fits = [&](int tw, int R, int stage_words) {
-    smem = set_tile(&a, tw, R, nt, stage_words);
-    if (smem <= kSmemLimit) js = stage_words;
-    return js != 0;
+  auto fits = [&](int tw, int R, int js, int buffers, int threads) {
+    smem = set_tile(&a, tw, R, nt, js, buffers);
+    if (smem <= (threads == 512 ? kSmemLimit : kSmemLimitOfTwo)) form = {nt, js, buffers, threads};
+    return form.nt != 0;
   };
-  for (;; nt = 64) {
-    for (int tw = 32; tw >= 1 && !js; tw >>= 1)
-      for (int R = rows; R >= (tw > 1 ? rows / 2 : 1) && !js; R -= R > 16 ? 16 : 1) fits(tw, R, 4) || fits(tw, R, 2);
-    if (js || nt == 64) break;
+  const int filters = nt;
+  if ((nt == 64 || a.n <= 96) && (positions + 127) / 128 * ((d.Cout + 63) / 64) > sms) {
+    nt = 64;
+    for (int tw = 32; tw >= 8 && !form.nt; tw >>= 1) fits(tw, kLanes, 4, 1, 256);
+    if (!form.nt) nt = filters;
   }
-  if (!js) return cudaErrorInvalidValue;
+  for (;; nt = 64) {
+    for (int tw = 32; tw >= 1 && !form.nt; tw >>= 1)
+      for (int R = rows; R >= (tw > 1 ? rows / 2 : 1) && !form.nt; R -= R > 16 ? 16 : 1)
+        fits(tw, R, 4, 2, 512) || (nt == 64 && a.khw >= 128 ? fits(tw, R, 4, 1, 512) : fits(tw, R, 2, 2, 512));
+    if (form.nt || nt == 64) break;
+  }
+  if (!form.nt) return cudaErrorInvalidValue;
   a.row_slots = a.R <= 64 ? 64 : kLanes;
-  const int64_t HW = (int64_t)d.H * d.W, pixels = (int64_t)d.N * HW;
-  if ((pixels + 31) / 32 > 0x7FFFFFFF) return cudaErrorInvalidValue;
-  wbin_pixmax_kernel<<<(unsigned)((pixels + 31) / 32), 32 * PM_WARPS, 0, stream>>>(x, pixmax, d.C, HW, pixels);
-  cudaError_t e = cudaGetLastError();
+  // A thread per pixel where those fill the device or there is little to share.  Eight shares against it: 64 x 3 x 224 x 224 890 and
+  // 806 us for the whole call, 64 x 64 x 56 x 56 167 and 160, 64 x 128 x 28 x 28 82 and 82, 64 x 256 x 14 x 14 54 and 57.
+  const int HW = d.H * d.W;  // (C * H * W is below 2^31)
+  const int64_t pixels = (int64_t)d.N * HW;
+  cudaError_t e = d.C <= 4 || pixels > 1 << 16 ? launch_pixmax<1>(x, pixmax, d.C, HW, pixels, stream)
+                                                : launch_pixmax<8>(x, pixmax, d.C, HW, pixels, stream);
   if (e != cudaSuccess) return e;
-  if (nt == 128) return js == 4 ? launch_tiles<128, 4>(a, smem, stream) : launch_tiles<128, 2>(a, smem, stream);
-  return js == 4 ? launch_tiles<64, 4>(a, smem, stream) : launch_tiles<64, 2>(a, smem, stream);
+  if (form.threads == 256) return launch_tiles<64, 4, 256, 1>(a, smem, stream);
+  if (form.nt == 128) return form.js == 4 ? launch_tiles<128, 4, 512, 2>(a, smem, stream) : launch_tiles<128, 2, 512, 2>(a, smem, stream);
+  if (form.js == 2) return launch_tiles<64, 2, 512, 2>(a, smem, stream);
+  return form.buffers == 2 ? launch_tiles<64, 4, 512, 2>(a, smem, stream) : launch_tiles<64, 4, 512, 1>(a, smem, stream);
 }
 
 cudaError_t read_wbin_wait_timeouts(unsigned int* count) {
