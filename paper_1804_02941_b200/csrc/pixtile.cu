@@ -44,6 +44,9 @@ constexpr float kSharp = 10.0f, kPrior = 0.2f;
 // Sums of at most 2048 values in 62 bits.  Values down to 2^-27 of the lowest resolved octave are exact; what smaller ones lose is
 // below the rounding of an fp64 sum with any resolved value in it, and patches without one are left to the other kernel.
 constexpr int kTinyBits = 51;
+// From this many pixels on a thread sums a pixel's buckets one after another; below it would leave most of them idle (4200 cycles for
+// 20 pixels where a warp per pixel takes 1500; at 100 pixels both take 5000, at 130 the warps 7000 to 10000).
+constexpr int kSerialPixels = 80;
 constexpr int kHullCap = 1024;     // values the search of one patch takes at most
 // A bucket is kept if its bound reaches the best edge objective times this: edges and inner corners are formed in fp32 from
 // sums rounded once (1e-6 relative), the place of a corner to 4e-7 of the bucket's count.
@@ -685,21 +688,49 @@ __global__ void __launch_bounds__(kTileThreads, 2) binarize_patches_tile_kernel(
       }
     }
     __syncthreads();
-    // ---- per pixel (a thread each): exclusive cumulative counts, inclusive cumulative sums ----
-    for (int p = tid; p <= pixels; p += THREADS) {
-      int run = 0;
-      double sum = 0.0;
-      const double inner_neg = __dmul_rn((double)(long long)tiny[p], tiny_unit), inner_pos = __dmul_rn((double)(long long)tiny[slots + p], tiny_unit);
+    // ---- per pixel: exclusive cumulative counts, inclusive cumulative sums ----
+    if (pixels < kSerialPixels) {  // a warp each, a lane per bucket
+      for (int p = warp; p <= pixels; p += WARPS) {
+        int run = 0;
+        double sum = 0.0;
+#pragma unroll
+        for (int j = 0; j < BPL; ++j) {
+          const int b = 32 * j + lane;
+          const uint2 cell = *reinterpret_cast<const uint2*>(cells + 2 * (b * slots + p));
+          double part = __dadd_rn(__dmul_rn((double)cell.x, grid.elo[b]), __dmul_rn((double)cell.y, grid.ulp[b]));
+          if (b == B0) part = __dmul_rn((double)(long long)tiny[slots + p], tiny_unit);
+          if (b == B0 - 1 && negatives) part = __dmul_rn((double)(long long)tiny[p], tiny_unit);
+          if (b >= nb) part = 0.0;  // (the buckets beyond nb are empty)
+          int c = (int)cell.x;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const int uc = __shfl_up_sync(0xFFFFFFFFu, c, o);
+            const double us = __shfl_up_sync(0xFFFFFFFFu, part, o);
+            if (lane >= o) { c += uc; part = __dadd_rn(part, us); }
+          }
+          part = __dadd_rn(part, sum);
+          counts[b * slots + p] = (uint16_t)(run + c - (int)cell.x);
+          sums[b * slots + p] = part;
+          run += __shfl_sync(0xFFFFFFFFu, c, 31);
+          sum = __shfl_sync(0xFFFFFFFFu, part, 31);
+        }
+      }
+    } else {  // a thread each
+      for (int p = tid; p <= pixels; p += THREADS) {
+        int run = 0;
+        double sum = 0.0;
+        const double inner_neg = __dmul_rn((double)(long long)tiny[p], tiny_unit), inner_pos = __dmul_rn((double)(long long)tiny[slots + p], tiny_unit);
 #pragma unroll 4
-      for (int b = 0; b < BUCKETS; ++b) {  // (the buckets beyond nb are empty)
-        const uint2 cell = *reinterpret_cast<const uint2*>(cells + 2 * (b * slots + p));
-        double part = __dadd_rn(__dmul_rn((double)cell.x, grid.elo[b]), __dmul_rn((double)cell.y, grid.ulp[b]));
-        if (b == B0) part = inner_pos;
-        if (b == B0 - 1 && negatives) part = inner_neg;
-        sum = b < nb ? __dadd_rn(sum, part) : sum;
-        counts[b * slots + p] = (uint16_t)run;
-        run += (int)cell.x;
-        sums[b * slots + p] = sum;
+        for (int b = 0; b < BUCKETS; ++b) {  // (the buckets beyond nb are empty)
+          const uint2 cell = *reinterpret_cast<const uint2*>(cells + 2 * (b * slots + p));
+          double part = __dadd_rn(__dmul_rn((double)cell.x, grid.elo[b]), __dmul_rn((double)cell.y, grid.ulp[b]));
+          if (b == B0) part = inner_pos;
+          if (b == B0 - 1 && negatives) part = inner_neg;
+          sum = b < nb ? __dadd_rn(sum, part) : sum;
+          counts[b * slots + p] = (uint16_t)run;
+          run += (int)cell.x;
+          sums[b * slots + p] = sum;
+        }
       }
     }
     __syncthreads();
@@ -852,12 +883,14 @@ constexpr size_t kSmemPerSm = 228 * 1024, kSmemCtaMax = 227 * 1024, kTileStatic 
 // The tile whose estimated time over the whole layer is least, in cycles.  From phase timings on 64 x 56 x 56 (7 x 14 tiles,
 // two CTAs per SM): per tile a fixed part, 4.3 per staged value and 6200 per round of 16 patches (a warp each); a CTA alone
 // on its SM takes 0.65 of that.  The model met the measured times of 30 tile shapes on four layers within 10 %.
+// Returned is what the chosen tiles take with all that is left out there because every tile has it (tables of offsets, the grid,
+// masks): 25000 cycles, 2.7 per staged value and 8100 per round for a CTA of a pair, 20000, 1.5 and 6000 for one alone.
 template <typename ListT>
 double choose_tile(TileArgs* a, size_t* smem_out) {
-  double best = 0.0;
+  double best = 0.0, whole = 0.0;
   int bh = 0, bw = 0;
   const int khw = a->d.kh * a->d.kw, sms = sm_count();
-  const double per_round = 6200.0 * (a->buckets > 32 ? 1.3 : 1.0) * (0.6 + 0.4 * khw / 9.0);
+  const double round_scale = (a->buckets > 32 ? 1.3 : 1.0) * (0.6 + 0.4 * khw / 9.0);
   // (extents that a number of tiles needs: a smaller one adds tiles or nothing)
   for (int nh = (a->Ho + 15) / 16, th = 17; th > 1; ++nh) {
     if ((a->Ho + nh - 1) / nh == th) continue;
@@ -874,15 +907,19 @@ double choose_tile(TileArgs* a, size_t* smem_out) {
       const int64_t tiles = (int64_t)t.tiles_h * t.tiles_w * t.d.N, resident = (int64_t)sms * (pair ? 2 : 1);
       const double waves = (double)((tiles + resident - 1) / resident);
       const int rounds = (t.TH * t.TW + kTileWarps - 1) / kTileWarps;
-      const double one = 8000.0 + 4.3 * t.slots * 4 * t.quads + rounds * per_round;
-      const double cost = waves * one * (pair && tiles > sms ? 1.0 : 0.65);
-      if (best == 0.0 || cost < best) { best = cost; bh = th; bw = tw; }
+      const double values = (double)t.slots * 4 * t.quads, searches = rounds * round_scale;
+      const bool paired = pair && tiles > sms;
+      const double cost = waves * (8000.0 + 4.3 * values + 6200.0 * searches) * (paired ? 1.0 : 0.65);
+      if (best == 0.0 || cost < best) {
+        best = cost; bh = th; bw = tw;
+        whole = waves * (paired ? 25000.0 + 2.7 * values + 8100.0 * searches : 20000.0 + 1.5 * values + 6000.0 * searches);
+      }
     }
   }
   if (best == 0.0) return 0.0;
   set_tile(a, bh, bw);
   *smem_out = tile_bytes<ListT>(a);
-  return (int64_t)a->tiles_h * a->tiles_w * a->d.N <= 0x7FFFFFFF ? best : 0.0;
+  return (int64_t)a->tiles_h * a->tiles_w * a->d.N <= 0x7FFFFFFF ? whole : 0.0;
 }
 
 template <int KHW, int BPL, typename ListT>
@@ -890,13 +927,16 @@ cudaError_t launch_tile(TileArgs& a, bool always, cudaStream_t stream, bool* app
   a.buckets = 32 * BPL;
   a.octaves = BPL == 1 ? 8 : 12;
   // A layer of few patches is done sooner by a CTA per patch: about 15000 cycles and 5 + 0.012 n per patch, where this kernel
-  // has some 45000 on top of its tiles (its code alone is 60 KB).  64 x 32 x 32 at batch 1, 1024 patches of 576: 35 us here, 20 us
-  // there; of 576 values the line is at about 3500 patches.
+  // has 8000 to 35000 on top of its tiles (the kernel for marked patches, code that is not in the cache, longer hulls in longer
+  // rows).  Measured, a CTA per patch and this, post-ReLU; N(0, 1): 2 x 64 x 28 x 28, 1568 patches of 576, 21 and 23 us; 21 and 28;
+  // 4 x 128 x 28 x 28, 3136 of 1152, 45 and 34; 46 and 48; 24 x 128 x 28 x 28 with stride 2, 4704 of 1152, 61 and 50; 62 and 60;
+  // 8 x 256 x 14 x 14, 1568 of 2304, 39 and 32; 38 and 44; 2 x 32 x 27 x 27 5 x 5, 1458 of 800, 23 and 26; 25 and 32.
   const double by_patch = always ? 1e30 : 15000.0 + (5.0 + 0.012 * a.n) * (double)a.d.N * a.Ho * a.Wo;
-  if (by_patch < 45000.0) return cudaSuccess;
+  const double set_up = (a.n < 1300 ? 5000.0 + 10.0 * a.n : 15000.0 + 2.4 * a.n) + (a.d.kh * a.d.kw > 9 ? 8000.0 : 0.0);
+  if (by_patch < set_up) return cudaSuccess;
   size_t smem = 0;
   const double cycles = choose_tile<ListT>(&a, &smem);
-  if (cycles == 0.0 || by_patch < 45000.0 + cycles) return cudaSuccess;
+  if (cycles == 0.0 || by_patch < set_up + cycles) return cudaSuccess;
   auto kern = binarize_patches_tile_kernel<KHW, BPL, ListT>;
   cudaError_t e = ensure_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
