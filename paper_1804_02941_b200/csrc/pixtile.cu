@@ -100,6 +100,16 @@ __device__ __forceinline__ int grid_bucket(const Grid& g, float v, int step, int
   return (int)g.lut[v < 0.0f ? side - 1 - step : side + step];
 }
 
+// Sum of a pixel's values in a bucket, channel by channel.
+__device__ __noinline__ double sum_by_channel(const Grid& g, const float* values, int C, int bucket) {
+  double sum = 0.0;
+  for (int c = 0; c < C; ++c) {
+    const float v = values[c];
+    if (v != 0.0f && grid_bucket(g, v, grid_step(__float_as_uint(v) & 0x7FFFFFFFu, g.base, g.side), g.side) == bucket) sum = __dadd_rn(sum, (double)v);
+  }
+  return sum;
+}
+
 // Inclusive prefix sum over the CTA; `total` in every thread.  part: THREADS / 32 words of shared memory.
 template <int THREADS, typename T>
 __device__ __forceinline__ T block_prefix(T v, T* part, T& total) {
@@ -218,8 +228,11 @@ __device__ __forceinline__ void choose_grid(Grid* g, int octaves, int buckets, i
   __syncthreads();
 }
 
+// KHW, the kernel's window: 9 (3 x 3, unrolled), kAnyWindow (up to 32 pixels, one per lane) or kWideWindow (up to 64, two).
+constexpr int kAnyWindow = 0, kWideWindow = -1;
+
 // The pixels of a patch's window: their slots (kh*kw of them).  3 x 3 windows keep them in registers.
-template <int KHW>
+template <int KHW, bool kFixed = (KHW > 0)>
 struct Window {
   int slot[KHW];
   const uint16_t* map;
@@ -232,8 +245,8 @@ struct Window {
   __device__ __forceinline__ int at(int i) const { return map[win[i]]; }  // (an index known at run time only)
   static __device__ __forceinline__ int count(const TileArgs&) { return KHW; }
 };
-template <>
-struct Window<0> {
+template <int KHW>
+struct Window<KHW, false> {
   const uint16_t* map;
   const uint16_t* win;
   __device__ __forceinline__ Window(const TileArgs&, const uint16_t* m, const uint16_t* w, int at) : map(m + at), win(w) {}
@@ -262,21 +275,37 @@ __device__ __forceinline__ double objective_near(double P, double T, int s, int 
   return P * P * r + Q * Q * q;
 }
 
+// The parts of a hull: lane i holds the part in pixel i of the window (and in pixel i + 32 of a wide one): the pixel's slot, where
+// the part begins in its list, and how many values come before it (lanes beyond the window hold the total).
+template <int KHW>
+struct HullParts {
+  static constexpr int kPerLane = KHW == kWideWindow ? 2 : 1;
+  int before[kPerLane], slot[kPerLane], begin[kPerLane];
+  int parts;
+  __device__ __forceinline__ int of(const int (&v)[kPerLane], int part) const {  // (any part per lane)
+    int r = __shfl_sync(0xFFFFFFFFu, v[0], part & 31);
+    if (kPerLane > 1) {
+      const int hi = __shfl_sync(0xFFFFFFFFu, v[kPerLane - 1], part & 31);
+      if (part >= 32) r = hi;
+    }
+    return r;
+  }
+};
+
 // The best split among the `size` values of a hull (and its run of z zeros, if `zeros`): E values a lane, sorted.  s_lo, P_lo:
-// count and sum below the hull.  Lane i < parts holds the part of the hull in pixel i of the window: the pixel's slot, where the
-// part begins in its list, and how many values come before it (lanes beyond hold the total).
-// E = 1: the values are in `gathered` already.
+// count and sum below the hull.  E = 1: the values are in `gathered` already.
 struct HullSplit {
   int s;             // 0: none
   double P;
   uint32_t above;    // a key that the high side reaches and the low side does not
 };
 
-template <int E, int WN, typename ListT>
-__device__ __forceinline__ HullSplit search_hull(const float* gathered, int before_me, int slot_me, int begin_me, int parts,
-                                                 const float* tile, int pitch, const ListT* list, int list_pitch, int size, bool zeros, int z, int s_lo, double P_lo, double T, int n,
+template <int E, int KHW, typename ListT>
+__device__ __forceinline__ HullSplit search_hull(const float* gathered, const HullParts<KHW>& h, const float* tile, int pitch,
+                                                 const ListT* list, int list_pitch, int size, bool zeros, int z, int s_lo, double P_lo, double T, int n,
                                                  int lane) {
   constexpr unsigned kAll = 0xFFFFFFFFu;
+  constexpr int WN = KHW > 0 ? 16 : 32 * HullParts<KHW>::kPerLane;  // at least the window's pixels
   uint32_t key[E];
 #pragma unroll
   for (int j = 0; j < E; ++j) {
@@ -288,10 +317,10 @@ __device__ __forceinline__ HullSplit search_hull(const float* gathered, int befo
     int part = 0;  // the last one that starts at or before i (parts that start there before it are empty)
 #pragma unroll
     for (int step = WN / 2; step >= 1; step >>= 1) {
-      const int o = __shfl_sync(kAll, before_me, (part + step) & 31);
-      if (part + step < parts && i >= o) part += step;
+      const int o = h.of(h.before, part + step);
+      if (part + step < h.parts && i >= o) part += step;
     }
-    const int o = __shfl_sync(kAll, before_me, part), slot = __shfl_sync(kAll, slot_me, part), begin = __shfl_sync(kAll, begin_me, part);
+    const int o = h.of(h.before, part), slot = h.of(h.slot, part), begin = h.of(h.begin, part);
     key[j] = zeros && i == size ? kZeroKey : kPadKey;
     if (i < size) key[j] = order_key(tile[slot * pitch + (int)list[slot * list_pitch + begin + i - o]]);
   }
@@ -358,11 +387,10 @@ __device__ __forceinline__ HullSplit search_hull(const float* gathered, int befo
   return best;
 }
 
-template <int E, int WN, typename ListT>
-__device__ __noinline__ HullSplit search_long_hull(int before_me, int slot_me, int begin_me, int parts, const float* tile, int pitch,
-                                                   const ListT* list, int list_pitch, int size, bool zeros, int z, int s_lo, double P_lo,
-                                                   double T, int n, int lane) {
-  return search_hull<E, WN>(nullptr, before_me, slot_me, begin_me, parts, tile, pitch, list, list_pitch, size, zeros, z, s_lo, P_lo, T, n, lane);
+template <int E, int KHW, typename ListT>
+__device__ __noinline__ HullSplit search_long_hull(const HullParts<KHW> h, const float* tile, int pitch, const ListT* list, int list_pitch,
+                                                   int size, bool zeros, int z, int s_lo, double P_lo, double T, int n, int lane) {
+  return search_hull<E>(nullptr, h, tile, pitch, list, list_pitch, size, zeros, z, s_lo, P_lo, T, n, lane);
 }
 
 // The best split of one patch, by a warp.  A segment is a bucket or, between the negative and the positive buckets (at
@@ -373,11 +401,14 @@ __device__ __forceinline__ PatchCode search_patch(const TileArgs& a, const Grid&
                                                   const double* sums, const uint16_t* counts, const ListT* list,
                                                   const float* tile, float* hull, int lane) {
   constexpr unsigned kAll = 0xFFFFFFFFu;
-  constexpr int WN = KHW ? 16 : 32;  // the window's pixels fit this many lanes
+  constexpr int PER_LANE = HullParts<KHW>::kPerLane;
   const int n = a.n, B0 = g.B0, slots = a.slots;
   const int wn = Window<KHW>::count(a);
   PatchCode code{kRowMark, 0.0f, 0.0f, __uint_as_float(0x7FC00000u), false};
-  const int own = lane < wn ? map[at + win[lane]] : 0;  // lane i holds pixel i of the window
+  HullParts<KHW> hp;
+  hp.parts = wn;
+#pragma unroll
+  for (int t = 0; t < PER_LANE; ++t) hp.slot[t] = 32 * t + lane < wn ? map[at + win[32 * t + lane]] : 0;
   // ---- count and sum at the upper edge of buckets lane, lane + 32 ----
   int cc[BPL];
   double cs[BPL];
@@ -394,12 +425,14 @@ __device__ __forceinline__ PatchCode search_patch(const TileArgs& a, const Grid&
         cs[j] = __dadd_rn(cs[j], S[32 * j * slots]);
       }
     };
-    if (KHW) {
+    if (KHW > 0) {
 #pragma unroll
-      for (int i = 0; i < KHW; ++i) add(__shfl_sync(kAll, own, i));
+      for (int i = 0; i < (KHW > 0 ? KHW : 0); ++i) add(__shfl_sync(kAll, hp.slot[0], i));
     } else {
+#pragma unroll
+      for (int t = 0; t < PER_LANE; ++t)
 #pragma unroll 4
-      for (int i = 0; i < wn; ++i) add(__shfl_sync(kAll, own, i));
+        for (int i = 0; i < min(32, wn - 32 * t); ++i) add(__shfl_sync(kAll, hp.slot[t], i));
     }
   }
   const int m = __shfl_sync(kAll, cc[BPL - 1], 31);
@@ -514,34 +547,41 @@ __device__ __forceinline__ PatchCode search_patch(const TileArgs& a, const Grid&
     if (upto - below == m) return code;
   }
   // ---- their values, from the lists of the window's pixels ----
-  int begin = 0, incl = 0;
-  if (lane < wn) {
-    begin = b_lo > 0 ? counts[(b_lo - 1) * slots + own] : 0;
-    incl = (b_end > 0 ? counts[(b_end - 1) * slots + own] : 0) - begin;
-  }
-  int before = -incl;
+  int count[PER_LANE], total = 0;
 #pragma unroll
-  for (int o = 1; o < WN; o <<= 1) {
-    const int u = __shfl_up_sync(kAll, incl, o);
-    if (lane >= o) incl += u;
+  for (int t = 0; t < PER_LANE; ++t) {
+    hp.begin[t] = count[t] = 0;
+    if (32 * t + lane < wn) {
+      hp.begin[t] = b_lo > 0 ? counts[(b_lo - 1) * slots + hp.slot[t]] : 0;
+      count[t] = (b_end > 0 ? counts[(b_end - 1) * slots + hp.slot[t]] : 0) - hp.begin[t];
+    }
+    int incl = count[t];
+#pragma unroll
+    for (int o = 1; o < (KHW > 0 ? 16 : 32); o <<= 1) {
+      const int u = __shfl_up_sync(kAll, incl, o);
+      if (lane >= o) incl += u;
+    }
+    hp.before[t] = total + incl - count[t];
+    if (t + 1 < PER_LANE) total += __shfl_sync(kAll, incl, 31);
   }
-  before += incl;
   HullSplit split;
-#define DAB_HULL before, own, begin, wn, tile, a.pitch, list, 4 * a.quads, size, zeros, z, s_lo, P_lo, T, n, lane
+#define DAB_HULL hp, tile, a.pitch, list, 4 * a.quads, size, zeros, z, s_lo, P_lo, T, n, lane
   if (size < 32) {  // the usual case: the pixels' lanes bring the values together in shared memory
-    const int count = lane < wn ? (b_end > 0 ? counts[(b_end - 1) * slots + own] : 0) - begin : 0;
-    const ListT* const from = list + own * 4 * a.quads + begin;
-    const float* const values = tile + own * a.pitch;
-    for (int k = 0; k < count; ++k) hull[before + k] = values[from[k]];
+#pragma unroll
+    for (int t = 0; t < PER_LANE; ++t) {
+      const ListT* const from = list + hp.slot[t] * 4 * a.quads + hp.begin[t];
+      const float* const values = tile + hp.slot[t] * a.pitch;
+      for (int k = 0; k < count[t]; ++k) hull[hp.before[t] + k] = values[from[k]];
+    }
     __syncwarp();
-    split = search_hull<1, WN>(hull, DAB_HULL);
+    split = search_hull<1>(hull, DAB_HULL);
     __syncwarp();
   }
-  else if (size < 64) split = search_long_hull<2, WN>(DAB_HULL);
-  else if (size < 128) split = search_long_hull<4, WN>(DAB_HULL);
-  else if (size < 256) split = search_long_hull<8, WN>(DAB_HULL);
-  else if (size < 512) split = search_long_hull<16, WN>(DAB_HULL);
-  else split = search_long_hull<32, WN>(DAB_HULL);
+  else if (size < 64) split = search_long_hull<2>(DAB_HULL);
+  else if (size < 128) split = search_long_hull<4>(DAB_HULL);
+  else if (size < 256) split = search_long_hull<8>(DAB_HULL);
+  else if (size < 512) split = search_long_hull<16>(DAB_HULL);
+  else split = search_long_hull<32>(DAB_HULL);
 #undef DAB_HULL
   if (split.s <= 0 || split.s >= n) return code;
   // the two means side by side in the even and the odd lanes
@@ -734,6 +774,17 @@ __global__ void __launch_bounds__(kTileThreads, 2) binarize_patches_tile_kernel(
       }
     }
     __syncthreads();
+    if (sizeof(ListT) > 1 && C > 512) {
+      // 32 bits hold the mantissas of 512 values: what a bucket with more of them has lost is some 2^32 units of its octave
+      for (int p = tid; p < pixels; p += THREADS)
+        for (int b = 0; b < nb; ++b) {  // (nb < BUCKETS)
+          if (counts[(b + 1) * slots + p] - counts[b * slots + p] <= 512 || b == B0 || (b == B0 - 1 && negatives)) continue;
+          const double lost = __dsub_rn(sum_by_channel(grid, tile + p * a.pitch, C, b), __dsub_rn(sums[b * slots + p], b ? sums[(b - 1) * slots + p] : 0.0));
+          const double unit = __dmul_rn(4294967296.0, grid.ulp[b]);
+          for (int q = b; q < BUCKETS; ++q) sums[q * slots + p] = __dadd_rn(sums[q * slots + p], __dmul_rn(rint(__ddiv_rn(lost, unit)), unit));
+        }
+      __syncthreads();
+    }
     // ---- per pixel: channels ordered by bucket; the cursors end as inclusive cumulative counts ----
 #pragma unroll 2
     for (int u = tid; u < units; u += THREADS) {
@@ -822,23 +873,30 @@ __global__ void __launch_bounds__(kTileThreads, 2) binarize_patches_tile_kernel(
         for (int j = 0; j < 4; ++j) append(b[j], 9);
       }
     } else {
-      const uint32_t all = khw == 32 ? 0xFFFFFFFFu : (1u << khw) - 1u;
+      const int low = KHW == kWideWindow ? 32 : khw;
       for (int q = 0; q < 8; ++q) {
-        uint32_t b[4] = {0u, 0u, 0u, 0u};
-        if (q < quads) {
+        uint32_t b[4] = {0u, 0u, 0u, 0u}, high[4] = {0u, 0u, 0u, 0u};  // high: pixels 32 and on of a wide window
+        auto bits_of = [&](uint32_t (&to)[4], int first, int count, uint32_t all) {
 #pragma unroll 5
-          for (int i = khw - 1; i >= 0; --i) {
+          for (int i = first + count - 1; i >= first; --i) {
             const float4 v = *reinterpret_cast<const float4*>(src + w(i) * a.pitch + 4 * q);
-            b[0] = __funnelshift_l(__float_as_uint(v.x - tv), b[0], 1);
-            b[1] = __funnelshift_l(__float_as_uint(v.y - tv), b[1], 1);
-            b[2] = __funnelshift_l(__float_as_uint(v.z - tv), b[2], 1);
-            b[3] = __funnelshift_l(__float_as_uint(v.w - tv), b[3], 1);
+            to[0] = __funnelshift_l(__float_as_uint(v.x - tv), to[0], 1);
+            to[1] = __funnelshift_l(__float_as_uint(v.y - tv), to[1], 1);
+            to[2] = __funnelshift_l(__float_as_uint(v.z - tv), to[2], 1);
+            to[3] = __funnelshift_l(__float_as_uint(v.w - tv), to[3], 1);
           }
 #pragma unroll
-          for (int j = 0; j < 4; ++j) b[j] = cb * 32 + 4 * q + j < C ? (b[j] ^ ~inv) & all : 0u;
+          for (int j = 0; j < 4; ++j) to[j] = cb * 32 + 4 * q + j < C ? (to[j] ^ ~inv) & all : 0u;
+        };
+        if (q < quads) {
+          bits_of(b, 0, low, low == 32 ? 0xFFFFFFFFu : (1u << low) - 1u);
+          if (KHW == kWideWindow) bits_of(high, 32, khw - 32, khw == 64 ? 0xFFFFFFFFu : (1u << (khw - 32)) - 1u);
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) append(b[j], khw);
+        for (int j = 0; j < 4; ++j) {
+          append(b[j], low);
+          if (KHW == kWideWindow) append(high[j], khw - 32);
+        }
       }
     }
   }
@@ -886,7 +944,7 @@ constexpr size_t kSmemPerSm = 228 * 1024, kSmemCtaMax = 227 * 1024, kTileStatic 
 // Returned is what the chosen tiles take with all that is left out there because every tile has it (tables of offsets, the grid,
 // masks): 25000 cycles, 2.7 per staged value and 8100 per round for a CTA of a pair, 20000, 1.5 and 6000 for one alone.
 template <typename ListT>
-double choose_tile(TileArgs* a, size_t* smem_out) {
+double choose_tile(TileArgs* a, size_t* smem_out, double* cost_out) {
   double best = 0.0, whole = 0.0;
   int bh = 0, bw = 0;
   const int khw = a->d.kh * a->d.kw, sms = sm_count();
@@ -916,6 +974,7 @@ double choose_tile(TileArgs* a, size_t* smem_out) {
       }
     }
   }
+  *cost_out = best;
   if (best == 0.0) return 0.0;
   set_tile(a, bh, bw);
   *smem_out = tile_bytes<ListT>(a);
@@ -935,7 +994,8 @@ cudaError_t launch_tile(TileArgs& a, bool always, cudaStream_t stream, bool* app
   const double set_up = (a.n < 1300 ? 5000.0 + 10.0 * a.n : 15000.0 + 2.4 * a.n) + (a.d.kh * a.d.kw > 9 ? 8000.0 : 0.0);
   if (by_patch < set_up) return cudaSuccess;
   size_t smem = 0;
-  const double cycles = choose_tile<ListT>(&a, &smem);
+  double cost;
+  const double cycles = choose_tile<ListT>(&a, &smem, &cost);
   if (cycles == 0.0 || by_patch < set_up + cycles) return cudaSuccess;
   auto kern = binarize_patches_tile_kernel<KHW, BPL, ListT>;
   cudaError_t e = ensure_dynamic_smem(kern, smem);
@@ -946,15 +1006,28 @@ cudaError_t launch_tile(TileArgs& a, bool always, cudaStream_t stream, bool* app
 }
 
 // 32 buckets for short rows, 64 from 1536 values on.  (Post-ReLU rows of 1152 take 13 % longer with 64, N(0, 1) ones 9 % less;
-// of 2304: 8 % longer and 15 % less.)
+// of 2304: 8 % longer and 15 % less.)  With a stride a tile stages many values for its patches, and tables of half the size may let
+// two tiles share an SM, or make them larger: 64 x 48 x 56 x 56 7 x 7 stride 2 post-ReLU 798 -> 467 us, N(0, 1) 753 -> 683.  Not for a
+// small gain, since N(0, 1) rows lose: 64 x 256 x 28 x 28 3 x 3 stride 2 (estimated gain 1.13) 213 -> 170, 207 -> 233.
 template <int KHW, typename ListT>
 cudaError_t launch_tile_buckets(TileArgs& a, bool always, cudaStream_t stream, bool* applicable) {
-  return a.n < 1536 ? launch_tile<KHW, 1, ListT>(a, always, stream, applicable) : launch_tile<KHW, 2, ListT>(a, always, stream, applicable);
+  bool longer = a.n >= 1536;
+  if (longer && a.d.stride_h * a.d.stride_w > 1) {
+    double cost[2];
+    for (int k = 0; k < 2; ++k) {
+      TileArgs t = a;
+      size_t smem;
+      t.buckets = 32 << k;
+      choose_tile<ListT>(&t, &smem, &cost[k]);
+    }
+    longer = cost[0] == 0.0 || (cost[1] > 0.0 && cost[1] <= (KHW == 9 ? 1.25 : 1.15) * cost[0]);
+  }
+  return longer ? launch_tile<KHW, 2, ListT>(a, always, stream, applicable) : launch_tile<KHW, 1, ListT>(a, always, stream, applicable);
 }
 
 }  // namespace
 
-// Patches of 257..8192 values of up to 512 channels through the tile coder and the kernel that codes what it marked.
+// Patches of 257..8192 values (up to 2048 channels, windows of up to 64 pixels) through the tile coder and the kernel that codes what it marked.
 // *applicable = false (nothing launched) when the geometry has no tile that fits shared memory or, unless `always`, when a CTA
 // per patch is expected to be faster.
 cudaError_t launch_binarize_patches_tile(const dab_conv_desc& d, int32_t Ho, int32_t Wo, const float* x, int32_t* pK,
@@ -964,7 +1037,7 @@ cudaError_t launch_binarize_patches_tile(const dab_conv_desc& d, int32_t Ho, int
   a.d = d; a.Ho = Ho; a.Wo = Wo; a.n = d.C * d.kh * d.kw;
   a.x = x; a.pK = pK; a.pgamma = pgamma; a.pdelta = pdelta; a.pflags = pflags; a.pmask = pmask; a.ldp = ldp;
   *applicable = false;
-  if (a.n <= 256 || a.n > 8192 || d.C > 512 || d.kh * d.kw > 32 || (int64_t)d.C * d.H * d.W > 0x7FFFFFFF) return cudaSuccess;
+  if (a.n <= 256 || a.n > 8192 || d.C > 2048 || d.kh * d.kw > 64 || (int64_t)d.C * d.H * d.W > 0x7FFFFFFF) return cudaSuccess;
   a.quads = (d.C + 3) / 4;
   a.pitch = 4 * (a.quads + 1 - (a.quads & 1));  // an odd number of quadruples: neighbouring pixels in different banks
   a.word_pitch = ldp | 1;
@@ -972,7 +1045,8 @@ cudaError_t launch_binarize_patches_tile(const dab_conv_desc& d, int32_t Ho, int
   cudaError_t e;
   if (d.kh == 3 && d.kw == 3)
     e = d.C <= 256 ? launch_tile_buckets<9, uint8_t>(a, always, stream, applicable) : launch_tile_buckets<9, uint16_t>(a, always, stream, applicable);
-  else e = launch_tile_buckets<0, uint16_t>(a, always, stream, applicable);
+  else if (d.kh * d.kw <= 32) e = launch_tile_buckets<kAnyWindow, uint16_t>(a, always, stream, applicable);
+  else e = launch_tile_buckets<kWideWindow, uint16_t>(a, always, stream, applicable);
   if (e != cudaSuccess || !*applicable) return e;
   return launch_binarize_patches_bucket(d, Ho, Wo, x, pK, pgamma, pdelta, pmask, ldp, pflags, /*marked_only=*/true, stream);
 }
