@@ -47,7 +47,11 @@ constexpr int kTinyBits = 51;
 // From this many pixels on a thread sums a pixel's buckets one after another; below it would leave most of them idle (4200 cycles for
 // 20 pixels where a warp per pixel takes 1500; at 100 pixels both take 5000, at 130 the warps 7000 to 10000).
 constexpr int kSerialPixels = 80;
-constexpr int kHullCap = 1024;     // values the search of one patch takes at most
+// Values the search of one patch takes at most; longer hulls are left to the CTA-per-patch kernel.  Short rows hardly have any, and a
+// search of 1024 in registers makes the kernel slower for all: 64 x 64 x 56 x 56 post-ReLU 426 us with it, 416 without; values
+// e^(4 N(0, 1)) 3.18 and 1.27 ms.  Longer rows need it: 61 x 256 x 14 x 14 N(0, 1) 131 us without it, 121 with.
+template <int BPL>
+__host__ __device__ constexpr int hull_cap() { return BPL == 1 ? 512 : 1024; }
 // A bucket is kept if its bound reaches the best edge objective times this: edges and inner corners are formed in fp32 from
 // sums rounded once (1e-6 relative), the place of a corner to 4e-7 of the bucket's count.
 constexpr float kKeep = 0.9999f;
@@ -538,7 +542,7 @@ __device__ __forceinline__ PatchCode search_patch(const TileArgs& a, const Grid&
     c_end = __shfl_sync(kAll, tc, (b_end - 1) & 31);
   }
   const int size = c_end - c_lo, s_lo = c_lo + (seg_lo > B0 ? z : 0);
-  if (size < 1 || size > kHullCap - 1 || (z == 0 && size == n)) return code;
+  if (size < 1 || size > hull_cap<BPL>() - 1 || (z == 0 && size == n)) return code;
   if (b_lo >= B0 - 1 && b_end <= B0 + 1) {  // the two buckets next to zero: does the patch have no other values?
     int below, upto;
     double unused;
@@ -580,8 +584,8 @@ __device__ __forceinline__ PatchCode search_patch(const TileArgs& a, const Grid&
   else if (size < 64) split = search_long_hull<2>(DAB_HULL);
   else if (size < 128) split = search_long_hull<4>(DAB_HULL);
   else if (size < 256) split = search_long_hull<8>(DAB_HULL);
-  else if (size < 512) split = search_long_hull<16>(DAB_HULL);
-  else split = search_long_hull<32>(DAB_HULL);
+  else if (BPL == 1 || size < 512) split = search_long_hull<16>(DAB_HULL);
+  else split = search_long_hull<(BPL == 1 ? 16 : 32)>(DAB_HULL);
 #undef DAB_HULL
   if (split.s <= 0 || split.s >= n) return code;
   // the two means side by side in the even and the odd lanes
