@@ -156,6 +156,7 @@ cudaError_t launch_binarize(const float* values, int64_t rows, int32_t n, int64_
   if (patch_coder_mode() == 1 || n <= 256)  // the setting covers the rows of matrices as well
     return launch_rows_sort(values, rows, n, ld_values, K, alpha, beta, mask, ld_mask, flags, stream);
   const RowOut out{K, alpha, beta, flags, mask, ld_mask, rows};
+  if (many_short_rows(rows, n)) return launch_rows_bucket<32>(values, n, ld_values, out, stream);
   if (n <= BucketShape<64>::kMaxN) return launch_rows_bucket<64>(values, n, ld_values, out, stream);
   if (n <= BucketShape<128>::kMaxN) return launch_rows_bucket<128>(values, n, ld_values, out, stream);
   return launch_rows_bucket<256>(values, n, ld_values, out, stream);

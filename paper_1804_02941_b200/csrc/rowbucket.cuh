@@ -29,9 +29,14 @@ namespace dab {
 // Shape of the coder by row length: T threads, PB of the 2 NB buckets each, 2^LOG2M per octave (12 octaves, 16 for the
 // longest rows).  A bucket's low sum takes 23 - LOG2M bits per value: it stays below 2^32 for kMaxCount values.
 template <int T> struct BucketShape;
+template <> struct BucketShape<32> { static constexpr int kMaxN = 512, LOG2M = 3, PB = 6, kHull = 256, kMaxCount = 4096; };
 template <> struct BucketShape<64> { static constexpr int kMaxN = 1024, LOG2M = 3, PB = 3, kHull = 256, kMaxCount = 4096; };
 template <> struct BucketShape<128> { static constexpr int kMaxN = 4096, LOG2M = 4, PB = 3, kHull = 512, kMaxCount = 8192; };
 template <> struct BucketShape<256> { static constexpr int kMaxN = DAB_MAX_N, LOG2M = 4, PB = 2, kHull = 1024, kMaxCount = 8192; };
+
+// A warp per row where there are rows for some 20 warps on every SM: it has no barriers to wait at.  Measured, two warps and one:
+// 512 rows of 300 values 7.8 and 9.8 us, 2048 11.6 and 11.7, 4096 21.3 and 16.9, 16384 74 and 57; 4096 of 512 20.7 and 18.1.
+inline bool many_short_rows(int64_t rows, int n) { return n <= BucketShape<32>::kMaxN && rows >= (int64_t)20 * sm_count(); }
 
 template <int T>
 struct __align__(16) BlockShared {  // (a multiple of 16 bytes: the staged values behind it are read 16 bytes at a time)
@@ -442,14 +447,18 @@ __device__ __forceinline__ void block_code_row(const Source& source, int n, unsi
         if (w == warp) { cw = m; sw = T_row; }
         m += bs->wcnt[w];
         T_row = __dadd_rn(T_row, bs->wsum[w]);
-        if (w == W / 2 - 1) { neg = m; Pneg = T_row; }  // the first half of the warps holds the negative buckets
+        if (w == W / 2 - 1) { neg = m; Pneg = T_row; }  // the first half of the threads holds the negative buckets
+      }
+      if (W == 1) {
+        neg = __shfl_sync(0xFFFFFFFFu, cincl, 15);
+        Pneg = __shfl_sync(0xFFFFFFFFu, sincl, 15);
       }
       cbefore += cw;
       sbefore = __dadd_rn(sw, sbefore);
       const int z = n - m;
       const double nd = (double)n;
       // ---- objective at the edges, bound inside each bucket ----
-      const bool positive = warp >= W / 2;
+      const bool positive = tid >= T / 2;
       const int zoff = positive ? z : 0;  // the zeros precede the positive buckets
       const float dz0 = z > 0 && neg > 0 ? objective_bound((double)neg, Pneg, T_row, nd) : -1.0f;
       const float dz1 = z > 0 && neg + z < n ? objective_bound((double)(neg + z), Pneg, T_row, nd) : -1.0f;
