@@ -170,22 +170,58 @@ __global__ void __launch_bounds__(256, 2) conv_dense_kernel(dab_conv_desc d, int
   }
 }
 
+// A thread per output, for one or two filters of few taps: there is nothing to share.
+__global__ void __launch_bounds__(kGlueThreads) conv_dense_direct_kernel(dab_conv_desc d, int Ho, int Wo, const float* __restrict__ x,
+                                                                         const float* __restrict__ w, const float* __restrict__ bias,
+                                                                         float* __restrict__ y, const PostOps post) {
+  const int64_t outputs = (int64_t)d.N * d.Cout * Ho * Wo;
+  const int n = d.C * d.kh * d.kw;
+  for (int64_t oi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; oi < outputs; oi += (int64_t)gridDim.x * blockDim.x) {
+    const int wo = (int)(oi % Wo);
+    const int64_t line = oi / Wo, plane = line / Ho;
+    const int ho = (int)(line % Ho), co = (int)(plane % d.Cout);
+    const float* const wrow = w + (int64_t)co * n;
+    const float* const ximg = x + plane / d.Cout * d.C * d.H * d.W;
+    const int hb = ho * d.stride_h - d.pad_h, wb = wo * d.stride_w - d.pad_w;
+    double acc = 0.0;
+    int k = 0;
+    for (int c = 0; c < d.C; ++c)
+      for (int r = 0; r < d.kh; ++r)
+        for (int s = 0; s < d.kw; ++s, ++k) {
+          const int h = hb + r, q = wb + s;
+          const float v = (unsigned)h < (unsigned)d.H && (unsigned)q < (unsigned)d.W ? __ldg(ximg + ((int64_t)c * d.H + h) * d.W + q) : 0.0f;
+          acc = __fma_rn((double)v, (double)__ldg(wrow + k), acc);
+        }
+    if (bias) acc = __dadd_rn(acc, (double)__ldg(bias + co));
+    const float v = (float)acc;
+    y[oi] = post.count > 0 ? apply_post(post, v, co, oi) : v;
+  }
+}
+
 // 128 positions x 64 filters (or 48, where that wastes fewer) where that gives the device work for every SM; otherwise
 // (batch 1, fully connected layers, where a chain of n dependent additions is what counts) 32 positions x 16 filters in
-// chunks of 64 taps, one memory latency each.
+// chunks of 64 taps, one memory latency each.  Layers of few filters take tiles of 8 or 16 of them.  Measured, 48 filters, this, and a
+// thread per output: 8 x 3 x 224 x 224 3 x 3, 8 filters 90, 46 and 107 us, 4 filters 89, 46 and 56, one filter 87, 46 and 18; 64 channels
+// 1 x 1 on 16 x 56 x 56, one filter 27, 14 and 26.
 cudaError_t launch_conv_dense(const dab_conv_desc& d, int Ho, int Wo, const float* x, const float* w, const float* bias, float* y,
                               const PostOps& post, cudaStream_t stream) {
   const int64_t positions = (int64_t)d.N * Ho * Wo;
+  auto run = [&](auto kernel, int pt, int ct) {
+    const int co_tiles = (d.Cout + ct - 1) / ct;
+    const int64_t blocks = (positions + pt - 1) / pt * co_tiles;
+    if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
+    kernel<<<(unsigned)blocks, 256, 0, stream>>>(d, Ho, Wo, co_tiles, x, w, bias, y, post);
+    return cudaGetLastError();
+  };
   const bool large = ((positions + 127) / 128) * ((d.Cout + 63) / 64) >= sm_count();
   const bool by48 = (d.Cout + 47) / 48 * 48 < (d.Cout + 63) / 64 * 64;
-  const int ct = large ? (by48 ? 48 : 64) : 16, pt = large ? 128 : 32;
-  const int co_tiles = (d.Cout + ct - 1) / ct;
-  const int64_t blocks = (positions + pt - 1) / pt * co_tiles;
-  if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
-  if (!large) conv_dense_kernel<1, 2, 64><<<(unsigned)blocks, 256, 0, stream>>>(d, Ho, Wo, co_tiles, x, w, bias, y, post);
-  else if (by48) conv_dense_kernel<4, 6, 16><<<(unsigned)blocks, 256, 0, stream>>>(d, Ho, Wo, co_tiles, x, w, bias, y, post);
-  else conv_dense_kernel<4, 8, 16><<<(unsigned)blocks, 256, 0, stream>>>(d, Ho, Wo, co_tiles, x, w, bias, y, post);
-  return cudaGetLastError();
+  if (!large) return run(conv_dense_kernel<1, 2, 64>, 32, 16);
+  if (d.Cout <= 2 && d.C * d.kh * d.kw <= 32) {
+    conv_dense_direct_kernel<<<glue_blocks(positions * d.Cout), kGlueThreads, 0, stream>>>(d, Ho, Wo, x, w, bias, y, post);
+    return cudaGetLastError();
+  }
+  if (d.Cout <= 16) return d.Cout <= 8 ? run(conv_dense_kernel<4, 1, 16>, 128, 8) : run(conv_dense_kernel<4, 2, 16>, 128, 16);
+  return by48 ? run(conv_dense_kernel<4, 6, 16>, 128, 48) : run(conv_dense_kernel<4, 8, 16>, 128, 64);
 }
 
 // Elementwise layers with no layer before them that could take them along: one pass, four elements a thread (VEC) where the
