@@ -143,6 +143,9 @@ cudaError_t launch_sign_rows(const float* values, int64_t rows, int32_t n, int64
 cudaError_t launch_sign_patches(const dab_conv_desc& d, int32_t Ho, int32_t Wo, const float* x, int32_t* pK,
                                 float* pgamma, float* pdelta, uint32_t* pmask, int32_t ldp, uint32_t* pflags,
                                 cudaStream_t stream);
+// The same, a warp per patch over a staged tile (patches.cu).  cudaErrorInvalidValue: no tile fits, nothing was launched.
+cudaError_t launch_sign_patches_staged(const dab_conv_desc& d, int32_t Ho, int32_t Wo, const float* x, int32_t* pK, float* pgamma,
+                                       float* pdelta, uint32_t* pmask, int32_t ldp, uint32_t* pflags, cudaStream_t stream);
 // Weights-only binarized convolution on the tensor cores; see wbin.cu.  pixmax: N*H*W words of scratch.
 // cudaErrorInvalidValue: no tile fits.
 cudaError_t launch_wbin_conv(const dab_conv_desc& d, int32_t Ho, int32_t Wo, const float* x, const uint32_t* wmask,

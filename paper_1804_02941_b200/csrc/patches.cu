@@ -4,6 +4,7 @@
 
 #include "histcode.cuh"
 #include "rowcode.cuh"
+#include "signrow.cuh"
 
 namespace dab {
 
@@ -389,6 +390,33 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, DAB_HIST_MINBLOCKS) binariz
   }
 }
 
+// Sign coding, a warp per patch over a staged tile: few channels or wide windows, where the coder of signcode.cu, which takes 32
+// channels and a ballot's width of pixels at a time, has little to put into them.
+__global__ void __launch_bounds__(kWarpsPerCta * 32) sign_patches_staged_kernel(const PatchArgs a) {
+  constexpr int THREADS = kWarpsPerCta * 32;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* tile = reinterpret_cast<float*>(smem_raw);
+  const int ch_words = a.in_h * a.pitch;
+  uint16_t* off = reinterpret_cast<uint16_t*>(tile + (size_t)a.d.C * ch_words);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  fill_offsets(a, off, ch_words, threadIdx.x, THREADS);
+  const int64_t total_tiles = (int64_t)a.tiles_h * a.tiles_w * a.d.N;
+  for (int64_t tile_id = blockIdx.x; tile_id < total_tiles; tile_id += gridDim.x) {
+    const TileCoord t = tile_coord(a, tile_id);
+    __syncthreads();
+    load_tile<false>(a, a.x + (int64_t)t.img * a.d.C * a.d.H * a.d.W, t.h0, t.w0, tile, ch_words, threadIdx.x, THREADS);
+    __syncthreads();
+    for (int p = warp; p < t.th * t.tw; p += kWarpsPerCta) {
+      const int lh = p / t.tw, lw = p % t.tw;
+      const float* origin = tile + lh * a.d.stride_h * a.pitch + lw * a.d.stride_w;
+      auto value = [origin, off](int i) { return origin[off[i]]; };
+      const int64_t pi = ((int64_t)t.img * a.Ho + (t.ho0 + lh)) * a.Wo + (t.wo0 + lw);
+      warp_sign_row(value, a.n, a.ldp, lane, a.pK + pi, a.pgamma + pi, a.pdelta + pi, a.pflags ? a.pflags + pi : nullptr,
+                    a.pmask + pi * (int64_t)a.ldp);
+    }
+  }
+}
+
 // 0: by tile density (default), 1: sort-based coders only, 2: histogram-pruned coder wherever it applies.
 static std::atomic<int> g_patch_coder_mode{0};
 
@@ -504,6 +532,16 @@ static cudaError_t launch_group_for(PatchArgs& a, cudaStream_t stream, bool shap
   if (a.n <= 8192) return launch_patches_group<16, 16, 16, false, true>(a, stream, shape_only);
   if (a.n == 9216) return launch_patches_group<16, 16, 18, true, false>(a, stream, shape_only);
   return launch_patches_group<16, 16, 32, false, false>(a, stream, shape_only);
+}
+
+cudaError_t launch_sign_patches_staged(const dab_conv_desc& d, int32_t Ho, int32_t Wo, const float* x, int32_t* pK, float* pgamma,
+                                       float* pdelta, uint32_t* pmask, int32_t ldp, uint32_t* pflags, cudaStream_t stream) {
+  PatchArgs a;
+  a.d = d; a.Ho = Ho; a.Wo = Wo; a.n = d.C * d.kh * d.kw;
+  a.scratch_words = 0;
+  a.defer_dense = 0; a.marked_only = 0; a.tile_shape = -1;
+  a.x = x; a.pK = pK; a.pgamma = pgamma; a.pdelta = pdelta; a.pflags = pflags; a.pmask = pmask; a.ldp = ldp;
+  return launch_patches(sign_patches_staged_kernel, a, 0, kWarpsPerCta * 32, kWarpsPerCta, stream);
 }
 
 cudaError_t launch_binarize_patches(const dab_conv_desc& d, int32_t Ho, int32_t Wo, const float* x, int32_t* pK,

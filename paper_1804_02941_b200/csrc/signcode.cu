@@ -10,7 +10,7 @@
 // on 256 x 128 x 28 x 28, 3 x 3: 495 us with every patch element gathered by a warp per patch -> 72 us (1.8 TB/s).
 #include <cmath>
 
-#include "rowcode.cuh"
+#include "signrow.cuh"
 
 namespace dab {
 namespace {
@@ -178,47 +178,6 @@ __global__ void __launch_bounds__(kSignThreads, 4) sign_patches_kernel(const Sig
   }
 }
 
-// One warp per row of a matrix; value(i) returns element i.
-template <typename Value>
-__device__ __forceinline__ void warp_sign_row(Value value, int n, int ld, int lane, int32_t* K_out, float* gamma_out,
-                                              float* delta_out, uint32_t* flags_out, uint32_t* __restrict__ mrow) {
-  double sum = 0.0;
-  int ones = 0, bad = 0;
-  uint32_t mine = 0;
-  const int words = (n + 31) >> 5;
-  for (int k = 0; k < words; ++k) {
-    const int i = k * 32 + lane;
-    float x = -1.0f;  // lanes beyond n contribute a 0 bit
-    if (i < n) {
-      x = value(i);
-      bad |= is_nonfinite(x);
-      sum += fabs((double)x);
-    }
-    const uint32_t word = __ballot_sync(0xFFFFFFFFu, i < n && x >= 0.0f);
-    ones += __popc(word);
-    if ((k & 31) == lane) mine = word;
-    if ((k & 31) == 31 || k == words - 1) {  // a batch of up to 32 words is complete: one coalesced store
-      const int w = (k & ~31) + lane;
-      if (w <= k) mrow[w] = mine;
-    }
-  }
-  for (int w = words + lane; w < ld; w += 32) mrow[w] = 0u;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
-  bad = __any_sync(0xFFFFFFFFu, bad);
-  if (bad) {  // flagged rows: empty mask, NaN scales
-    __syncwarp();
-    for (int w = lane; w < ld; w += 32) mrow[w] = 0u;
-  }
-  if (lane == 0) {
-    const float g = bad ? __uint_as_float(0x7FC00000u) : (float)(sum / (double)n);
-    *K_out = bad ? 0 : ones;
-    *gamma_out = g;
-    *delta_out = -g;
-    if (flags_out) *flags_out = bad ? DAB_ROW_NONFINITE : 0u;
-  }
-}
-
 __global__ void __launch_bounds__(256) sign_rows_kernel(const float* __restrict__ values, int64_t rows, int32_t n,
                                                         int64_t ld_values, int32_t* K, float* alpha, float* beta,
                                                         uint32_t* mask, int32_t ld_mask, uint32_t* flags) {
@@ -254,7 +213,8 @@ __global__ void __launch_bounds__(kSignThreads) sign_wide_patches_kernel(const S
 // Rows of output positions per tile: the number whose estimated cycles over the whole layer are fewest.  A ballot of a
 // channel costs a warp about 10 instructions, 32 channels of 32 patches about 38 per window position (the proportions
 // matter, not the scale); tiles share the halo of kh - stride rows, and a small layer needs enough of them.
-bool choose_sign_tile(SignArgs* a, size_t* smem_out) {
+// *us_out: what that tile's estimate comes to, a generic window's rows at 500 instructions each.
+bool choose_sign_tile(SignArgs* a, size_t* smem_out, double* us_out) {
   const dab_conv_desc& d = a->d;
   if (d.kw > 32) return false;
   const int widest = (32 - d.kw) / d.stride_w + 1;
@@ -281,6 +241,9 @@ bool choose_sign_tile(SignArgs* a, size_t* smem_out) {
       best = cost;
       a->TH = th; a->in_h = in_h; a->groups = groups;
       *smem_out = smem;
+      const double unit = d.kh == 3 && d.kw == 3 ? 342.0 : 500.0 * d.kh * (d.stride_h * d.stride_w > 1 ? 2.0 : 1.0);
+      *us_out = 3.0 + (double)((tiles + slots - 1) / slots) * sqrt((double)ctas) *
+                          (1500.0 + 10.0 * groups * ((d.C + 7) / 8) * 8 + unit * ((units + 7) / 8) * 8) / 3000.0;
     }
   }
   if (best == 0.0) return false;
@@ -307,8 +270,19 @@ cudaError_t launch_sign_patches(const dab_conv_desc& d, int32_t Ho, int32_t Wo, 
   a.x = x; a.pK = pK; a.pgamma = pgamma; a.pdelta = pdelta; a.pflags = pflags; a.pmask = pmask; a.ldp = ldp;
   a.magic_ldp = (uint32_t)((0x100000000ull + (uint64_t)ldp - 1) / (uint64_t)ldp);
   size_t smem = 0;
-  if (!choose_sign_tile(&a, &smem)) {
-    const int64_t blocks = ((int64_t)d.N * Ho * Wo + kSignWarps - 1) / kSignWarps;
+  double us = 0.0;
+  const double patches = (double)d.N * Ho * Wo;
+  // The other coder: a warp's chain of n / 32 words, and per patch what it reads and stages.  It is ahead for few channels with wide
+  // windows, strides and small layers.  Measured, that one and this: 128 x 3 x 64 x 64 11 x 11 stride 4 32 and 132 us, 128 x 2 x 80 x 80 31 x 31
+  // stride 5 106 and 823, 1024 channels 1 x 1 on 7 x 7 11 and 24; 128 x 8 x 56 x 56 7 x 7 285 and 125, 128 x 128 x 28 x 28 3 x 3 215 and 33.
+  const double staged = 3.0 + 0.0037 * a.n + patches * (0.25 + 0.0015 * a.n + 0.002 * d.C * d.stride_h * d.stride_w) / 1000.0;
+  const bool tiled = choose_sign_tile(&a, &smem, &us);
+  if (!tiled || staged < us) {
+    const cudaError_t e = launch_sign_patches_staged(d, Ho, Wo, x, pK, pgamma, pdelta, pmask, ldp, pflags, stream);
+    if (e != cudaErrorInvalidValue) return e;
+  }
+  if (!tiled) {
+    const int64_t blocks = ((int64_t)patches + kSignWarps - 1) / kSignWarps;
     sign_wide_patches_kernel<<<(unsigned)(blocks < sm_count() * 16 ? blocks : sm_count() * 16), kSignThreads, 0, stream>>>(a);
     return cudaGetLastError();
   }
