@@ -26,17 +26,17 @@ __device__ __forceinline__ float post_affine(const PostOp& o, float v, int chann
   return (float)__dadd_rn(__dmul_rn((double)__ldg(o.a + channel), (double)v), (double)__ldg(o.b + channel));
 }
 
-// at: the element's place in the tensor (all tensors of the chain have one shape).
-__device__ __forceinline__ float apply_post_op(const PostOp& o, float v, int channel, int64_t at) {
+// at: the element's place in the tensor (all tensors of the chain have one shape); extent: elements of it.
+__device__ __forceinline__ float apply_post_op(const PostOp& o, float v, int channel, int64_t at, int64_t extent = INT64_MAX) {
   if (o.kind == kPostAffine) v = post_affine(o, v, channel);
   else if (o.kind == kPostRelu) v = v > 0.0f ? v : 0.0f;
-  else if (o.kind == kPostAdd) v = __fadd_rn(v, o.a[at]);
-  else o.to[at] = v;
+  else if (o.kind == kPostAdd) v = __fadd_rn(v, o.a[DAB_IDX(at, extent)]);
+  else if (DAB_IN_BOUNDS(at, extent)) o.to[at] = v;
   return v;
 }
-__device__ __forceinline__ float apply_post(const PostOps& ops, float v, int channel, int64_t at) {
+__device__ __forceinline__ float apply_post(const PostOps& ops, float v, int channel, int64_t at, int64_t extent = INT64_MAX) {
 #pragma unroll 1
-  for (int k = 0; k < ops.count; ++k) v = apply_post_op(ops.op[k], v, channel, at);
+  for (int k = 0; k < ops.count; ++k) v = apply_post_op(ops.op[k], v, channel, at, extent);
   return v;
 }
 

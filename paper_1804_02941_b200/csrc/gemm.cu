@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) binary_gemm_kernel(const GemmArg
         const int64_t to = (gi / g.map.inner) * g.map.outer_stride + (gi % g.map.inner) * g.map.row_stride + gj * g.map.col_stride;
         const float y = decltype(each_pair)::value ? rescale_any(g, p11, gi, gj) : rescale(p11, weight(gj), activation(gi));
         if (!decltype(each_pair)::value) gathered = gathered && weight_gathers(gj) && activation_gathers(gi);
-        if (DAB_IN_BOUNDS(to, g.c_extent)) g.C[to] = apply_post(g.post, y, (int)gj, to);
+        if (DAB_IN_BOUNDS(to, g.c_extent)) g.C[to] = apply_post(g.post, y, (int)gj, to, g.c_extent);
         if (g.p11 && DAB_IN_BOUNDS(gi * g.ldp + gj, (g.M - 1) * g.ldp + g.N)) g.p11[gi * g.ldp + gj] = p11;
       }
     };
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) binary_gemm_kernel(const GemmArg
       int p11 = ones[i][j] + 2 * twos[i][j];
       if (DAB_IN_BOUNDS(base + gj * g.map.col_stride, g.c_extent))
         g.C[base + gj * g.map.col_stride] =
-            apply_post(g.post, rescale(p11, side[j], act), (int)gj, base + gj * g.map.col_stride);
+            apply_post(g.post, rescale(p11, side[j], act), (int)gj, base + gj * g.map.col_stride, g.c_extent);
       if (g.p11 && DAB_IN_BOUNDS(gi * g.ldp + gj, (g.M - 1) * g.ldp + g.N)) g.p11[gi * g.ldp + gj] = p11;
     }
   }
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) binary_gemm_kernel(const GemmArg
       if (gi >= g.M || gj >= g.N) continue;
       const int64_t to = place(gi, gj);
       if (DAB_IN_BOUNDS(to, g.c_extent))
-        g.C[to] = apply_post(g.post, rescale_any(g, __float_as_int(g.C[to]), gi, gj), (int)gj, to);
+        g.C[to] = apply_post(g.post, rescale_any(g, __float_as_int(g.C[to]), gi, gj), (int)gj, to, g.c_extent);
     }
   }
 }

@@ -78,7 +78,7 @@ __device__ __forceinline__ void store_columns(const GemmArgs& g, uint32_t (&v)[3
       if (!DAB_IN_BOUNDS(to, g.c_extent)) continue;
       const int p11 = __float_as_int(g.C[to]);
       const float y = kLanesAreActivations ? rescale_any(g, p11, gl, at) : rescale_any(g, p11, at, gl);
-      g.C[to] = kPost ? apply_post(g.post, y, (int)at, to) : y;
+      g.C[to] = kPost ? apply_post(g.post, y, (int)at, to, g.c_extent) : y;
       if (g.p11 && DAB_IN_BOUNDS(pblock + jj * pstep, (g.M - 1) * g.ldp + g.N)) g.p11[pblock + jj * pstep] = p11;
     }
     return;
@@ -109,7 +109,7 @@ __device__ __forceinline__ void store_columns(const GemmArgs& g, uint32_t (&v)[3
 #pragma unroll
       for (int jj = 0; jj < 32; ++jj) {
         if (jj >= left) break;
-        v[jj] = __float_as_uint(apply_post_op(o, __uint_as_float(v[jj]), (int)first + jj, at + jj * step));
+        v[jj] = __float_as_uint(apply_post_op(o, __uint_as_float(v[jj]), (int)first + jj, at + jj * step, g.c_extent));
       }
     }
 #pragma unroll
@@ -334,19 +334,19 @@ __global__ void __launch_bounds__(WIDE_THREADS, 2) binary_gemm_wide_kernel(const
   const int quarter = warp & 3, half = warp >> 2;
   const int64_t gl = i0 + quarter * 32 + lane;
   const bool row_in = gl < L.rows;
-  const uint32_t* const row = L.mask + (row_in ? gl : 0) * (int64_t)L.ld + 4 * half;
+  const int64_t row_at = (row_in ? gl : 0) * (int64_t)L.ld + 4 * half;
   const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
   // column side: thread = row and two words; eight neighbouring threads write 128 contiguous bytes
   const int crow = (tid >> 4) * 8 + (tid & 7), piece = (tid >> 3) & 1;
   const bool col_in = crow < nrows;
-  const uint32_t* const column = S.mask + (j0 + (col_in ? crow : 0)) * (int64_t)S.ld + 4 * piece;
+  const int64_t col_at = (j0 + (col_in ? crow : 0)) * (int64_t)S.ld + 4 * piece;
   const int chunks = (g.words + WIDE_WORDS - 1) / WIDE_WORDS, real_words = (g.n + 31) >> 5;
 
   uint4 qa, qb;
   auto fetch = [&](int c) {
     const int w = c * WIDE_WORDS;
-    qa = row_in && w + 4 * half < g.words ? __ldg(reinterpret_cast<const uint4*>(row + w)) : make_uint4(0, 0, 0, 0);
-    qb = col_in && w + 4 * piece < g.words ? __ldg(reinterpret_cast<const uint4*>(column + w)) : make_uint4(0, 0, 0, 0);
+    qa = row_in && w + 4 * half < g.words ? __ldg(reinterpret_cast<const uint4*>(L.mask + DAB_IDX(row_at + w, L.rows * L.ld - 3))) : make_uint4(0, 0, 0, 0);
+    qb = col_in && w + 4 * piece < g.words ? __ldg(reinterpret_cast<const uint4*>(S.mask + DAB_IDX(col_at + w, S.rows * S.ld - 3))) : make_uint4(0, 0, 0, 0);
   };
   bool dead = false;
   if (warp == WIDE_WORKERS / 32) {  // the last warp issues the products

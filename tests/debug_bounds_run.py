@@ -77,6 +77,26 @@ def main():
         calls += 1
     dab.dab_set_patch_coder(dab.PATCHES_AUTO)
     dab.dab_set_contraction(dab.CONTRACT_AUTO)
+    # the contraction of long rows (tiles of 128 x 128 for every SM, ragged on both sides), row-major and behind a convolution
+    for M, N, n in ((1793, 2690, 2303), (2690, 1793, 1025)):
+        a = dab.dab_binarize(to_dev(dab_synth.normal((M, n), 1.0, stream=600 + n)))
+        b = dab.dab_binarize(to_dev(dab_synth.normal((N, n), 1.0, stream=601 + n)))
+        dab.dab_binary_gemm(a, b, want_p11=True)
+        dab.dab_binary_conv(to_dev(dab_synth.normal((M, n, 1, 1), 1.0, stream=602 + n)), b, 1, 1)
+        calls += 2
+    # a network's elementwise layers in the kernels before them: shortcuts, remembered and kept tensors, over both contractions
+    conv = lambda k: {"kind": "conv_binary", "w": dab_synth.normal((130, 130 * 9), 0.05, stream=620 + k), "kh": 3, "kw": 3,
+                      "stride": (1, 1), "pad": (1, 1), "Cout": 130}
+    affine = {"kind": "affine", "scale": dab_synth.normal((130,), 1.0, stream=630), "shift": dab_synth.normal((130,), 1.0, stream=631)}
+    layers = [{"kind": "save"}, conv(0), affine, {"kind": "relu"}, conv(1), affine, {"kind": "add"}, {"kind": "relu"}, {"kind": "save"},
+              conv(2), {"kind": "add"}, {"kind": "relu"}]
+    for batch in (1, 20):
+        for path in (dab.CONTRACT_TENSOR, dab.CONTRACT_POPC, dab.CONTRACT_AUTO):
+            dab.dab_set_contraction(path)
+            x = to_dev(dab_synth.normal((batch, 130, 31, 33), 1.0, stream=640))
+            dab.dab_network_forward(dab.Network(layers), x, keep_layers=True, layer_shapes=[(130, 31, 33)] * len(layers))
+            calls += 1
+    dab.dab_set_contraction(dab.CONTRACT_AUTO)
     torch.cuda.synchronize()
     report = dab.dab_debug_bounds_report(reset=True)
     report.update(calls=calls, compared=compared, wait_failures=int(dab.dab_contraction_wait_failures()))
