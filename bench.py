@@ -27,7 +27,8 @@ WORDS_PER_POPC = 1.5              # the contraction compresses 3 AND-ed words in
 
 
 # Sources of the patch coder: a measured DRAM-traffic record is only quoted while these files are unchanged.
-PATCH_CODER_SOURCES = ("pixtile.cu", "patchrows.cu", "patches.cu", "rowbucket.cuh", "rowcode.cuh", "common.cuh")
+PATCH_CODER_SOURCES = ("pixtile.cu", "patchrows.cu", "patches.cu", "binarize.cu", "rowbucket.cuh", "bucket_bound.cuh", "histcode.cuh",
+                       "rowcode.cuh", "common.cuh")
 TRAFFIC_RECORD = os.path.join(ROOT, "profiles", "patch_coder_dram_traffic.json")
 
 
@@ -68,8 +69,8 @@ def parse_args():
                     help="contraction kernel: auto (tensor cores except on tiny problems; every layer of this workload takes "
                          "them), tensor (forced) or popc (AND + population counts)")
     ap.add_argument("--patch-coder", default="auto", choices=["auto", "sort", "hist", "pixel"],
-                    help="patch coder: auto (pixel-histogram coder wherever patches overlap), sort (full sort per patch), "
-                         "hist (histogram-pruned search per patch) or pixel (pixel-histogram coder wherever it applies)")
+                    help="patch coder: auto (tile coder wherever patches overlap and are many), sort (full sort per patch), "
+                         "hist (histogram-pruned search per patch) or pixel (tile coder wherever it applies)")
     ap.add_argument("--filters", default="side", choices=["side", "inline"],
                     help="side: the filter coding of all layers runs on a second stream beside the patch coding (each "
                          "contraction waits for its filters); inline: everything on one stream, layer by layer")
@@ -233,13 +234,13 @@ def patch_launches(L, coder):
     n = L.n
     if n <= 256:
         return 1
-    pixel = n <= 8192 and L.kh * L.kw >= 4 and L.patches >= 1024
-    if coder == "pixel" or (coder == "auto" and pixel):
-        # tile coder, then the kernel that codes the patches it marked; long rows of strided windows, which share little, may go to
-        # a CTA per patch at once (a lower bound)
-        return 1 if coder == "auto" and L.stride > 1 and n > 2048 else 2
+    tiles = n <= 8192 and L.C <= 2048 and L.kh * L.kw <= 64
+    if coder == "pixel" and tiles:
+        return 2                      # tile coder, then the kernel that codes the patches it marked
     if coder == "auto" and (L.kh * L.kw >= 4 or L.patches < 1024 or n > 8192):
-        return 1                      # a CTA per patch
+        # The same from some thousand patches on (the library estimates both), below a CTA per patch: 1, a lower bound there.
+        # Every layer of the default workload is above.
+        return 2 if tiles and L.kh * L.kw >= 4 and L.patches >= 10000 else 1
     if coder == "auto":
         return 3                      # sort-based coder, histogram coder on the dense tiles, group kernel on the rest
     if coder == "hist":

@@ -134,7 +134,7 @@ cudaError_t launch_binarize_patches_tile(const dab_conv_desc& d, int32_t Ho, int
                                          float* pgamma, float* pdelta, uint32_t* pmask, int32_t ldp, uint32_t* pflags,
                                          bool always, cudaStream_t stream, bool* applicable);
 // Patch coder selection: 0 default, 1 sort-based only, 2 histogram-pruned per patch wherever it applies,
-// 3 pixel-histogram coder wherever it applies.
+// 3 tile coder wherever it applies.
 int patch_coder_mode();
 void set_patch_coder_mode(int mode);
 constexpr int32_t kRowMark = -1;  // K of a row or of a tile's first patch that the next kernel of a chain has to code

@@ -1,6 +1,6 @@
 // Patches through the bucket-pruned search of rowbucket.cuh, a CTA per patch whose values are gathered straight from the
 // image: layers with too few patches for the tile coders to fill the device (batch 1, fully connected layers; a chain
-// of three mostly idle kernels before), and the patches that the pixel-histogram coder marked (a sort of 8 warps each
+// of three mostly idle kernels before), and the patches that the tile coder marked (a sort of 8 warps each
 // before).  Latency bounds the first use, the search of rowbucket.cuh the second.  Measured, before -> this: the
 // Sketch-A-Net-shaped network at batch 1 581 -> 334 us, its fully connected layer of 12544 values 209 -> 53 us; the
 // marked patches of the AlexNet-shaped network at batch 32 3.0 -> 0.43 ms.

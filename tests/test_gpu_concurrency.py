@@ -1,9 +1,10 @@
 """Calls from two host threads on two streams at once: kernels of one call hand work to each other only through
 that call's own output arrays, so concurrent calls cannot disturb each other, whichever coders they take.
 
-One thread runs a layer that takes the pixel-histogram coder, the other a small layer that takes the chain of
-sorting and per-patch histogram kernels (tiles handed on through marks) while the process-wide coder choice is
-switched back and forth; every result must equal the one obtained alone, and the first ones the CPU checker's.
+One thread runs a layer that takes the tile coder and the kernel for the patches it marks (an image of few distinct values is
+marked throughout), the other a small layer that takes a CTA per patch, the chain of sorting and per-patch histogram kernels
+(tiles handed on through marks) or the tile coder as the process-wide coder choice is switched back and forth; every result must
+equal the one obtained alone, and the first ones the CPU checker's.
 """
 import threading
 
@@ -29,13 +30,15 @@ def dab():
 
 
 def test_two_threads_two_streams(dab):
-    big = configs.ConvLayer("big", 4, 64, 20, 20, 32, 3, 3, 1, 1, 0.05)        # 1600 patches: pixel-histogram coder
-    small = configs.ConvLayer("small", 1, 128, 14, 14, 16, 3, 3, 1, 1, 0.05)   # 196 patches: the marking chain
+    big = configs.ConvLayer("big", 24, 64, 20, 20, 32, 3, 3, 1, 1, 0.05)       # 9600 patches: the tile coder
+    small = configs.ConvLayer("small", 1, 128, 14, 14, 16, 3, 3, 1, 1, 0.05)   # 196 patches: a CTA per patch
     jobs = []
     for L, dense in ((big, False), (small, True)):
         x = L.inputs(stream=500, dense=dense)
         if dense:
             x[:, :, :7] = L.inputs(stream=501)[:, :, :7]                       # sparse and dense tiles in one image
+        else:
+            x[5] = np.where(x[5] > 0.3, 0.5, -0.25)                            # hulls of some hundred values: marked
         w = L.weights(stream=500)
         wd = dab.dab_binarize(to_dev(w))
         xd = to_dev(x)
