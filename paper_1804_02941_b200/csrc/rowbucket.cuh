@@ -15,8 +15,8 @@
 // 2^-40..2^40) have the distinct values of their hull counted; where those are many, the row is sorted in place by the whole CTA and
 // every split is evaluated.  Sorted before: 512 rows of 4608 values -1, 0, 1 152 -> 29 us, 512 of 16384 values 0, 1 650 -> 109 us.
 //
-// Bound by instruction issue (60 % of the slots, ALU pipe 55 %) and the barriers between the passes; about 70 warp
-// instructions per 32 values.  It replaced a sorting network over the whole row with up to 32 warps per row, and a
+// Bound by instruction issue (61 % of the slots, ALU pipe 49 %) and the barriers between the passes; 100 warp
+// instructions per 32 values in rows of 4608.  It replaced a sorting network over the whole row with up to 32 warps per row, and a
 // one-warp histogram for large matrices.  Measured, before -> this: 4096 x 9216 N(0, 1) 4.27 -> 0.128 ms (1.2 TB/s of
 // values read), 8192 x 4608 Laplace 1.05 -> 0.22 ms, 4096 x 2304 0.22 -> 0.066 ms, 512 x 4608 0.114 -> 0.023 ms.
 #pragma once
@@ -51,6 +51,7 @@ struct __align__(16) BlockShared {  // (a multiple of 16 bytes: the staged value
   int wlo[W], whi[W], wbestS[W];
   uint32_t wbestT[W];
   int c_below, c_upto, fill, overflow;
+  uint32_t hull_first, hull_last;  // keys; 0: the segments that can hold the best split are not known
   RowResult result;
 };
 
@@ -338,7 +339,7 @@ __device__ __forceinline__ void block_code_row(const Source& source, int n, unsi
   // ---- stage the row; largest magnitude ----
 #pragma unroll
   for (int j = 0; j < 2 * PB; ++j) hist[j * T + tid] = 0u;
-  if (tid == 0) bs->fill = bs->overflow = 0;
+  if (tid == 0) { bs->fill = bs->overflow = 0; bs->hull_last = 0u; }
   const int words = (n + 31) >> 5, quads = 8 * words;
   uint32_t top = source.template stage<T>(vals, quads, bs);
   top = __reduce_max_sync(0xFFFFFFFFu, top);
@@ -352,8 +353,7 @@ __device__ __forceinline__ void block_code_row(const Source& source, int n, unsi
   if (top >= 0x7F800000u || top == 0u) {
     res = trivial_row(top != 0u, 0.0f);
   } else {
-    bool retry = e < -40 || e > 40, hull = false;  // hull: the segments that can hold the best split are known
-    uint32_t hull_first = 0u, hull_last = kPadKey;
+    bool retry = e < -40 || e > 40;
     const int base = (int)(top >> SHIFT) - (NB - 1);
     int m_sub = 0, z_in = 0, s_below = 0;
     double T_row = 0.0;
@@ -528,10 +528,9 @@ __device__ __forceinline__ void block_code_row(const Source& source, int n, unsi
           }
         }
         // ---- gather the hull: values from the smallest of bucket b_lo to the largest of bucket b_hi, zeros left out ----
-        hull = true;
-        hull_first = bucket_first_key<SHIFT>(b_lo, NB, base);
-        hull_last = bucket_last_key<SHIFT>(b_hi, NB, base);
-        const float vfirst = key_value(hull_first), vlast = key_value(hull_last);
+        const uint32_t first = bucket_first_key<SHIFT>(b_lo, NB, base), last = bucket_last_key<SHIFT>(b_hi, NB, base);
+        if (tid == 0) { bs->hull_first = first; bs->hull_last = last; }
+        const float vfirst = key_value(first), vlast = key_value(last);
         const unsigned lt = (1u << lane) - 1u;
 #pragma unroll 2
         for (int q0 = warp * 32; q0 < quads; q0 += T) {
@@ -577,9 +576,12 @@ __device__ __forceinline__ void block_code_row(const Source& source, int n, unsi
       retry = bs->result.tkey == kPadKey;  // a split at the hull's outer edge won: not certified
     }
     if (retry) {
+      const uint32_t first = bs->hull_first, last = bs->hull_last;
+      const bool hull = last != 0u;
       const double P_below = hull ? bs->P_below : 0.0;
       __syncthreads();
-      if (!block_distinct_code<T>(vals, n, hist, hull_first, hull_last, !hull || z_in > 0, s_below, P_below, T_row, !hull || m_sub + z_in == n, bs)) {
+      if (!block_distinct_code<T>(vals, n, hist, hull ? first : 0u, hull ? last : kPadKey, !hull || z_in > 0, s_below, P_below, T_row,
+                                  !hull || m_sub + z_in == n, bs)) {
         block_sort_code<T>(reinterpret_cast<uint32_t*>(vals), n, bs);
         source.template restage<T>(vals, quads);  // for the mask
         __syncthreads();
