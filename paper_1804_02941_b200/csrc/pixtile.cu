@@ -985,22 +985,15 @@ double choose_tile(TileArgs* a, size_t* smem_out, double* cost_out) {
   return (int64_t)a->tiles_h * a->tiles_w * a->d.N <= 0x7FFFFFFF ? whole : 0.0;
 }
 
+// budget: cycles that the tiles may take.
 template <int KHW, int BPL, typename ListT>
-cudaError_t launch_tile(TileArgs& a, bool always, cudaStream_t stream, bool* applicable) {
+cudaError_t launch_tile(TileArgs& a, double budget, cudaStream_t stream, bool* applicable) {
   a.buckets = 32 * BPL;
   a.octaves = BPL == 1 ? 8 : 12;
-  // A layer of few patches is done sooner by a CTA per patch: about 15000 cycles and 5 + 0.012 n per patch, where this kernel
-  // has 8000 to 35000 on top of its tiles (the kernel for marked patches, code that is not in the cache, longer hulls in longer
-  // rows).  Measured, a CTA per patch and this, post-ReLU; N(0, 1): 2 x 64 x 28 x 28, 1568 patches of 576, 21 and 23 us; 21 and 28;
-  // 4 x 128 x 28 x 28, 3136 of 1152, 45 and 34; 46 and 48; 24 x 128 x 28 x 28 with stride 2, 4704 of 1152, 61 and 50; 62 and 60;
-  // 8 x 256 x 14 x 14, 1568 of 2304, 39 and 32; 38 and 44; 2 x 32 x 27 x 27 5 x 5, 1458 of 800, 23 and 26; 25 and 32.
-  const double by_patch = always ? 1e30 : 15000.0 + (5.0 + 0.012 * a.n) * (double)a.d.N * a.Ho * a.Wo;
-  const double set_up = (a.n < 1300 ? 5000.0 + 10.0 * a.n : 15000.0 + 2.4 * a.n) + (a.d.kh * a.d.kw > 9 ? 8000.0 : 0.0);
-  if (by_patch < set_up) return cudaSuccess;
   size_t smem = 0;
   double cost;
   const double cycles = choose_tile<ListT>(&a, &smem, &cost);
-  if (cycles == 0.0 || by_patch < set_up + cycles) return cudaSuccess;
+  if (cycles == 0.0 || budget < cycles) return cudaSuccess;
   auto kern = binarize_patches_tile_kernel<KHW, BPL, ListT>;
   cudaError_t e = ensure_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
@@ -1015,6 +1008,19 @@ cudaError_t launch_tile(TileArgs& a, bool always, cudaStream_t stream, bool* app
 // small gain, since N(0, 1) rows lose: 64 x 256 x 28 x 28 3 x 3 stride 2 (estimated gain 1.13) 213 -> 170, 207 -> 233.
 template <int KHW, typename ListT>
 cudaError_t launch_tile_buckets(TileArgs& a, bool always, cudaStream_t stream, bool* applicable) {
+  // A layer of few patches is done sooner by a CTA per patch: about 15000 cycles and 5 + 0.012 n per patch, where this kernel
+  // has 8000 to 35000 on top of its tiles (the kernel for marked patches, code that is not in the cache, longer hulls in longer
+  // rows).  Measured, a CTA per patch and this, post-ReLU; N(0, 1): 2 x 64 x 28 x 28, 1568 patches of 576, 21 and 23 us; 21 and 28;
+  // 4 x 128 x 28 x 28, 3136 of 1152, 45 and 34; 46 and 48; 24 x 128 x 28 x 28 with stride 2, 4704 of 1152, 61 and 50; 62 and 60;
+  // 8 x 256 x 14 x 14, 1568 of 2304, 39 and 32; 38 and 44; 2 x 32 x 27 x 27 5 x 5, 1458 of 800, 23 and 26; 25 and 32;
+  // 32 x 256 x 14 x 14 with stride 2, 1568 of 2304, 38 and 45; 38 and 46.
+  const double by_patch = 15000.0 + (5.0 + 0.012 * a.n) * (double)a.d.N * a.Ho * a.Wo;
+  const double set_up = (a.n < 1300 ? 5000.0 + 10.0 * a.n : 15000.0 + 2.4 * a.n) + (a.d.kh * a.d.kw > 9 ? 8000.0 : 0.0) +
+                        (a.n >= 1536 && a.d.stride_h * a.d.stride_w > 1 ? 10000.0 : 0.0);
+  const double budget = always ? 1e30 : by_patch - set_up;
+  // Less than choose_tile estimates for any tile: the smallest calls are spared its trying all of them (1.6 us of 25 on the host for
+  // 64 x 32 x 32 at batch 1).
+  if (budget < 20000.0 + 6000.0 * (0.6 + 0.4 * a.d.kh * a.d.kw / 9.0)) return cudaSuccess;
   bool longer = a.n >= 1536;
   if (longer && a.d.stride_h * a.d.stride_w > 1) {
     double cost[2];
@@ -1026,7 +1032,7 @@ cudaError_t launch_tile_buckets(TileArgs& a, bool always, cudaStream_t stream, b
     }
     longer = cost[0] == 0.0 || (cost[1] > 0.0 && cost[1] <= (KHW == 9 ? 1.25 : 1.15) * cost[0]);
   }
-  return longer ? launch_tile<KHW, 2, ListT>(a, always, stream, applicable) : launch_tile<KHW, 1, ListT>(a, always, stream, applicable);
+  return longer ? launch_tile<KHW, 2, ListT>(a, budget, stream, applicable) : launch_tile<KHW, 1, ListT>(a, budget, stream, applicable);
 }
 
 }  // namespace
