@@ -373,15 +373,18 @@ dab_contraction dab_get_contraction(void);
  *                      at the corners of the region the bucket's count, sum and value bounds allow; only the few
  *                      buckets whose bound reaches the best edge value are searched exactly.  Work per pixel is
  *                      shared by the up to kh*kw patches that contain it.  Patches it cannot settle (a hull of more
- *                      than 1023 values, a constant row without zeros, magnitudes outside 2^-40..2^40, a NaN or an
- *                      infinity in the tile) are coded by a second kernel, a CTA per patch.  At most 512 channels and 32
- *                      pixels per window;
+ *                      than 511 values, 1023 in patches of 1536 values and more, a constant row without zeros, magnitudes
+ *                      outside 2^-40..2^40, a NaN or an infinity in the tile) are coded by a second kernel, a CTA per
+ *                      patch.  At most 2048 channels and 64 pixels per window;
  *   DAB_PATCHES_HIST   patches of 257..8192 values, one warp each: a histogram of the patch's own values
  *                      quantised to 24 bits of the tile's range, the same bound per bucket with a margin for the
  *                      quantisation, exact search of what survives; what it cannot settle falls to the sorting kernel.
- *                      Rows of a matrix of more than 256 values: a CTA per row, exact counts and sums per bucket;
- *   DAB_PATCHES_AUTO   (default) patches: DAB_PATCHES_PIXEL for windows of at least four pixels; layers of few patches and
- *                      patches of more than 8192 values a CTA per patch, which prunes by buckets of its own; windows of one to
+ *                      Rows of a matrix of more than 256 values: a CTA per row (a warp where there are many of up to 512
+ *                      values), exact counts and sums per bucket; of what that leaves, rows of few distinct values by
+ *                      counting them, the others by sorting;
+ *   DAB_PATCHES_AUTO   (default) patches of up to 256 values: a warp each, sorted in full; longer ones: DAB_PATCHES_PIXEL for
+ *                      windows of at least four pixels; layers of few patches and patches that coder does not take (more than
+ *                      8192 values) a CTA per patch, which prunes by buckets of its own; windows of one to
  *                      three pixels in larger layers per tile of the input the sorting kernels for tiles with few
  *                      non-zero values and DAB_PATCHES_HIST for the others.  Rows of a matrix: DAB_PATCHES_HIST.
  * Process-wide, read once at the start of each call.

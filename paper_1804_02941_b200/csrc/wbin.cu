@@ -19,8 +19,8 @@
 // SM, or a wide window leaves no room, the operands are not: see launch_wbin_conv.)
 //
 // Bound by shared memory: per stage of 128 elements and 128 filters the tensor cores read 128 KB of operands, the gather
-// 64 KB of values (twice where lanes of a warp lie in different output rows) and writes 64 KB.  The conversion, some 8
-// instructions per element, is what a CTA of 128 filters halves over one of 64.
+// 64 KB of values (twice where lanes of a warp lie in different output rows) and writes 64 KB.  An element takes some 20
+// instructions in all, the 8 or so of its conversion among them; a CTA of 128 filters halves that over one of 64.
 #include <algorithm>
 #include <climits>
 

@@ -1,5 +1,4 @@
-"""The tensor-core contraction of long rows, tiles of 256 x 128: row and column remainders, a second accumulator without rows,
-row lengths around its stages of 256 bits, both output layouts.  Rows at the edges of tiles against the CPU checker (counts bit
+"""The tensor-core contraction of long rows, tiles of 128 x 128: row and column remainders, row lengths around its stages of 256 bits, both output layouts.  Rows at the edges of tiles against the CPU checker (counts bit
 for bit, outputs within 1e-5 relative: one rounding of the same fp64 sum each), everything bit for bit against population counts."""
 import numpy as np
 import pytest
