@@ -22,8 +22,9 @@ struct PostOps {
   PostOp op[kMaxPostOps];
 };
 
+// One rounding of the exact scale * v + shift (in fp64 the sum was rounded twice, and the three conversions cost more than the store).
 __device__ __forceinline__ float post_affine(const PostOp& o, float v, int channel) {
-  return (float)__dadd_rn(__dmul_rn((double)__ldg(o.a + channel), (double)v), (double)__ldg(o.b + channel));
+  return __fmaf_rn(__ldg(o.a + channel), v, __ldg(o.b + channel));
 }
 
 // at: the element's place in the tensor (all tensors of the chain have one shape); extent: elements of it.
