@@ -271,28 +271,71 @@ cudaError_t launch_glue(const float* x, int32_t N, int32_t C, int64_t plane, con
   return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(kGlueThreads) maxpool_kernel(dab_conv_desc d, int Ho, int Wo, const float* __restrict__ x,
-                                                               const PostOps post, float* __restrict__ y) {
+// i / d: by multiply-high where the magic number is exact for the whole range (0: it is not).
+__host__ inline uint32_t magic_for(int64_t count, int64_t d) { return d > 1 && count * d < 0x100000000ll ? (uint32_t)((0x100000000ull + d - 1) / d) : 0u; }
+__device__ __forceinline__ int64_t divide(int64_t i, int d, uint32_t magic) { return magic ? (int64_t)__umulhi((unsigned)i, magic) : i / d; }
+
+// K x K windows unrolled, all loads of an output in flight together (K = 0: any window, four loads at a time).  The first value of the window
+// counts as it is and a later one if it is larger, in this order.
+// 32 x 64 x 112 x 112, 3 x 3 stride 2, is 130 MB, 20 us at the memory's rate: 51 us (with 64-bit divisions and a
+// load at a time 104); 32 x 96 x 55 x 55 18 (37).
+template <int K>
+__global__ void __launch_bounds__(kGlueThreads) maxpool_kernel(dab_conv_desc d, int Ho, int Wo, uint32_t magic_wo, uint32_t magic_ho, uint32_t magic_c,
+                                                               const float* __restrict__ x, const PostOps post, float* __restrict__ y) {
   const int64_t outputs = (int64_t)d.N * d.C * Ho * Wo;
+  const int kh = K ? K : d.kh, kw = K ? K : d.kw;
   for (int64_t oi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; oi < outputs; oi += (int64_t)gridDim.x * blockDim.x) {
-    const int wo = (int)(oi % Wo);
-    const int ho = (int)((oi / Wo) % Ho);
-    const int64_t plane = oi / ((int64_t)Wo * Ho);
-    const float* xp = x + plane * d.H * d.W;
+    const int64_t line = divide(oi, Wo, magic_wo), plane = divide(line, Ho, magic_ho);
+    const int h0 = (int)(line - plane * Ho) * d.stride_h - d.pad_h, w0 = (int)(oi - line * Wo) * d.stride_w - d.pad_w;
+    const float* const xp = x + plane * d.H * d.W + (int64_t)h0 * d.W + w0;
     bool seen = false;
     float best = 0.0f;
-    for (int r = 0; r < d.kh; ++r)
-      for (int s = 0; s < d.kw; ++s) {
-        const int h = ho * d.stride_h - d.pad_h + r, wq = wo * d.stride_w - d.pad_w + s;
-        if ((unsigned)h < (unsigned)d.H && (unsigned)wq < (unsigned)d.W) {
-          const float v = xp[(int64_t)h * d.W + wq];
-          if (!seen || v > best) best = v;
-          seen = true;
+    auto take = [&](float v, bool in) {
+      if (in && (!seen || v > best)) best = v;
+      seen = seen || in;
+    };
+    if (K) {
+      float v[K ? K * K : 1];
+      bool in[K ? K * K : 1];
+#pragma unroll
+      for (int i = 0; i < K * K; ++i) {
+        const int r = i / (K ? K : 1), s = i % (K ? K : 1);
+        in[i] = (unsigned)(h0 + r) < (unsigned)d.H && (unsigned)(w0 + s) < (unsigned)d.W;
+        v[i] = in[i] ? __ldg(xp + (int64_t)r * d.W + s) : 0.0f;
+      }
+#pragma unroll
+      for (int i = 0; i < K * K; ++i) take(v[i], in[i]);
+    } else {
+      for (int r = 0; r < kh; ++r) {
+        if ((unsigned)(h0 + r) >= (unsigned)d.H) continue;
+        for (int s = 0; s < kw; s += 4) {
+          float v[4];
+          bool in[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            in[j] = s + j < kw && (unsigned)(w0 + s + j) < (unsigned)d.W;
+            v[j] = in[j] ? __ldg(xp + (int64_t)r * d.W + s + j) : 0.0f;
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) take(v[j], in[j]);
         }
       }
-    if (post.count > 0) best = apply_post(post, best, (int)(plane % d.C), oi);
+    }
+    if (post.count > 0) best = apply_post(post, best, (int)(plane - divide(plane, d.C, magic_c) * d.C), oi);
     y[oi] = best;
   }
+}
+
+cudaError_t launch_maxpool(const dab_conv_desc& d, int Ho, int Wo, const float* x, const PostOps& post, float* y, cudaStream_t stream) {
+  const int64_t planes = (int64_t)d.N * d.C, outputs = planes * Ho * Wo;
+  const uint32_t magic_wo = Wo > 1 ? magic_for(outputs, Wo) : 0u, magic_ho = magic_for(planes * Ho, Ho), magic_c = magic_for(planes, d.C);
+  auto run = [&](auto kernel) {
+    kernel<<<glue_blocks(outputs), kGlueThreads, 0, stream>>>(d, Ho, Wo, magic_wo, magic_ho, magic_c, x, post, y);
+    return cudaGetLastError();
+  };
+  if (d.kh == 3 && d.kw == 3) return run(maxpool_kernel<3>);
+  if (d.kh == 2 && d.kw == 2) return run(maxpool_kernel<2>);
+  return run(maxpool_kernel<0>);
 }
 
 inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -479,8 +522,7 @@ dab_status dab_network_forward(const dab_layer* layers, int32_t count, int32_t N
         break;
       }
       case DAB_LAYER_MAXPOOL:
-        maxpool_kernel<<<glue_blocks(out.count(N)), kGlueThreads, 0, cs>>>(d, out.H, out.W, src, post, dst);
-        e = cudaGetLastError();
+        e = launch_maxpool(d, out.H, out.W, src, post, dst, cs);
         break;
       default:
         e = launch_glue(src, N, out.C, (int64_t)out.H * out.W, post, dst, cs);
