@@ -47,14 +47,13 @@ constexpr int kTinyBits = 51;
 // From this many pixels on a thread sums a pixel's buckets one after another; below it would leave most of them idle (4200 cycles for
 // 20 pixels where a warp per pixel takes 1500; at 100 pixels both take 5000, at 130 the warps 7000 to 10000).
 constexpr int kSerialPixels = 80;
-// Values the search of one patch takes at most; longer hulls are left to the CTA-per-patch kernel.  Short rows hardly have any, and a
-// search of 1024 in registers makes the kernel slower for all: 64 x 64 x 56 x 56 post-ReLU 426 us with it, 416 without; values
-// e^(4 N(0, 1)) 3.18 and 1.27 ms.  Longer rows need it: 61 x 256 x 14 x 14 N(0, 1) 131 us without it, 121 with.
-template <int BPL>
-__host__ __device__ constexpr int hull_cap() { return BPL == 1 ? 512 : 1024; }
+// Hulls of 64 values and more are narrowed before they are sorted in short rows; in longer ones, where a warp has three or four patches of a
+// tile and one that cannot be narrowed holds up the others, sorted: 61 x 256 x 14 x 14 N(0, 1) 117 us, 124 narrowed; 32 x 256 x 13 x 13 of a
+// network 95 and 118, 32 x 384 x 13 x 13 156 and 134.
 // A bucket is kept if its bound reaches the best edge objective times this: edges and inner corners are formed in fp32 from
 // sums rounded once (1e-6 relative), the place of a corner to 4e-7 of the bucket's count.
 constexpr float kKeep = 0.9999f;
+constexpr float kWeak = 1e-13f;             // relative difference of objectives that their rounding (4e-16) stays far below
 constexpr double kCloseBand = 1.0 - 1e-11;  // objectives this close are compared in their exactly rounded form
 
 struct TileArgs {
@@ -82,11 +81,16 @@ __device__ __forceinline__ int64_t patch_count(const TileArgs& a) { return (int6
 
 // The bucket grid of a tile, in shared memory.  Steps and cells ascend in value over both signs.
 struct Grid {
-  double elo[kMaxBuckets];       // signed start of the bucket's octave and signed unit of the mantissas there:
-  double ulp[kMaxBuckets];       // sum of a bucket = count * elo + sum of the mantissas * ulp
+  union {
+    struct {
+      double elo[kMaxBuckets];       // signed start of the bucket's octave and signed unit of the mantissas there:
+      double ulp[kMaxBuckets];       // sum of a bucket = count * elo + sum of the mantissas * ulp
+      uint32_t hist[kTileWarps * 32];  // sampled values per cell
+      uint8_t lut[kMaxSteps + 2];    // bucket of a step
+    };
+    uint32_t scratch[kTileWarps][64];  // of each warp's search, once the tables are made
+  };
   float edge[kMaxBuckets + 1];   // ascending; edge[B0] = 0
-  uint32_t hist[kTileWarps * 32];  // sampled values per cell; once the grid is chosen, 32 words for each warp's search
-  uint8_t lut[kMaxSteps + 2];    // bucket of a step
   float part[2][kTileWarps];     // per-warp partial sums
   uint32_t ipart[kTileWarps];
   uint32_t best;                 // largest objective of the sample (bits)
@@ -279,6 +283,152 @@ __device__ __forceinline__ double objective_near(double P, double T, int s, int 
   return P * P * r + Q * Q * q;
 }
 
+// A split of a row as the bucket test sees it: the means of its two sides and the objective, in fp32 from sums rounded once.  A side
+// without values has the bound that its first value would obey (vlo, vhi) as its mean.
+struct SplitState {
+  float lo, hi, d;
+};
+__device__ __forceinline__ SplitState split_state(int s, float P, float Q, int n, float vlo, float vhi) {
+  SplitState e;
+  e.lo = s > 0 ? __fdividef(P, count_to_float(s)) : vlo;
+  e.hi = s < n ? __fdividef(Q, count_to_float(n - s)) : vhi;
+  e.d = __fmaf_rn(e.lo, P, e.hi * Q);  // (at s = 0 and s = n T^2 / n, which no split falls short of)
+  return e;
+}
+
+// Can the best split lie in a bucket?  Two tests of the splits from its lower to its upper edge, the values between them in
+// [vlo, vhi]:
+//   bound   along the chord between the edges' (s, P) the objective is convex, so at most the larger of the edges'.  A split is off
+//           the chord by at most c (vhi - vlo) / 4 =: e in P, where the objective's slope is at most twice the difference of the means
+//           and its curvature adds e (vhi - vlo) at most;
+//   means   a value that is closer to the other side's mean would improve the objective by changing sides, so the best
+//           split's threshold is the middle of its two means.  Both means grow with the split: the middle lies between those of the
+//           edges, and has to be in the bucket.
+// The second alone leaves a few buckets, but far ones too where the objective has several maxima.
+struct BucketTest {
+  float edges, bound, mid_lo, mid_hi, gap;
+  BucketTest() = default;
+  __device__ __forceinline__ BucketTest(const SplitState& L, const SplitState& U, int c, float vlo, float vhi) {
+    const float w = vhi - vlo;
+    edges = fmaxf(L.d, U.d);
+    bound = __fmaf_rn(0.5f * count_to_float(c) * w, U.hi - L.lo + w, edges);
+    mid_lo = 0.5f * (L.lo + L.hi);
+    mid_hi = 0.5f * (U.lo + U.hi);
+    gap = L.hi - U.lo;
+  }
+  // margin: error of the middles.  A split that fails by more is worse than another by 2 * gap * margin; where that is not far above the
+  // rounding of the objective (weak: the gap below which it is not), the test does not count.
+  __device__ __forceinline__ bool passes(float need, float margin, float weak, float vlo, float vhi) const {
+    return bound >= need && ((mid_lo - margin <= vhi && mid_hi + margin >= vlo) || !(gap >= weak));
+  }
+};
+
+// The values of a hull, by the lists of the window's pixels: `step` lanes share a pixel (in wide windows a lane has two).
+template <int KHW, typename ListT>
+struct HullLists {
+  static constexpr int kPerLane = KHW == kWideWindow ? 2 : 1;
+  const ListT* from[kPerLane];
+  const float* values[kPerLane];
+  int count[kPerLane];
+  int sub, step;
+  template <typename F>
+  __device__ __forceinline__ void each(F f) const {  // f(value, is there one), the whole warp together
+#pragma unroll
+    for (int t = 0; t < kPerLane; ++t)
+      for (int k = sub; __any_sync(0xFFFFFFFFu, k < count[t]); k += step) {
+        const bool in = k < count[t];
+        f(in ? values[t][from[t][k]] : 0.0f, in);
+      }
+  }
+};
+
+// A hull as the search ends it: values with lo <= hull_place(value) < hi, `size` of them.
+constexpr uint32_t kPlaces = 1u << 22;  // (the sum of 1023 places fits 32 bits)
+constexpr int kHullMax = 1023;
+struct HullRange {
+  float origin, scale;
+  uint32_t lo, hi;
+  int size;
+};
+__device__ __forceinline__ uint32_t hull_place(float v, float origin, float scale) {  // (grows with v)
+  return min((uint32_t)__float2uint_rz(__fmul_rn(__fsub_rn(v, origin), scale)), kPlaces - 1u);
+}
+
+// Narrows a hull of more than 31 values: they are spread over 32 buckets of equal width, a lane each, and the buckets tested as before,
+// until 31 are left or nothing changes.  Values of `zero` place are z more (0: none).  s_lo, P_lo: count and sum below the hull; best: an objective that is
+// reached; table: 64 words.
+// (Hulls of 32 to 500 values were sorted before, in registers, 2 to 16 values a lane by as many variants of the code; the warps of
+// an SM at different ones waited for instructions half of the time: network inputs, 32 x 64 x 56 x 56, 524 us.)
+template <int KHW, typename ListT>
+__device__ __noinline__ void narrow_hull(const HullLists<KHW, ListT> lists, HullRange* range, uint32_t* table, float vlo, float vhi, int s_lo, double P_lo,
+                                         double T, int n, int z, float best, float margin, int lane) {
+  constexpr unsigned kAll = 0xFFFFFFFFu;
+  HullRange r = *range;
+  r.origin = vlo;
+  r.scale = __fdividef((float)kPlaces, vhi - vlo);
+  r.lo = 0u;
+  r.hi = kPlaces;
+  const float unit = (vhi - vlo) * (1.0f / kPlaces), Tf = (float)T;
+  const uint32_t zero = hull_place(0.0f, r.origin, r.scale);
+  int c_below = 0;          // values of the hull below r.lo, and the sum of their places
+  uint32_t q_below = 0u;
+  for (int level = 0; r.size + (z > 0 ? 1 : 0) > 31; ++level) {
+    const uint32_t span = r.hi - r.lo;
+    const int shift = max(27 - __clz((int)(span - 1u)), 0);  // at most 32 buckets
+    table[lane] = 0u;
+    table[32 + lane] = 0u;
+    __syncwarp();
+    lists.each([&](float v, bool in) {
+      const uint32_t q = hull_place(v, r.origin, r.scale);
+      if (in && q >= r.lo && q < r.hi) {
+        atomicAdd(table + ((q - r.lo) >> shift), 1u);
+        atomicAdd(table + 32 + ((q - r.lo) >> shift), q);
+      }
+    });
+    __syncwarp();
+    const int c = (int)table[lane];
+    const uint32_t qc = table[32 + lane];
+    int c1 = c;
+    uint32_t q1 = qc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int uc = __shfl_up_sync(kAll, c1, o);
+      const uint32_t uq = __shfl_up_sync(kAll, q1, o);
+      if (lane >= o) { c1 += uc; q1 += uq; }
+    }
+    const int c0 = c1 - c;
+    const uint32_t q0 = q1 - qc;
+    // places are rounded: 1.5 units off the middle of one at most
+    auto sum_of = [&](int count, uint32_t places) {
+      return P_lo + int_to_double(count) * ((double)vlo + 0.5 * (double)unit) + (double)places * (double)unit;
+    };
+    const uint32_t from = r.lo + ((uint32_t)lane << shift), to = from + (1u << shift);
+    const float blo = vlo + (float)from * unit, bhi = vlo + (float)to * unit;
+    const double P0 = sum_of(c_below + c0, q_below + q0), P1 = sum_of(c_below + c1, q_below + q1);
+    const int s0 = s_lo + c_below + c0 + (zero < from ? z : 0), s1 = s_lo + c_below + c1 + (zero < to ? z : 0);
+    const SplitState L = split_state(s0, (float)P0, s0 > 0 ? (float)(T - P0) : Tf, n, blo, bhi), U = split_state(s1, (float)P1, (float)(T - P1), n, blo, bhi);
+    const BucketTest test(L, U, c, blo, bhi);
+    const float off = 1.5f * unit * count_to_float(c_below + c1);  // of a sum
+    const float off_d = 2.0f * off * (fabsf(U.hi - L.lo) + bhi - blo);
+    const float here = from < r.hi ? fmaxf(L.d, U.d) - off_d : 0.0f;
+    best = fmaxf(best, __uint_as_float(__reduce_max_sync(kAll, __float_as_uint(fmaxf(here, 0.0f)))));
+    const float m = margin + 2.0f * unit + 0.5f * off * (__fdividef(1.0f, count_to_float(max(s0, 1))) + __fdividef(1.0f, count_to_float(max(n - s1, 1))));
+    const unsigned keep = __ballot_sync(kAll, from < r.hi && test.passes(best * kKeep - off_d, m, best * (kWeak / margin), blo, bhi));
+    if (keep == 0u) { r.size = kHullMax + 1; break; }
+    const int first = __ffs((int)keep) - 1, last = 31 - __clz((int)keep);
+    const int upto = __shfl_sync(kAll, c1, last), below = __shfl_sync(kAll, c0, first);
+    const uint32_t q_first = __shfl_sync(kAll, q0, first);
+    const int before = r.size;
+    c_below += below;
+    q_below += q_first;
+    r.size = upto - below;
+    r.hi = min(r.hi, r.lo + ((uint32_t)(last + 1) << shift));
+    r.lo += (uint32_t)first << shift;
+    if (shift == 0 || level == 3 || (4 * r.size > 3 * before && last - first >= 8)) break;
+  }
+  *range = r;
+}
+
 // The parts of a hull: lane i holds the part in pixel i of the window (and in pixel i + 32 of a wide one): the pixel's slot, where
 // the part begins in its list, and how many values come before it (lanes beyond the window hold the total).
 template <int KHW>
@@ -388,6 +538,81 @@ __device__ __forceinline__ HullSplit search_hull(const float* gathered, const Hu
   best.s = __shfl_sync(kAll, best.s, src);
   best.P = __shfl_sync(kAll, best.P, src);
   best.above = __shfl_sync(kAll, best.above, src);
+  return best;
+}
+
+// The best split among up to 32 E - 1 values in no order (the zeros as one of them, if `zeros`), E a lane: those behind each value and, if
+// `above` is not 0, that before all of them, whose high side reaches the key `above`.  s_lo, P_lo: count and sum below.
+template <int E>
+__device__ __noinline__ HullSplit search_narrowed(const float* hull, int size, bool zeros, int z, int s_lo, double P_lo, double T, int n, uint32_t above, int lane) {
+  constexpr unsigned kAll = 0xFFFFFFFFu;
+  const int values = size + (zeros ? 1 : 0);
+  float x[E];
+  int s[E];
+  double P[E];
+#pragma unroll
+  for (int i = 0; i < E; ++i) {
+    const int at = 32 * i + lane;
+    x[i] = at < size ? hull[at] : (at < values ? 0.0f : __uint_as_float(0xFF800000u));
+    s[i] = s_lo;
+    P[i] = 0.0;
+  }
+#pragma unroll 2
+  for (int j = 0; j < size; ++j) {
+    const float v = hull[j];
+    const double vd = (double)v;
+#pragma unroll
+    for (int i = 0; i < E; ++i)
+      if (v <= x[i]) { ++s[i]; P[i] = __dadd_rn(P[i], vd); }
+  }
+  double D[E], top = -1.0;
+#pragma unroll
+  for (int i = 0; i < E; ++i) {
+    const int at = 32 * i + lane;
+    if (zeros && x[i] >= 0.0f) s[i] += z;
+    P[i] = __dadd_rn(P_lo, P[i]);
+    D[i] = (at < values || (at == 32 * E - 1 && above != 0u)) && s[i] > 0 && s[i] < n ? objective_near(P[i], T, s[i], n) : -1.0;
+    top = fmax(top, D[i]);
+  }
+  HullSplit best{0, 0.0, 0u};
+  auto warp_max = [&](double v) {  // (at least zero, or -1 in every lane)
+    const int hi = __double2hiint(v), hmax = __reduce_max_sync(kAll, hi);
+    return __hiloint2double(hmax, (int)__reduce_max_sync(kAll, hi == hmax ? (uint32_t)__double2loint(v) : 0u));
+  };
+  top = warp_max(top);
+  if (top < 0.0) return best;
+  const double least = top * kCloseBand;
+  int rivals = 0, pick = 0;
+#pragma unroll
+  for (int i = 0; i < E; ++i)
+    if (D[i] >= least) { ++rivals; pick = i; }
+  unsigned who = __ballot_sync(kAll, rivals > 0);
+  if ((who & (who - 1u)) || __any_sync(kAll, rivals > 1)) {  // Algorithm 1's ">=" on the exactly rounded objective: the largest split of equal ones
+    double exact[E], most = -1.0;
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+      exact[i] = D[i] >= least ? objective(P[i], T, s[i], n) : -1.0;
+      most = fmax(most, exact[i]);
+    }
+    most = warp_max(most);
+    int largest = 0;
+#pragma unroll
+    for (int i = 0; i < E; ++i)
+      if (exact[i] == most && s[i] > largest) { largest = s[i]; pick = i; }
+    const int all = __reduce_max_sync(kAll, largest);
+    who = __ballot_sync(kAll, largest == all);
+  }
+  double Pp = P[0];
+  int sp = s[0];
+  float xp = x[0];
+#pragma unroll
+  for (int i = 1; i < E; ++i)
+    if (pick == i) { Pp = P[i]; sp = s[i]; xp = x[i]; }
+  if (32 * pick + lane < values) above = order_key(xp) + 1u;
+  const int src = 31 - __clz((int)who);
+  best.s = __shfl_sync(kAll, sp, src);
+  best.P = __shfl_sync(kAll, Pp, src);
+  best.above = __shfl_sync(kAll, above, src);
   return best;
 }
 
@@ -542,7 +767,7 @@ __device__ __forceinline__ PatchCode search_patch(const TileArgs& a, const Grid&
     c_end = __shfl_sync(kAll, tc, (b_end - 1) & 31);
   }
   const int size = c_end - c_lo, s_lo = c_lo + (seg_lo > B0 ? z : 0);
-  if (size < 1 || size > hull_cap<BPL>() - 1 || (z == 0 && size == n)) return code;
+  if (size < 1 || size > (BPL == 1 ? 511 : kHullMax) || (z == 0 && size == n)) return code;
   if (b_lo >= B0 - 1 && b_end <= B0 + 1) {  // the two buckets next to zero: does the patch have no other values?
     int below, upto;
     double unused;
@@ -582,10 +807,63 @@ __device__ __forceinline__ PatchCode search_patch(const TileArgs& a, const Grid&
     __syncwarp();
   }
   else if (size < 64) split = search_long_hull<2>(DAB_HULL);
-  else if (size < 128) split = search_long_hull<4>(DAB_HULL);
-  else if (size < 256) split = search_long_hull<8>(DAB_HULL);
-  else if (BPL == 1 || size < 512) split = search_long_hull<16>(DAB_HULL);
-  else split = search_long_hull<(BPL == 1 ? 16 : 32)>(DAB_HULL);
+  else if (BPL > 1 && size < 128) split = search_long_hull<4>(DAB_HULL);
+  else if (BPL > 1 && size < 256) split = search_long_hull<8>(DAB_HULL);
+  else if (BPL > 1 && size < 512) split = search_long_hull<16>(DAB_HULL);
+  else if (BPL > 1) split = search_long_hull<32>(DAB_HULL);
+  else {  // narrowed first
+    HullLists<KHW, ListT> lists;
+    lists.step = KHW == 9 ? 3 : (KHW == kWideWindow ? 1 : 32 / wn);
+    lists.sub = lane % lists.step;
+#pragma unroll
+    for (int t = 0; t < PER_LANE; ++t) {
+      const int i = 32 * t + lane / lists.step;
+      lists.count[t] = 0;
+      if (i < wn) {
+        const int slot = map[at + win[i]], begin = b_lo > 0 ? counts[(b_lo - 1) * slots + slot] : 0;
+        lists.count[t] = (int)counts[(b_end - 1) * slots + slot] - begin;
+        lists.from[t] = list + slot * 4 * a.quads + begin;
+        lists.values[t] = tile + slot * a.pitch;
+      }
+    }
+    HullRange r;
+    r.size = size;
+    const float margin = 2e-6f * __uint_as_float(g.top);  // (the middles are good to 1e-6 of the larger mean)
+    narrow_hull<KHW>(lists, &r, reinterpret_cast<uint32_t*>(hull), g.edge[b_lo], g.edge[b_end], s_lo, P_lo, T, n, zeros ? z : 0, best, margin, lane);
+    bool inside = zeros;
+    int s_base = s_lo;
+    uint32_t top = 0u;  // a key above all that lies below
+    if (zeros) {
+      const uint32_t q = hull_place(0.0f, r.origin, r.scale);
+      if (q < r.lo) { s_base += z; top = kZeroKey + 1u; }
+      inside = q >= r.lo && q < r.hi;
+    }
+    if (r.size + (inside ? 1 : 0) > 63) {
+      if (size >= 256) return code;
+      split = size < 128 ? search_long_hull<4>(DAB_HULL) : search_long_hull<8>(DAB_HULL);
+    } else {
+      int fill = 0;
+      double below = 0.0;
+      lists.each([&](float v, bool in) {
+        const uint32_t q = hull_place(v, r.origin, r.scale);
+        const bool is_low = in && q < r.lo;
+        in = in && q >= r.lo && q < r.hi;
+        const unsigned bal = __ballot_sync(kAll, in);
+        if (in) hull[fill + __popc(bal & ((1u << lane) - 1u))] = v;
+        fill += __popc(bal);
+        s_base += __popc(__ballot_sync(kAll, is_low));
+        if (is_low) { below = __dadd_rn(below, (double)v); top = max(top, order_key(v) + 1u); }
+      });
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) below = __dadd_rn(below, __shfl_xor_sync(kAll, below, o));
+      top = __reduce_max_sync(kAll, top);
+      __syncwarp();
+      below = __dadd_rn(P_lo, below);
+      split = fill < 31 ? search_narrowed<1>(hull, fill, inside, z, s_base, below, T, n, top, lane)
+                        : search_narrowed<2>(hull, fill, inside, z, s_base, below, T, n, top, lane);
+      __syncwarp();
+    }
+  }
 #undef DAB_HULL
   if (split.s <= 0 || split.s >= n) return code;
   // the two means side by side in the even and the odd lanes
@@ -825,7 +1103,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) binarize_patches_tile_kernel(
   // ---- the search: a warp per patch ----
   for (int p = warp; p < npatch; p += WARPS) {
     PatchCode code{0, 0.0f, 0.0f, __uint_as_float(0x7FC00000u), false};
-    if (top != 0u) code = search_patch<KHW, BPL>(a, grid, map, win, window_at(p), sums, counts, list, tile, reinterpret_cast<float*>(grid.hist) + 32 * warp, lane);
+    if (top != 0u) code = search_patch<KHW, BPL>(a, grid, map, win, window_at(p), sums, counts, list, tile, reinterpret_cast<float*>(grid.scratch[warp]), lane);
     __syncwarp();
     if (lane == 0) store(p, code);
   }
