@@ -296,8 +296,8 @@ __device__ __forceinline__ SplitState split_state(int s, float P, float Q, int n
   return e;
 }
 
-// Can the best split lie in a bucket?  Two tests of the splits from its lower to its upper edge, the values between them in
-// [vlo, vhi]:
+// Can the best split lie in a bucket?  Two tests of the splits from its lower to its upper edge, the c values between them in
+// [vlo, vhi] (c: all that the two splits differ by, a run of zeros among them):
 //   bound   along the chord between the edges' (s, P) the objective is convex, so at most the larger of the edges'.  A split is off
 //           the chord by at most c (vhi - vlo) / 4 =: e in P, where the objective's slope is at most twice the difference of the means
 //           and its curvature adds e (vhi - vlo) at most;
@@ -407,7 +407,7 @@ __device__ __noinline__ void narrow_hull(const HullLists<KHW, ListT> lists, Hull
     const double P0 = sum_of(c_below + c0, q_below + q0), P1 = sum_of(c_below + c1, q_below + q1);
     const int s0 = s_lo + c_below + c0 + (zero < from ? z : 0), s1 = s_lo + c_below + c1 + (zero < to ? z : 0);
     const SplitState L = split_state(s0, (float)P0, s0 > 0 ? (float)(T - P0) : Tf, n, blo, bhi), U = split_state(s1, (float)P1, (float)(T - P1), n, blo, bhi);
-    const BucketTest test(L, U, c, blo, bhi);
+    const BucketTest test(L, U, s1 - s0, blo, bhi);
     const float off = 1.5f * unit * count_to_float(c_below + c1);  // of a sum
     const float off_d = 2.0f * off * (fabsf(U.hi - L.lo) + bhi - blo);
     const float here = from < r.hi ? fmaxf(L.d, U.d) - off_d : 0.0f;
