@@ -107,6 +107,7 @@ __device__ __forceinline__ void store_columns(const GemmArgs& g, uint32_t (&v)[3
     // Bound by the stores and the tensor to add.  The kind of a layer is looked at once for 32 columns, and columns beyond the last repeat
     // it, so that no branch stands between the loads: 16 are in flight.  One element at a time, with its kind: 32 x 64 x 56 x 56 -> 64 with
     // a normalisation layer and ReLU behind it 32 us, this 23; with a shortcut to add as well 79 and 30; 128 x 28 x 28 57 and 21.
+    // Ordinary loads of the tensor to add: this thread may have stored it, in a kPostStore of the same chain.
     for (int k = 0; k < g.post.count; ++k) {
       const PostOp o = g.post.op[k];
       if (o.kind == kPostAffine) {
@@ -122,7 +123,7 @@ __device__ __forceinline__ void store_columns(const GemmArgs& g, uint32_t (&v)[3
           float other[16];
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            other[j] = __ldg(o.a + DAB_IDX(to, g.c_extent));
+            other[j] = o.a[DAB_IDX(to, g.c_extent)];
             if (j0 + j < left - 1) to += step;
           }
 #pragma unroll

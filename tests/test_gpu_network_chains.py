@@ -70,3 +70,21 @@ def test_chains(N, C, H, W, Cout):
         else:
             cur = got
     assert np.array_equal(plain.cpu().numpy(), cur)
+
+
+@pytest.mark.parametrize("Cout", [20, 64, 300])
+@pytest.mark.parametrize("contraction", ["CONTRACT_TENSOR", "CONTRACT_POPC"])
+def test_a_tensor_stored_and_added_in_one_chain(contraction, Cout):
+    # both contractions read what they have just written: the sum is twice the remembered tensor, then three times it
+    import paper_1804_02941_b200 as dab
+    rng = np.random.default_rng(Cout)
+    conv = dict(kind="conv_binary", w=(rng.standard_normal((Cout, 27)) * 0.1).astype(np.float32), kh=3, kw=3, stride=(1, 1), pad=(1, 1), Cout=Cout)
+    x = to_dev(rng.standard_normal((16, 3, 28, 28)).astype(np.float32))
+    dab.dab_set_contraction(getattr(dab, contraction))
+    try:
+        once = dab.dab_network_forward(dab.Network([conv]), x)
+        y = dab.dab_network_forward(dab.Network([conv, dict(kind="save"), dict(kind="add"), dict(kind="add")]), x)
+    finally:
+        dab.dab_set_contraction(dab.CONTRACT_AUTO)
+    torch.cuda.synchronize()
+    assert torch.equal(y, (once + once) + once)
