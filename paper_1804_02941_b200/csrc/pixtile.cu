@@ -838,30 +838,40 @@ __device__ __forceinline__ PatchCode search_patch(const TileArgs& a, const Grid&
       if (q < r.lo) { s_base += z; top = kZeroKey + 1u; }
       inside = q >= r.lo && q < r.hi;
     }
-    if (r.size + (inside ? 1 : 0) > 63) {
-      if (size >= 256) return code;
-      split = size < 128 ? search_long_hull<4>(DAB_HULL) : search_long_hull<8>(DAB_HULL);
-    } else {
+    bool sorted = r.size + (inside ? 1 : 0) > 63;  // the whole hull
+    if (!sorted) {
+      // The lists are in the order in which threads came.  From 2^(e - 20) on, e the largest value's exponent, values are multiples of
+      // 2^(e - 43), and 511 of them stay below 2^(e + 10): their sums are exact in any order.  A hull with a smaller one is sorted.
+      const float exact_from = __uint_as_float((g.top & 0x7F800000u) - (20u << 23));
       int fill = 0;
       double below = 0.0;
+      bool inexact = false;
       lists.each([&](float v, bool in) {
         const uint32_t q = hull_place(v, r.origin, r.scale);
         const bool is_low = in && q < r.lo;
         in = in && q >= r.lo && q < r.hi;
+        inexact = inexact || ((in || is_low) && fabsf(v) < exact_from);
         const unsigned bal = __ballot_sync(kAll, in);
         if (in) hull[fill + __popc(bal & ((1u << lane) - 1u))] = v;
         fill += __popc(bal);
         s_base += __popc(__ballot_sync(kAll, is_low));
         if (is_low) { below = __dadd_rn(below, (double)v); top = max(top, order_key(v) + 1u); }
       });
+      sorted = __any_sync(kAll, inexact);
+      if (!sorted) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) below = __dadd_rn(below, __shfl_xor_sync(kAll, below, o));
-      top = __reduce_max_sync(kAll, top);
+        for (int o = 16; o > 0; o >>= 1) below = __dadd_rn(below, __shfl_xor_sync(kAll, below, o));
+        top = __reduce_max_sync(kAll, top);
+        __syncwarp();
+        below = __dadd_rn(P_lo, below);
+        split = fill < 31 ? search_narrowed<1>(hull, fill, inside, z, s_base, below, T, n, top, lane)
+                          : search_narrowed<2>(hull, fill, inside, z, s_base, below, T, n, top, lane);
+      }
       __syncwarp();
-      below = __dadd_rn(P_lo, below);
-      split = fill < 31 ? search_narrowed<1>(hull, fill, inside, z, s_base, below, T, n, top, lane)
-                        : search_narrowed<2>(hull, fill, inside, z, s_base, below, T, n, top, lane);
-      __syncwarp();
+    }
+    if (sorted) {
+      if (size >= 256) return code;
+      split = size < 128 ? search_long_hull<4>(DAB_HULL) : search_long_hull<8>(DAB_HULL);
     }
   }
 #undef DAB_HULL
