@@ -47,9 +47,21 @@ constexpr int kTinyBits = 51;
 // From this many pixels on a thread sums a pixel's buckets one after another; below it would leave most of them idle (4200 cycles for
 // 20 pixels where a warp per pixel takes 1500; at 100 pixels both take 5000, at 130 the warps 7000 to 10000).
 constexpr int kSerialPixels = 80;
-// Hulls of 64 values and more are narrowed before they are sorted in short rows; in longer ones, where a warp has three or four patches of a
-// tile and one that cannot be narrowed holds up the others, sorted: 61 x 256 x 14 x 14 N(0, 1) 117 us, 124 narrowed; 32 x 256 x 13 x 13 of a
-// network 95 and 118, 32 x 384 x 13 x 13 156 and 134.
+// Hulls of kNarrowFrom values and more are narrowed before they are sorted, in 3 x 3 windows of short rows (32 buckets).  Code that few
+// patches reach is not in the instruction cache and costs some 30 cycles an instruction, which the patch's whole tile waits for, so that a
+// narrowing tried in vain is dear.  64 x 56 x 56 at batch 32, us: all sorted; narrowed from 128 on; from 64 on:
+//   N(0, 1)|N(0, 1)| 587, 451, 430   steps of 1/8 213, 214, 229   N(0, 1) + 4 291, 293, 324   half zeros 214, 217, 226
+// 128 x 28 x 28: 219, 214, 202   101, 108, 140   163, 145, 154   108, 109, 114
+// and the ResNet-18-shaped network at batch 32 4270, 3500, 3390.
+// In wider windows a lane or two walk the list of a pixel alone: 32 x 48 x 27 x 27 5 x 5 steps of 1/8 107 us sorted, 166 narrowed, N(0, 1)
+// 114 and 131, N(0, 1)|N(0, 1)| 247 and 227.  In longer rows a warp has three or four patches of a tile, and one that cannot be narrowed
+// holds up the others: 61 x 256 x 14 x 14 N(0, 1) 117 us sorted, 124 narrowed; 32 x 256 x 13 x 13 of a network 95 and 118, though
+// 32 x 384 x 13 x 13 156 and 134.
+constexpr int kNarrowFrom = 128;
+// One of 256 values and more that cannot be narrowed is left to the CTA-per-patch kernel in rows of up to kMarkRows values, else sorted.  A
+// single marked patch costs that kernel's latency, many of them less than a sort of 16 values a lane: 64 x 56 x 56 at batch 32, values in
+// steps of 1/8 N(0, 1)|N(0, 1)| 368 us marked and 475 sorted, e^(4 N(0, 1)) 667 and 779; 128 x 28 x 28 N(0, 1) 117 and 109, steps of 1/8 117 and 108.
+constexpr int kMarkRows = 768;
 // A bucket is kept if its bound reaches the best edge objective times this: edges and inner corners are formed in fp32 from
 // sums rounded once (1e-6 relative), the place of a corner to 4e-7 of the bucket's count.
 constexpr float kKeep = 0.9999f;
@@ -323,28 +335,25 @@ struct BucketTest {
   }
 };
 
-// The values of a hull, by the lists of the window's pixels: `step` lanes share a pixel (in wide windows a lane has two).
-template <int KHW, typename ListT>
+// The values of a hull, by the lists of the pixels of a 3 x 3 window: three lanes share a pixel.
+template <typename ListT>
 struct HullLists {
-  static constexpr int kPerLane = KHW == kWideWindow ? 2 : 1;
-  const ListT* from[kPerLane];
-  const float* values[kPerLane];
-  int count[kPerLane];
-  int sub, step;
+  static constexpr int kStep = 3;
+  const ListT* from;
+  const float* values;
+  int count, sub;
   template <typename F>
   __device__ __forceinline__ void each(F f) const {  // f(value, is there one), the whole warp together
-#pragma unroll
-    for (int t = 0; t < kPerLane; ++t)
-      for (int k = sub; __any_sync(0xFFFFFFFFu, k < count[t]); k += step) {
-        const bool in = k < count[t];
-        f(in ? values[t][from[t][k]] : 0.0f, in);
-      }
+    for (int k = sub; __any_sync(0xFFFFFFFFu, k < count); k += kStep) {
+      const bool in = k < count;
+      f(in ? values[from[k]] : 0.0f, in);
+    }
   }
 };
 
 // A hull as the search ends it: values with lo <= hull_place(value) < hi, `size` of them.
-constexpr uint32_t kPlaces = 1u << 22;  // (the sum of 1023 places fits 32 bits)
-constexpr int kHullMax = 1023;
+constexpr int kHullMax32 = 511, kHullMax64 = 1023;  // values of a hull at most, with 32 buckets (where it may be narrowed) and with 64
+constexpr uint32_t kPlaces = 1u << 22;              // (the sum of that many places fits 32 bits)
 struct HullRange {
   float origin, scale;
   uint32_t lo, hi;
@@ -354,13 +363,13 @@ __device__ __forceinline__ uint32_t hull_place(float v, float origin, float scal
   return min((uint32_t)__float2uint_rz(__fmul_rn(__fsub_rn(v, origin), scale)), kPlaces - 1u);
 }
 
-// Narrows a hull of more than 31 values: they are spread over 32 buckets of equal width, a lane each, and the buckets tested as before,
-// until 31 are left or nothing changes.  Values of `zero` place are z more (0: none).  s_lo, P_lo: count and sum below the hull; best: an objective that is
-// reached; table: 64 words.
-// (Hulls of 32 to 500 values were sorted before, in registers, 2 to 16 values a lane by as many variants of the code; the warps of
-// an SM at different ones waited for instructions half of the time: network inputs, 32 x 64 x 56 x 56, 524 us.)
-template <int KHW, typename ListT>
-__device__ __noinline__ void narrow_hull(const HullLists<KHW, ListT> lists, HullRange* range, uint32_t* table, float vlo, float vhi, int s_lo, double P_lo,
+// Narrows a hull of kNarrowFrom values and more: they are spread over 32 buckets of equal width, a lane each, and the buckets tested by
+// BucketTest, until 31 are left or little changes.  z: zeros, at the place of 0 (0: none in the hull).  s_lo, P_lo: count and sum below the hull; best:
+// an objective that is reached; table: 64 words.
+// (Sorted in registers, 4 to 16 values a lane by as many variants of the code, they kept the warps of an SM waiting for instructions half of
+// the time: inputs of the first binarized layer of the ResNet-18-shaped network at batch 32 544 us, narrowed from 64 values on 338.)
+template <typename ListT>
+__device__ __noinline__ void narrow_hull(const HullLists<ListT> lists, HullRange* range, uint32_t* table, float vlo, float vhi, int s_lo, double P_lo,
                                          double T, int n, int z, float best, float margin, int lane) {
   constexpr unsigned kAll = 0xFFFFFFFFu;
   HullRange r = *range;
@@ -414,7 +423,7 @@ __device__ __noinline__ void narrow_hull(const HullLists<KHW, ListT> lists, Hull
     best = fmaxf(best, __uint_as_float(__reduce_max_sync(kAll, __float_as_uint(fmaxf(here, 0.0f)))));
     const float m = margin + 2.0f * unit + 0.5f * off * (__fdividef(1.0f, count_to_float(max(s0, 1))) + __fdividef(1.0f, count_to_float(max(n - s1, 1))));
     const unsigned keep = __ballot_sync(kAll, from < r.hi && test.passes(best * kKeep - off_d, m, best * (kWeak / margin), blo, bhi));
-    if (keep == 0u) { r.size = kHullMax + 1; break; }
+    if (keep == 0u) { r.size = kHullMax32 + 1; break; }
     const int first = __ffs((int)keep) - 1, last = 31 - __clz((int)keep);
     const int upto = __shfl_sync(kAll, c1, last), below = __shfl_sync(kAll, c0, first);
     const uint32_t q_first = __shfl_sync(kAll, q0, first);
@@ -623,7 +632,7 @@ __device__ __noinline__ HullSplit search_long_hull(const HullParts<KHW> h, const
 }
 
 // The best split of one patch, by a warp.  A segment is a bucket or, between the negative and the positive buckets (at
-// index B0), the run of zeros.  at: the window's first pixel in `map`; hull: 32 words of
+// index B0), the run of zeros.  at: the window's first pixel in `map`; hull: 64 words of
 // shared memory of the warp's own.  The result is valid in all lanes.
 template <int KHW, int BPL, typename ListT>
 __device__ __forceinline__ PatchCode search_patch(const TileArgs& a, const Grid& g, const uint16_t* map, const uint16_t* win, int at,
@@ -767,7 +776,7 @@ __device__ __forceinline__ PatchCode search_patch(const TileArgs& a, const Grid&
     c_end = __shfl_sync(kAll, tc, (b_end - 1) & 31);
   }
   const int size = c_end - c_lo, s_lo = c_lo + (seg_lo > B0 ? z : 0);
-  if (size < 1 || size > (BPL == 1 ? 511 : kHullMax) || (z == 0 && size == n)) return code;
+  if (size < 1 || size > (BPL == 1 ? kHullMax32 : kHullMax64) || (z == 0 && size == n)) return code;
   if (b_lo >= B0 - 1 && b_end <= B0 + 1) {  // the two buckets next to zero: does the patch have no other values?
     int below, upto;
     double unused;
@@ -793,6 +802,7 @@ __device__ __forceinline__ PatchCode search_patch(const TileArgs& a, const Grid&
     hp.before[t] = total + incl - count[t];
     if (t + 1 < PER_LANE) total += __shfl_sync(kAll, incl, 31);
   }
+  constexpr bool kNarrow = KHW == 9 && BPL == 1;
   HullSplit split;
 #define DAB_HULL hp, tile, a.pitch, list, 4 * a.quads, size, zeros, z, s_lo, P_lo, T, n, lane
   if (size < 32) {  // the usual case: the pixels' lanes bring the values together in shared memory
@@ -807,29 +817,24 @@ __device__ __forceinline__ PatchCode search_patch(const TileArgs& a, const Grid&
     __syncwarp();
   }
   else if (size < 64) split = search_long_hull<2>(DAB_HULL);
-  else if (BPL > 1 && size < 128) split = search_long_hull<4>(DAB_HULL);
-  else if (BPL > 1 && size < 256) split = search_long_hull<8>(DAB_HULL);
-  else if (BPL > 1 && size < 512) split = search_long_hull<16>(DAB_HULL);
-  else if (BPL > 1) split = search_long_hull<32>(DAB_HULL);
+  else if (size < kNarrowFrom) split = search_long_hull<4>(DAB_HULL);
+  else if (!kNarrow && size < 256) split = search_long_hull<8>(DAB_HULL);
+  else if (!kNarrow && (BPL == 1 || size < 512)) split = search_long_hull<16>(DAB_HULL);
+  else if (!kNarrow) split = search_long_hull<(BPL == 1 ? 16 : 32)>(DAB_HULL);
   else {  // narrowed first
-    HullLists<KHW, ListT> lists;
-    lists.step = KHW == 9 ? 3 : (KHW == kWideWindow ? 1 : 32 / wn);
-    lists.sub = lane % lists.step;
-#pragma unroll
-    for (int t = 0; t < PER_LANE; ++t) {
-      const int i = 32 * t + lane / lists.step;
-      lists.count[t] = 0;
-      if (i < wn) {
-        const int slot = map[at + win[i]], begin = b_lo > 0 ? counts[(b_lo - 1) * slots + slot] : 0;
-        lists.count[t] = (int)counts[(b_end - 1) * slots + slot] - begin;
-        lists.from[t] = list + slot * 4 * a.quads + begin;
-        lists.values[t] = tile + slot * a.pitch;
-      }
+    HullLists<ListT> lists;
+    lists.sub = lane % lists.kStep;
+    lists.count = 0;
+    if (lane / lists.kStep < wn) {
+      const int slot = map[at + win[lane / lists.kStep]], begin = b_lo > 0 ? counts[(b_lo - 1) * slots + slot] : 0;
+      lists.count = (int)counts[(b_end - 1) * slots + slot] - begin;
+      lists.from = list + slot * 4 * a.quads + begin;
+      lists.values = tile + slot * a.pitch;
     }
     HullRange r;
     r.size = size;
     const float margin = 2e-6f * __uint_as_float(g.top);  // (the middles are good to 1e-6 of the larger mean)
-    narrow_hull<KHW>(lists, &r, reinterpret_cast<uint32_t*>(hull), g.edge[b_lo], g.edge[b_end], s_lo, P_lo, T, n, zeros ? z : 0, best, margin, lane);
+    narrow_hull(lists, &r, reinterpret_cast<uint32_t*>(hull), g.edge[b_lo], g.edge[b_end], s_lo, P_lo, T, n, zeros ? z : 0, best, margin, lane);
     bool inside = zeros;
     int s_base = s_lo;
     uint32_t top = 0u;  // a key above all that lies below
@@ -840,9 +845,10 @@ __device__ __forceinline__ PatchCode search_patch(const TileArgs& a, const Grid&
     }
     bool sorted = r.size + (inside ? 1 : 0) > 63;  // the whole hull
     if (!sorted) {
-      // The lists are in the order in which threads came.  From 2^(e - 20) on, e the largest value's exponent, values are multiples of
-      // 2^(e - 43), and 511 of them stay below 2^(e + 10): their sums are exact in any order.  A hull with a smaller one is sorted.
-      const float exact_from = __uint_as_float((g.top & 0x7F800000u) - (20u << 23));
+      // The lists are in the order in which threads came.  From 2^(e - 20) on, e the exponent of the hull's larger edge, values are multiples
+      // of 2^(e - 43), and 511 of them stay below 2^(e + 10): their sums are exact in any order.  A hull with a smaller one is sorted.
+      const float edge = fmaxf(fabsf(g.edge[b_lo]), fabsf(g.edge[b_end]));
+      const float exact_from = __uint_as_float((__float_as_uint(edge) & 0x7F800000u) - (20u << 23));
       int fill = 0;
       double below = 0.0;
       bool inexact = false;
@@ -870,8 +876,8 @@ __device__ __forceinline__ PatchCode search_patch(const TileArgs& a, const Grid&
       __syncwarp();
     }
     if (sorted) {
-      if (size >= 256) return code;
-      split = size < 128 ? search_long_hull<4>(DAB_HULL) : search_long_hull<8>(DAB_HULL);
+      if (size >= 256 && n <= kMarkRows) return code;
+      split = size < 256 ? search_long_hull<8>(DAB_HULL) : search_long_hull<16>(DAB_HULL);
     }
   }
 #undef DAB_HULL
