@@ -83,6 +83,7 @@ template <int T>
 __device__ __noinline__ void block_sort_code(uint32_t* keys, int n, BlockShared<T>* bs) {
   constexpr int W = T / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __syncthreads();  // another warp may still read its sample of the values (block_distinct_code)
   for (int i = tid; i < n; i += T) keys[i] = order_key(__uint_as_float(keys[i]));
   int half = 1;  // half of the padded length
   while (2 * half < n) half <<= 1;
