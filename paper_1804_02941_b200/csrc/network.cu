@@ -278,7 +278,8 @@ __device__ __forceinline__ int64_t divide(int64_t i, int d, uint32_t magic) { re
 // K x K windows unrolled, all loads of an output in flight together (K = 0: any window, four loads at a time).  The first value of the window
 // counts as it is and a later one if it is larger, in this order.
 // 32 x 64 x 112 x 112, 3 x 3 stride 2, is 130 MB, 20 us at the memory's rate: 51 us (with 64-bit divisions and a
-// load at a time 104); 32 x 96 x 55 x 55 18 (37).
+// load at a time 104); 32 x 96 x 55 x 55 18 (37).  Windows of K = 0, the values beyond the last four one at a time: 32 x 64 x 56 x 56 5 x 5
+// stride 2 pad 2 40.4 (42.0; with loads of all fours, masked, 44.0), 4 x 32 x 64 x 64 9 x 9 pad 4 32.3 (33.8; 36.3).
 template <int K>
 __global__ void __launch_bounds__(kGlueThreads) maxpool_kernel(dab_conv_desc d, int Ho, int Wo, uint32_t magic_wo, uint32_t magic_ho, uint32_t magic_c,
                                                                const float* __restrict__ x, const PostOps post, float* __restrict__ y) {
@@ -290,6 +291,7 @@ __global__ void __launch_bounds__(kGlueThreads) maxpool_kernel(dab_conv_desc d, 
     const float* const xp = x + plane * d.H * d.W + (int64_t)h0 * d.W + w0;
     bool seen = false;
     float best = 0.0f;
+    auto inside = [&](int s) { return (unsigned)(w0 + s) < (unsigned)d.W; };
     auto take = [&](float v, bool in) {
       if (in && (!seen || v > best)) best = v;
       seen = seen || in;
@@ -308,17 +310,17 @@ __global__ void __launch_bounds__(kGlueThreads) maxpool_kernel(dab_conv_desc d, 
     } else {
       for (int r = 0; r < kh; ++r) {
         if ((unsigned)(h0 + r) >= (unsigned)d.H) continue;
-        for (int s = 0; s < kw; s += 4) {
+        const float* const row = xp + (int64_t)r * d.W;
+        int s = 0;
+        for (; s + 4 <= kw; s += 4) {
           float v[4];
-          bool in[4];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            in[j] = s + j < kw && (unsigned)(w0 + s + j) < (unsigned)d.W;
-            v[j] = in[j] ? __ldg(xp + (int64_t)r * d.W + s + j) : 0.0f;
-          }
+          for (int j = 0; j < 4; ++j) v[j] = inside(s + j) ? __ldg(row + s + j) : 0.0f;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) take(v[j], in[j]);
+          for (int j = 0; j < 4; ++j) take(v[j], inside(s + j));
         }
+        for (; s < kw; ++s)
+          if (inside(s)) take(__ldg(row + s), true);
       }
     }
     if (post.count > 0) best = apply_post(post, best, (int)(plane - divide(plane, d.C, magic_c) * d.C), oi);
