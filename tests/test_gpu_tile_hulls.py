@@ -1,6 +1,7 @@
-"""Patches that leave the tile coder more values than it sorts at once, against the CPU checker: they are narrowed first.  Heavy tails (a
-few dozen to a few hundred values, as in a residual network), zeros among the values, many equal values, clusters of values too close
-for another bucket width, and two far clusters with nearly the same objective."""
+"""Patches that leave the tile coder more values than a warp's 32, against the CPU checker: sorted, two to 32 a lane, or marked (few are
+narrowed here, see test_gpu_narrowed_hulls.py).  Heavy tails (a few dozen to a few hundred values, as in a residual network), zeros among
+the values, many equal values, clusters of values too close for another bucket width, and two far clusters with nearly the same
+objective."""
 import numpy as np
 import pytest
 import torch
@@ -11,13 +12,16 @@ from parity_util import check_coded, to_dev
 pytestmark = pytest.mark.gpu
 
 CASES = [  # C, H, W, kh, kw, stride, pad
-    (64, 15, 17, 3, 3, 1, 1),    # n = 576: narrowed from 64 values on
-    (128, 9, 10, 3, 3, 2, 1),
-    (200, 7, 8, 3, 3, 1, 1),     # n = 1800: from 128 values on
+    (64, 15, 17, 3, 3, 1, 1),    # n = 576: what cannot be narrowed is marked
+    (128, 9, 10, 3, 3, 2, 1),    # n = 1152: sorted
+    (200, 7, 8, 3, 3, 1, 1),     # n = 1800: 64 buckets, sorted
     (300, 5, 6, 3, 3, 1, 0),     # channels in 16 bits
-    (24, 11, 12, 5, 5, 1, 2),    # a lane per pixel
-    (40, 9, 9, 2, 4, 1, 0),      # four lanes per pixel
+    (24, 11, 12, 5, 5, 1, 2),    # other windows: sorted
+    (40, 9, 9, 2, 4, 1, 0),
     (30, 9, 12, 6, 7, 1, 3),     # two pixels per lane
+    (85, 9, 11, 3, 3, 1, 1),     # n = 765 and 774: on either side of what is marked and sorted
+    (86, 9, 11, 3, 3, 1, 1),
+    (170, 8, 7, 3, 3, 1, 0),     # n = 1530
 ]
 
 
