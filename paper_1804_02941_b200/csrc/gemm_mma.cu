@@ -107,6 +107,8 @@ __device__ __forceinline__ void store_columns(const GemmArgs& g, uint32_t (&v)[3
     // Bound by the stores and the tensor to add.  The kind of a layer is looked at once for 32 columns, and columns beyond the last repeat
     // it, so that no branch stands between the loads: 16 are in flight.  One element at a time, with its kind: 32 x 64 x 56 x 56 -> 64 with
     // a normalisation layer and ReLU behind it 32 us, this 23; with a shortcut to add as well 79 and 30; 128 x 28 x 28 57 and 21.
+    // In the form for 65 to 128 filters and rows below 32 words 128 bytes a thread are spilled, and it is ahead all the same: 16 x 64 x 56 x 56
+    // -> 128, coder included, 141 and 129, 16 x 96 x 56 x 56 -> 96 with a shortcut 193 and 163.
     // Ordinary loads of the tensor to add: this thread may have stored it, in a kPostStore of the same chain.
     for (int k = 0; k < g.post.count; ++k) {
       const PostOp o = g.post.op[k];

@@ -15,7 +15,8 @@
 //              whose bound reaches the best edge value can hold the maximum;
 //   search     the values of those buckets (a dozen or two) are gathered from the lists and sorted, a value a lane, which
 //              with the exact state below them gives the exact split size and prefix sum behind each.  Objectives closer
-//              than their error are compared once more in exactly rounded form, with Algorithm 1's ">=".
+//              than their error are compared once more in exactly rounded form, with Algorithm 1's ">=".  Where 128 and more are left,
+//              3 x 3 windows of short rows narrow them first (narrow_hull); others sort several a lane.
 // The mask is a threshold compare: a thread per patch and 32 channels, values of four channels per load.
 // A patch the search does not settle (too many values in its buckets, as with few distinct ones; magnitudes outside
 // 2^-40..2^40, a NaN or an infinity in the tile) is marked K = kRowMark and coded by the CTA-per-patch kernel of
@@ -318,12 +319,10 @@ __device__ __forceinline__ SplitState split_state(int s, float P, float Q, int n
 //           edges, and has to be in the bucket.
 // The second alone leaves a few buckets, but far ones too where the objective has several maxima.
 struct BucketTest {
-  float edges, bound, mid_lo, mid_hi, gap;
-  BucketTest() = default;
+  float bound, mid_lo, mid_hi, gap;
   __device__ __forceinline__ BucketTest(const SplitState& L, const SplitState& U, int c, float vlo, float vhi) {
     const float w = vhi - vlo;
-    edges = fmaxf(L.d, U.d);
-    bound = __fmaf_rn(0.5f * count_to_float(c) * w, U.hi - L.lo + w, edges);
+    bound = __fmaf_rn(0.5f * count_to_float(c) * w, U.hi - L.lo + w, fmaxf(L.d, U.d));
     mid_lo = 0.5f * (L.lo + L.hi);
     mid_hi = 0.5f * (U.lo + U.hi);
     gap = L.hi - U.lo;
